@@ -1109,56 +1109,196 @@ def emit_contract_program(lv: Level):
     for a_, bas in enumerate(lv.bases):
         starts.append(len(prog))
         prog += [1, boff + a_, len(bas)] + [goff + k for k in bas]
-    # dependency levels of the records (for the warp-parallel interpreter):
-    # a record's level is one more than the highest level among the records
-    # that produce its inputs (moments and the constant 1 are level 0)
-    vlevel = {}
-    rlevel = []
-    for st in starts:
-        typ, dst, cnt = prog[st], prog[st + 1], prog[st + 2]
-        if typ == 0:
-            ins = [prog[st + 3 + 3 * t] for t in range(cnt)] + [prog[st + 4 + 3 * t] for t in range(cnt)]
-        else:
-            ins = [prog[st + 3 + t] for t in range(cnt)]
-        lev = 1 + max(vlevel.get(v, 0) for v in ins)
-        vlevel[dst] = lev
-        rlevel.append(lev)
-    nlev = max(rlevel)
-    order = sorted(range(len(starts)), key=lambda r: (rlevel[r], r))
-    level_off = [0] * (nlev + 1)
-    for r in order:
-        level_off[rlevel[r]] += 1
-    for k in range(1, nlev + 1):
-        level_off[k] += level_off[k - 1]
     L = []
     nm = "L%d" % lv.level
     L.append("  static constexpr int NVALUES = %d, ONE = %d, BOFF = %d, NRECORDS = %d;" % (nv, one, boff, len(starts)))
-    L.append("  static constexpr int NLEVELS = %d;   // dependency levels of the records" % nlev)
     L.append("  template <class R, bool WANT_B>")
     L.append("  __device__ static R contract(const R* __restrict__ M, const typename ScalarOf<R>::T* __restrict__ xi, "
              "R* __restrict__ D, R* __restrict__ B) {")
     L.append("    return interpret_contract<R, WANT_B, NCOMP, NVALUES, ONE, BOFF, NBASIS, NRECORDS>("
              "kProg%s, kStarts%s, M, xi, D, B);" % (nm, nm))
     L.append("  }")
-    L.append("  // one warp: V, A shared arrays of NVALUES (V[0, NCOMP) = moments on entry, A[0, NCOMP) = dE/dM on")
-    L.append("  // return); the records of each dependency level are spread over the lanes")
-    L.append("  template <class R, bool WANT_B, class BV>")
-    L.append("  __device__ static R contract_warp(R* V, R* A, const typename ScalarOf<R>::T* __restrict__ xi, BV B, "
-             "int lane) {")
-    L.append("    return interpret_values_warp<R, WANT_B, NCOMP, NVALUES, ONE, BOFF, NBASIS, NLEVELS>("
-             "kProg%s, kStarts%s, kLevelOrder%s, kLevelOff%s, V, A, xi, B, lane);" % (nm, nm, nm, nm))
-    L.append("  }")
-    L.append("  // V[0, NCOMP) = moments on entry, A[0, NCOMP) = dE/dM on return (arrays of NVALUES)")
-    L.append("  template <class R, bool WANT_B>")
-    L.append("  __device__ static R contract_values(R* V, R* A, const typename ScalarOf<R>::T* __restrict__ xi, "
-             "R* B) {")
-    L.append("    return interpret_values<R, WANT_B, NCOMP, NVALUES, ONE, BOFF, NBASIS, NRECORDS>("
-             "kProg%s, kStarts%s, V, A, xi, B);" % (nm, nm))
-    L.append("  }")
     tables = ["__device__ const int32_t kProg%s[] = {%s};" % (nm, ",".join(str(v) for v in prog)),
-              "__device__ const int32_t kStarts%s[] = {%s};" % (nm, ",".join(str(v) for v in starts)),
-              "__device__ const int32_t kLevelOrder%s[] = {%s};" % (nm, ",".join(str(v) for v in order)),
-              "__device__ const int32_t kLevelOff%s[] = {0,%s};" % (nm, ",".join(str(v) for v in level_off[1:]))]
+              "__device__ const int32_t kStarts%s[] = {%s};" % (nm, ",".join(str(v) for v in starts))]
+    return L, tables
+
+
+# ---------------------------------------------------------------------------
+# the contraction as a program for a block of threads on tiles of atoms
+# ---------------------------------------------------------------------------
+
+TILE_LANES = 16        # records that run side by side (two threads of a warp per record)
+TILE_MAX_TERMS = 11    # longest gather of the reverse pass before it is split into partial sums
+TILE_NONE = 0x1FFF     # destination of a padding record
+
+
+class TileProgram:
+    """Contraction and reverse pass of a level as phases of independent dot
+    products over one array of slots, S[dst] (+)= sum w S[x] S[y].
+
+    Slots: V(v) = v for the values (moment components, DAG node components,
+    graph sums, basis products), ONE and ZERO, then A(v) = AOFF + v for their
+    adjoints.  Forward phases follow the dependency levels.  The reverse pass
+    gathers instead of scattering: in the phase of level L every input v of a
+    record of that level receives A(v) += sum over its uses of
+    w A(dst) V(other), one thread pair per v, so no two threads add to the same
+    slot.  A gather of more than TILE_MAX_TERMS uses is cut into pieces whose
+    partial sums go to slots that nothing needs any more (adjoints of higher
+    levels, values of this level and above) and are added in one more phase.
+    Components with a z-exponent of 2 and more are formed from the swept ones
+    by z^2 = 1 - x^2 - y^2 in one step (binomial weights)."""
+
+    def __init__(self, lv):
+        dag = lv.dag
+        C = len(lv.comps)
+        base, nv = {}, C
+        for n, (key, rank) in enumerate(dag.nodes):
+            if key[0] == "C":
+                base[n] = nv
+                nv += n_sym(rank)
+
+        def ref(n, K):
+            key, rank = dag.nodes[n]
+            if key[0] == "M":
+                _, mu, nu, off = key
+                return lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))]
+            return base[n] + multi_indices(rank).index(K)
+
+        recs = []                                   # (dst, [(x, y, w)]), y None: the constant 1
+        for c in sorted(lv.expand):
+            mu, (a, b, z) = lv.comps[c]
+            m = z // 2
+            terms = []
+            for i in range(m + 1):
+                for j in range(m + 1 - i):
+                    w = (-1) ** (i + j) * (math.factorial(m) // (math.factorial(i) * math.factorial(j) * math.factorial(m - i - j)))
+                    terms.append((lv.comp_index[(mu, (a + 2 * i, b + 2 * j, z - 2 * m))], None, w))
+            recs.append((c, terms))
+        for n, (key, rank) in enumerate(dag.nodes):
+            if key[0] == "C":
+                _, a, b = key
+                for ki, K in enumerate(multi_indices(rank)):
+                    recs.append((base[n] + ki, [(ref(a, tuple(K[d] + P[d] for d in range(3))), ref(b, P),
+                                                 multinomial_weight(P)) for P in multi_indices(dag.rank(b))]))
+        gval = []
+        for roots in lv.roots:
+            if len(roots) == 1 and roots[0][0] == 1:
+                gval.append(ref(roots[0][1], (0, 0, 0)))
+            else:
+                recs.append((nv, [(ref(node, (0, 0, 0)), None, w) for w, node in roots]))
+                gval.append(nv)
+                nv += 1
+        prods = {}
+        for bas in lv.bases:
+            for k in range(2, len(bas) + 1):        # a product is its prefix times the last factor
+                if tuple(bas[:k]) not in prods:
+                    prev = gval[bas[0]] if k == 2 else prods[tuple(bas[:k - 1])]
+                    recs.append((nv, [(prev, gval[bas[k - 1]], 1)]))
+                    prods[tuple(bas[:k])] = nv
+                    nv += 1
+        self.basis = [gval[b[0]] if len(b) == 1 else prods[tuple(b)] for b in lv.bases]
+        assert len(set(self.basis)) == len(self.basis)
+        self.nv, self.one, self.zero, self.aoff = nv, nv, nv + 1, nv + 2
+        self.slots = 2 * nv + 2
+        assert self.slots < TILE_NONE
+
+        level = [0] * nv
+        for dst, terms in recs:
+            level[dst] = 1 + max(max(level[x], level[y] if y is not None else 0) for x, y, _ in terms)
+        top = max(level)
+        one, A = self.one, self.aoff
+        self.phases = [[] for _ in range(top)]      # phases of (dst, accumulate, terms)
+        for dst, terms in recs:
+            self.phases[level[dst] - 1].append((dst, False, [(x, one if y is None else y, w) for x, y, w in terms]))
+        self.n_forward = top
+        written = {A + b for b in self.basis}       # seeded with xi before the reverse pass
+        for lev in range(top, 0, -1):
+            uses = {}
+            for dst, terms in recs:
+                if level[dst] != lev:
+                    continue
+                for x, y, w in terms:
+                    if x == y:
+                        uses.setdefault(x, []).append((A + dst, x, 2 * w))
+                        continue
+                    uses.setdefault(x, []).append((A + dst, one if y is None else y, w))
+                    if y is not None:
+                        uses.setdefault(y, []).append((A + dst, x, w))
+            free = [A + v for v in range(nv) if level[v] > lev] + [v for v in range(nv) if level[v] >= lev]
+            first, second = [], []
+            for v in sorted(uses):
+                u = uses[v]
+                pieces = -(-len(u) // TILE_MAX_TERMS)
+                parts = [u[k::pieces] for k in range(pieces)]
+                first.append((A + v, A + v in written, parts[0]))
+                written.add(A + v)
+                extra = []
+                for p in parts[1:]:
+                    s = free.pop()
+                    first.append((s, False, p))
+                    extra.append((s, one, 1))
+                if extra:
+                    second.append((A + v, True, extra))
+            self.phases.append(first)
+            if second:
+                self.phases.append(second)
+        assert all(A + c in written for c in lv.swept)
+        self.weights = sorted({w for ph in self.phases for _, _, ts in ph for _, _, w in ts} - {1})
+        self.weights.insert(0, 1)
+        assert len(self.weights) <= 64
+
+    def encode(self):
+        """(words, slabs, phase_off): per phase its records, TILE_LANES at a time (a slab, all of the same number
+        of 16-byte chunks), chunk-major so that the lanes of a warp read consecutive chunks.  A record's first chunk
+        holds its destination (bit 13: accumulate) and 3 terms, the others 4 terms each; a term is
+        x | y << 13 | weight index << 26.  slabs: (first chunk, chunks << 1 | all weights are 1)."""
+        widx = {w: k for k, w in enumerate(self.weights)}
+        words, slabs, phase_off = [], [], [0]
+        pad = self.zero | self.zero << 13
+        for ph in self.phases:
+            def chunks(r):
+                return 1 + max(0, -(-(len(r[2]) - 3) // 4))
+            recs = sorted(ph, key=lambda r: (all(w == 1 for _, _, w in r[2]), -chunks(r), r[0]))
+            mine = []
+            for k in range(0, len(recs), TILE_LANES):
+                part = recs[k:k + TILE_LANES]
+                n = max(chunks(r) for r in part)
+                unit = all(w == 1 for r in part for _, _, w in r[2])
+                cols = []
+                for r in part:
+                    cols.append([r[0] | int(r[1]) << 13] + [x | y << 13 | widx[w] << 26 for x, y, w in r[2]])
+                while len(cols) < TILE_LANES:
+                    cols.append([TILE_NONE])
+                for c in cols:
+                    c += [pad] * (4 * n - len(c))
+                mine.append((n, unit, [c[4 * q + i] for q in range(n) for c in cols for i in range(4)]))
+            for n, unit, w in sorted(mine, key=lambda t: -t[0]):
+                slabs.append((len(words) // 4, n << 1 | int(unit)))
+                words += w
+            phase_off.append(len(slabs))
+        return words, slabs, phase_off
+
+
+def emit_tile_program(lv):
+    """Tables and constants of the level's TileProgram."""
+    tp = TileProgram(lv)
+    words, slabs, phase_off = tp.encode()
+    nm = "L%d" % lv.level
+    tables = ["__device__ const uint4 kTileProg%s[] = {%s};" % (
+                  nm, ",".join("{%uu,%uu,%uu,%uu}" % tuple(words[k:k + 4]) for k in range(0, len(words), 4))),
+              "__device__ const uint2 kTileSlab%s[] = {%s};" % (nm, ",".join("{%du,%du}" % s for s in slabs)),
+              "__device__ const int32_t kTilePhase%s[] = {%s};" % (nm, ",".join(str(v) for v in phase_off)),
+              "__device__ const int32_t kTileWeight%s[] = {%s};" % (nm, ",".join(str(v) for v in tp.weights)),
+              "__device__ const int32_t kTileBasis%s[] = {%s};" % (nm, ",".join(str(v) for v in tp.basis))]
+    L = ["  // the contraction as phases of dot products over slots (tile_contract_kernel)",
+         "  static constexpr int TILE_ONE = %d, TILE_ZERO = %d, TILE_AOFF = %d, TILE_SLOTS = %d;" % (
+             tp.one, tp.zero, tp.aoff, tp.slots),
+         "  static constexpr int TILE_FORWARD = %d, TILE_PHASES = %d, TILE_WEIGHTS = %d;" % (
+             tp.n_forward, len(tp.phases), len(tp.weights))]
+    for fn, ty, tab in (("tile_prog", "uint4", "kTileProg"), ("tile_slab", "uint2", "kTileSlab"),
+                        ("tile_phase", "int32_t", "kTilePhase"), ("tile_weight", "int32_t", "kTileWeight"),
+                        ("tile_basis", "int32_t", "kTileBasis")):
+        L.append("  __device__ __forceinline__ static const %s* %s() { return %s%s; }" % (ty, fn, tab, nm))
     return L, tables
 
 
@@ -1231,6 +1371,8 @@ def emit_header(lv: Level):
         out += emit_groups(lv)
     if lv.level >= INTERPRET_FROM_LEVEL:
         body, tables = emit_contract_program(lv)
+        tile_body, tile_tables = emit_tile_program(lv)
+        body, tables = body + tile_body, tables + tile_tables
         out = out[:out.index("struct %s {" % name)] + tables + out[out.index("struct %s {" % name):]
         out += body
     else:

@@ -62,7 +62,7 @@ def generate_sources(levels=LEVELS):
         path = os.path.join(GEN, "efv_level%d.cu" % L)
         _write(path, (
             "// Generated by paper_2510_00193_gb300/build.py.\n"
-            "#include \"efv_kernel.cuh\"\n#include \"grade_kernel.cuh\"\n#include \"batch_kernel.cuh\"\n"
+            "#include \"efv_split.cuh\"\n#include \"grade_kernel.cuh\"\n#include \"batch_kernel.cuh\"\n"
             "#include \"tangent_kernel.cuh\"\n#include \"efv_team.cuh\"\n"
             "#include \"mtp_level%d.cuh\"\n"
             "namespace mtp {\nint efv_level%d(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t s) {\n"

@@ -887,138 +887,6 @@ __global__ void __launch_bounds__(kEfvFusedThreads) efv_kernel(const EfvArgs a) 
   efv_block_flush<LV, R, DTHETA>(sm, e_i, w, a.e_total, a.virial, a.dtheta);
 }
 
-// Levels with component groups (interpreted contraction) and a scratch
-// buffer a.mbuf run as three kernels: the interpreter's per-thread value
-// arrays stream through local memory, which needs many resident warps, while
-// the neighbour sweeps need many registers per thread.  a.mbuf holds the
-// moment vectors of the atom range and then their adjoints, component-major:
-// [2][c][atom - atom_begin].
-template <class LV, class R>
-__global__ void __launch_bounds__(kEfvThreads) split_moments_kernel(const EfvArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  EfvShared<R, LV::NMU, false> sm;
-  sm.setup(a, smem_raw);
-  __syncthreads();
-  const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = t < n;
-  if (!__any_sync(0xffffffffu, active)) return;
-  const int64_t i = a.atom_begin + (active ? t : 0);
-  PairGeom<R> geom;
-  geom.load_centre(a, i, cell_of<R>(a));
-  const int zi = species_at(a.z, i, a.n_species);
-  const int64_t beg = active ? __ldg(a.offsets + i) : 0, end = active ? __ldg(a.offsets + i + 1) : 0;
-  R* buf = static_cast<R*>(a.mbuf) + (active ? t : 0);
-  {
-    R Mg[LV::NCOMP];
-#pragma unroll
-    for (int c = 0; c < LV::NCOMP; ++c) Mg[c] = R(0);
-    moment_sweep<LV, R, false, 0, true>(a, sm, geom, a.cell, zi, beg, end, Mg);
-    if (active) LV::template store_group<0, R>(Mg, buf, n);
-  }
-  {
-    R Mg[LV::NCOMP];
-#pragma unroll
-    for (int c = 0; c < LV::NCOMP; ++c) Mg[c] = R(0);
-    moment_sweep<LV, R, false, 1, true>(a, sm, geom, a.cell, zi, beg, end, Mg);
-    if (active) LV::template store_group<1, R>(Mg, buf, n);
-  }
-}
-
-template <class LV, class R, bool DTHETA>
-__global__ void __launch_bounds__(kEfvThreads) split_contract_kernel(const EfvArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  EfvShared<R, LV::NMU, DTHETA> sm;
-  sm.setup(a, smem_raw);
-  sm.zero_gradients();
-  __syncthreads();
-  const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = t < n;
-  double e_i = 0.0;
-  const R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-  if (__any_sync(0xffffffffu, active)) {
-    const R* __restrict__ mrow = static_cast<const R*>(a.mbuf) + (active ? t : 0);
-    R* __restrict__ drow = static_cast<R*>(a.mbuf) + (size_t)LV::NCOMP * n + (active ? t : 0);
-    R V[LV::NVALUES], A[LV::NVALUES];
-    R Bv[DTHETA ? LV::NBASIS : 1];
-    for (int c = 0; c < LV::NCOMP; ++c) V[c] = active ? mrow[c * n] : R(0);
-    const R ei = LV::template contract_values<R, DTHETA>(V, A, sm.xi, Bv);
-    if (active)
-      for (int c = 0; c < LV::NCOMP; ++c) drow[c * n] = A[c];
-    if (DTHETA) {
-      const int lane = threadIdx.x & 31;
-#pragma unroll
-      for (int u = 0; u < (DTHETA ? LV::NBASIS : 1); ++u) {
-        const R v = warp_sum_r(active ? Bv[u] : R(0));
-        if (lane == 0) atomicAdd(sm.dxi + u, v);
-      }
-    }
-    if (active) {
-      const int64_t i = a.atom_begin + t;
-      const int zi = species_at(a.z, i, a.n_species);
-      e_i = a.species_energy[zi] + (double)ei;
-      a.e_atom[i] = e_i;
-      if (!isfinite(e_i)) flag_status(a.status, MTP_ERR_NONFINITE);
-      if (DTHETA) atomicAdd(sm.cnt + zi, 1);
-    }
-  }
-  efv_block_flush<LV, R, DTHETA>(sm, e_i, w, a.e_total, a.virial, a.dtheta, kFlushEW | kFlushDxi);
-}
-
-template <class LV, class R, bool DTHETA>
-__global__ void __launch_bounds__(kEfvThreads) split_adjoint_kernel(const EfvArgs a) {
-  constexpr int NMU = LV::NMU;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  EfvShared<R, NMU, DTHETA> sm;
-  sm.setup(a, smem_raw);
-  sm.zero_gradients();
-  __syncthreads();
-  const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = t < n;
-  R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-  if (__any_sync(0xffffffffu, active)) {
-    const int64_t i = a.atom_begin + (active ? t : 0);
-    PairGeom<R> geom;
-    geom.load_centre(a, i, cell_of<R>(a));
-    const int zi = species_at(a.z, i, a.n_species);
-    const int64_t beg = active ? __ldg(a.offsets + i) : 0, end = active ? __ldg(a.offsets + i + 1) : 0;
-    const R* buf = static_cast<const R*>(a.mbuf) + (size_t)LV::NCOMP * n + (active ? t : 0);
-    R fx = R(0), fy = R(0), fz = R(0);
-    constexpr int kAccS = 4;
-    R acc_local[(DTHETA && sizeof(R) == 8) ? kAccS * NMU * kMaxQ : 1];
-    const AccView<R> acc = (sizeof(R) == 4) ? AccView<R>{sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x}
-                                            : AccView<R>{acc_local, 1};
-    const bool own_acc = DTHETA && sm.S <= kAccS && acc.p != nullptr;
-    if (own_acc) {
-      for (int u = 0; u < sm.S * NMU * sm.nq; ++u) acc[u] = R(0);
-    }
-    {
-      R Dg[LV::NCOMP];
-      LV::template load_group<0, R>(buf, n, Dg);
-      adjoint_sweep<LV, R, DTHETA, 0, true>(a, sm, geom, a.cell, zi, beg, end, Dg, fx, fy, fz, w, acc, own_acc);
-    }
-    {
-      R Dg[LV::NCOMP];
-      LV::template load_group<1, R>(buf, n, Dg);
-      adjoint_sweep<LV, R, DTHETA, 1, true>(a, sm, geom, a.cell, zi, beg, end, Dg, fx, fy, fz, w, acc, own_acc);
-    }
-    if (active) {
-      if (own_acc) {
-        for (int zj = 0; zj < sm.S; ++zj) {
-          R* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-          for (int u = 0; u < NMU * sm.nq; ++u) atomicAdd(dst + u, acc[zj * NMU * sm.nq + u]);
-        }
-      }
-      scatter_force(a, i, fx, fy, fz);
-      if (!isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
-        flag_status(a.status, MTP_ERR_NONFINITE);
-    }
-  }
-  efv_block_flush<LV, R, DTHETA>(sm, 0.0, w, a.e_total, a.virial, a.dtheta, kFlushEW | kFlushDc);
-}
-
 constexpr int kFixedQ = 8;
 
 template <class K>
@@ -1031,74 +899,6 @@ int set_smem(K kern, size_t bytes) {
     }
   }
   return MTP_OK;
-}
-
-template <class LV, class R, bool DTHETA>
-int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
-  const int SS = a.n_species * a.n_species;
-  const int64_t n = a.atom_end - a.atom_begin;
-  if (n <= 0) return MTP_OK;
-  const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
-  const size_t b0 = efv_smem_bytes<R, LV::NMU, false>(SS, a.n_q, a.m);
-  const size_t b1 = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                    efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvThreads);
-  int rc;
-  // the contraction kernel has no dE/dc accumulators: without them its blocks
-  // stay small, so that many warps hide the interpreter's local-memory traffic
-  const size_t bc = efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m);
-  if ((rc = set_smem(split_moments_kernel<LV, R>, b0)) != MTP_OK) return rc;
-  if ((rc = set_smem(split_contract_kernel<LV, R, DTHETA>, bc)) != MTP_OK) return rc;
-  if ((rc = set_smem(split_adjoint_kernel<LV, R, DTHETA>, b1)) != MTP_OK) return rc;
-  split_moments_kernel<LV, R><<<grid, kEfvThreads, b0, stream>>>(a);
-  split_contract_kernel<LV, R, DTHETA><<<grid, kEfvThreads, bc, stream>>>(a);
-  split_adjoint_kernel<LV, R, DTHETA><<<grid, kEfvThreads, b1, stream>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    set_error("efv split kernels (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
-    return MTP_ERR_CUDA;
-  }
-  return MTP_OK;
-}
-
-template <class LV, class R, bool DTHETA>
-int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
-  if constexpr (LV::NGROUPS > 1) {
-    if (a.mbuf) return efv_split_launch<LV, R, DTHETA>(a, stream);
-  }
-  const int SS = a.n_species * a.n_species;
-  const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                       efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvFusedThreads);
-  auto kern = efv_kernel<LV, R, DTHETA>;
-  // the mixed path of the single-group levels with the common radial basis
-  // size n_q = 8 runs with n_q fixed at compile time
-  if constexpr (std::is_same<R, float>::value && LV::NGROUPS == 1) {
-    if (a.n_q == kFixedQ) kern = efv_kernel<LV, R, DTHETA, kFixedQ>;
-  }
-  if (bytes > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-      set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-  }
-  const int64_t n = a.atom_end - a.atom_begin;
-  if (n <= 0) return MTP_OK;
-  const unsigned grid = (unsigned)((n + kEfvFusedThreads - 1) / kEfvFusedThreads);
-  kern<<<grid, kEfvFusedThreads, bytes, stream>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    set_error("efv kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
-    return MTP_ERR_CUDA;
-  }
-  return MTP_OK;
-}
-
-template <class LV>
-int efv_launch(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t stream) {
-  if (precision == MTP_MIXED) {
-    return want_dtheta ? efv_launch_typed<LV, float, true>(a, stream) : efv_launch_typed<LV, float, false>(a, stream);
-  }
-  return want_dtheta ? efv_launch_typed<LV, double, true>(a, stream) : efv_launch_typed<LV, double, false>(a, stream);
 }
 
 }  // namespace mtp

@@ -1,0 +1,195 @@
+// Levels with component groups (18 and 20: 201 and 295 moment components, too
+// many for registers) and a scratch buffer a.mbuf run as three kernels: the
+// neighbour sweeps need many registers per thread, the contraction the whole
+// shared memory of an SM.
+//
+// Sweeps: one thread per atom, component group (mu = 0, mu >= 1: a group's
+// moments or adjoints fit in registers) and share of the atom's neighbours
+// (a.n_parts of them); blockIdx.y = 2 share + group.  Every share writes its
+// own partial moments, which the contraction adds when it loads them, so the
+// shares never wait for one another.  Scratch layout: tile_offset.
+#pragma once
+#include "efv_kernel.cuh"
+#include "tile_contract.cuh"
+
+namespace mtp {
+
+// This thread's atom of the range and its share of the neighbours.
+struct SplitShare {
+  int64_t t, i, beg, end;
+  bool active;
+  __device__ __forceinline__ bool setup(const EfvArgs& a, int64_t n) {
+    t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    active = t < n;
+    i = a.atom_begin + (active ? t : 0);
+    const int part = blockIdx.y >> 1;
+    const int64_t b = __ldg(a.offsets + i), len = __ldg(a.offsets + i + 1) - b;
+    beg = b + len * part / a.n_parts;
+    end = active ? b + len * (part + 1) / a.n_parts : beg;
+    return __any_sync(0xffffffffu, t < tile_padded(n));
+  }
+};
+
+template <class LV, class R, int G>
+__device__ __forceinline__ void split_moments(const EfvArgs& a, const EfvShared<R, LV::NMU, false>& sm,
+                                              const SplitShare& s, int64_t n) {
+  PairGeom<R> geom;
+  geom.load_centre(a, s.i, cell_of<R>(a));
+  const int zi = species_at(a.z, s.i, a.n_species);
+  R Mg[LV::NCOMP];
+#pragma unroll
+  for (int c = 0; c < LV::NCOMP; ++c) Mg[c] = R(0);
+  moment_sweep<LV, R, false, G, true>(a, sm, geom, a.cell, zi, s.beg, s.end, Mg);
+  // the atoms that pad the last tile get zero moments
+  if (s.t < tile_padded(n)) {
+    R* buf = static_cast<R*>(a.mbuf) + (int64_t)(blockIdx.y >> 1) * (tile_padded(n) * LV::NCOMP);
+    LV::template store_group<G, R>(Mg, buf + tile_offset<R>(s.t, LV::NCOMP), tile_atoms<R>());
+  }
+}
+
+template <class LV, class R>
+__global__ void __launch_bounds__(kEfvThreads) split_moments_kernel(const EfvArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  EfvShared<R, LV::NMU, false> sm;
+  sm.setup(a, smem_raw);
+  __syncthreads();
+  const int64_t n = a.atom_end - a.atom_begin;
+  SplitShare s;
+  if (!s.setup(a, n)) return;
+  if ((blockIdx.y & 1) == 0) split_moments<LV, R, 0>(a, sm, s, n);
+  else split_moments<LV, R, 1>(a, sm, s, n);
+}
+
+template <class LV, class R, bool DTHETA, int G>
+__device__ __forceinline__ void split_adjoint(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm,
+                                              const SplitShare& s, int64_t n, R* w) {
+  constexpr int NMU = LV::NMU;
+  PairGeom<R> geom;
+  geom.load_centre(a, s.i, cell_of<R>(a));
+  const int zi = species_at(a.z, s.i, a.n_species);
+  R fx = R(0), fy = R(0), fz = R(0);
+  constexpr int kAccS = 4;
+  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccS * NMU * kMaxQ : 1];
+  const AccView<R> acc = (sizeof(R) == 4) ? AccView<R>{sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x}
+                                          : AccView<R>{acc_local, 1};
+  const bool own_acc = DTHETA && sm.S <= kAccS && acc.p != nullptr;
+  if (own_acc) {
+    for (int u = 0; u < sm.S * NMU * sm.nq; ++u) acc[u] = R(0);
+  }
+  R Dg[LV::NCOMP];
+  const R* buf = static_cast<const R*>(a.mbuf) + (int64_t)a.n_parts * (tile_padded(n) * LV::NCOMP);
+  LV::template load_group<G, R>(buf + tile_offset<R>(s.active ? s.t : 0, LV::NCOMP), tile_atoms<R>(), Dg);
+  adjoint_sweep<LV, R, DTHETA, G, true>(a, sm, geom, a.cell, zi, s.beg, s.end, Dg, fx, fy, fz, w, acc, own_acc);
+  if (!s.active) return;
+  if (own_acc) {
+    constexpr int lo = LV::GROUP_MU_LO[G], hi = LV::GROUP_MU_HI[G];
+    for (int zj = 0; zj < sm.S; ++zj) {
+      R* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
+      for (int u = lo * sm.nq; u < hi * sm.nq; ++u) atomicAdd(dst + u, acc[zj * NMU * sm.nq + u]);
+    }
+  }
+  scatter_force(a, s.i, fx, fy, fz);
+  if (!isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
+    flag_status(a.status, MTP_ERR_NONFINITE);
+}
+
+template <class LV, class R, bool DTHETA>
+__global__ void __launch_bounds__(kEfvThreads) split_adjoint_kernel(const EfvArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  EfvShared<R, LV::NMU, DTHETA> sm;
+  sm.setup(a, smem_raw);
+  sm.zero_gradients();
+  __syncthreads();
+  const int64_t n = a.atom_end - a.atom_begin;
+  R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+  SplitShare s;
+  if (s.setup(a, n)) {
+    if ((blockIdx.y & 1) == 0) split_adjoint<LV, R, DTHETA, 0>(a, sm, s, n, w);
+    else split_adjoint<LV, R, DTHETA, 1>(a, sm, s, n, w);
+  }
+  efv_block_flush<LV, R, DTHETA>(sm, 0.0, w, a.e_total, a.virial, a.dtheta, kFlushEW | kFlushDc);
+}
+
+// Contraction kernel: one block per resident slot of the device, each taking
+// tile after tile.
+template <class LV, class R, bool WANT_B>
+int tile_contract_launch(const EfvArgs& a, double* theta, cudaStream_t stream) {
+  auto kern = tile_contract_kernel<LV, R, WANT_B>;
+  constexpr size_t bytes = tile_smem_bytes<LV, R>();
+  int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
+  const int64_t n = a.atom_end - a.atom_begin;
+  const int64_t tiles = (n + tile_atoms<R>() - 1) / tile_atoms<R>();
+  constexpr int resident = (int)(227 * 1024 / (bytes + 1024)) < 3 ? (int)(227 * 1024 / (bytes + 1024)) : 3;
+  static_assert(resident >= 1, "a tile's slots fit in the shared memory of an SM");
+  const int64_t grid = std::min<int64_t>(tiles, (int64_t)device_sms() * resident);
+  kern<<<(unsigned)grid, kTileThreads, bytes, stream>>>(a, theta);
+  return MTP_OK;
+}
+
+template <class LV, class R, bool DTHETA>
+int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
+  const int SS = a.n_species * a.n_species;
+  const int64_t n = a.atom_end - a.atom_begin;
+  if (n <= 0) return MTP_OK;
+  // every thread of the last block that pads a tile must exist: 128 is a multiple of the tile's atoms
+  const dim3 grid((unsigned)((n + kEfvThreads - 1) / kEfvThreads), 2 * a.n_parts);
+  const size_t b0 = efv_smem_bytes<R, LV::NMU, false>(SS, a.n_q, a.m);
+  const size_t b1 = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
+                    efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvThreads);
+  int rc;
+  if ((rc = set_smem(split_moments_kernel<LV, R>, b0)) != MTP_OK) return rc;
+  if ((rc = set_smem(split_adjoint_kernel<LV, R, DTHETA>, b1)) != MTP_OK) return rc;
+  split_moments_kernel<LV, R><<<grid, kEfvThreads, b0, stream>>>(a);
+  if ((rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream)) != MTP_OK) return rc;
+  split_adjoint_kernel<LV, R, DTHETA><<<grid, kEfvThreads, b1, stream>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("efv split kernels (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+    return MTP_ERR_CUDA;
+  }
+  return MTP_OK;
+}
+
+template <class LV, class R, bool DTHETA>
+int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
+  if constexpr (LV::NGROUPS > 1) {
+    if (a.mbuf) return efv_split_launch<LV, R, DTHETA>(a, stream);
+  }
+  const int SS = a.n_species * a.n_species;
+  const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
+                       efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvFusedThreads);
+  auto kern = efv_kernel<LV, R, DTHETA>;
+  // the mixed path of the single-group levels with the common radial basis
+  // size n_q = 8 runs with n_q fixed at compile time
+  if constexpr (std::is_same<R, float>::value && LV::NGROUPS == 1) {
+    if (a.n_q == kFixedQ) kern = efv_kernel<LV, R, DTHETA, kFixedQ>;
+  }
+  if (bytes > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) {
+      set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+      return MTP_ERR_CUDA;
+    }
+  }
+  const int64_t n = a.atom_end - a.atom_begin;
+  if (n <= 0) return MTP_OK;
+  const unsigned grid = (unsigned)((n + kEfvFusedThreads - 1) / kEfvFusedThreads);
+  kern<<<grid, kEfvFusedThreads, bytes, stream>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("efv kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+    return MTP_ERR_CUDA;
+  }
+  return MTP_OK;
+}
+
+template <class LV>
+int efv_launch(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t stream) {
+  if (precision == MTP_MIXED) {
+    return want_dtheta ? efv_launch_typed<LV, float, true>(a, stream) : efv_launch_typed<LV, float, false>(a, stream);
+  }
+  return want_dtheta ? efv_launch_typed<LV, double, true>(a, stream) : efv_launch_typed<LV, double, false>(a, stream);
+}
+
+}  // namespace mtp

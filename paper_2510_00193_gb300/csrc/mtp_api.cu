@@ -492,12 +492,13 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
     variant = h->tuned[precision == MTP_MIXED ? 1 : 0][bucket];
     if (variant == 0) variant = n <= kTeamDefaultAtoms ? 2 : 1;
   }
-  if (h->ops->split_comps > 0 && n > 0 && variant == 1) {
-    // moment/adjoint scratch of the split kernels (levels with an interpreted
-    // contraction), bounded by the chunk as the paper's chunk size bounds memory
-    const size_t bytes = 2 * (size_t)h->ops->split_comps * (size_t)std::min<int64_t>(chunk, n) *
-                         (precision == MTP_MIXED ? sizeof(float) : sizeof(double));
-    int rc = h->mbuf.ensure(bytes);
+  if (h->ops->split_comps > 0 && n > 0) {
+    // moment/adjoint scratch of the split kernels (levels with component
+    // groups), bounded by the chunk as the paper's chunk size bounds memory
+    const int64_t range = std::min<int64_t>(chunk, n);
+    a.n_parts = split_parts(range, device_sms());
+    int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, range, a.n_parts,
+                                                precision == MTP_MIXED ? sizeof(float) : sizeof(double)));
     if (rc != MTP_OK) return rc;
     a.mbuf = h->mbuf.ptr;
   }
@@ -680,10 +681,10 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
   t.base.atom_begin = 0;
   t.base.atom_end = n;
   if (h->ops->split_comps > 0 && n > 0) {
-    // dual moments and adjoints of the split tangent kernels: 2 x components x atoms (value, tangent) pairs
-    const size_t bytes = 4 * (size_t)h->ops->split_comps * (size_t)n *
-                         (precision == MTP_MIXED ? sizeof(float) : sizeof(double));
-    int rc = h->mbuf.ensure(bytes);
+    // dual moments and adjoints of the split tangent kernels: (value, tangent) pairs
+    t.base.n_parts = split_parts(n, device_sms());
+    int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, n, t.base.n_parts,
+                                                2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double))));
     if (rc != MTP_OK) return rc;
     t.base.mbuf = h->mbuf.ptr;
   }

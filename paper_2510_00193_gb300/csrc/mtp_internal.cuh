@@ -78,9 +78,36 @@ struct EfvArgs {
   double* e_total;
   double* dtheta;           // nullable
   int* status;
-  void* mbuf;               // levels with component groups: moment and adjoint scratch
-                            // [2][NCOMP][atom_end - atom_begin] in the working precision (nullptr: one fused kernel)
+  void* mbuf;               // levels with component groups: scratch of the split kernels in the working precision,
+                            // n_parts buffers of partial moments, then the adjoints (nullptr: one fused kernel)
+  int n_parts;              // shares into which the split kernels cut each atom's neighbours
 };
+
+// Shares of each atom's neighbours in the split sweeps (levels with component
+// groups) of n atoms.  One thread per atom, component group and share: at 255
+// registers two 128-thread blocks are resident per SM, and a small system
+// leaves most of them empty, so its neighbours are cut into shares until one
+// wave is full (level 20, 4,000 atoms, FP64: one share left 32 blocks for 152
+// SMs).  The contraction adds the shares' moments when it loads them.
+constexpr int kSplitMaxParts = 16;
+// SMs of the current device.
+inline int device_sms() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+    return 1;
+  return n;
+}
+inline int split_parts(int64_t n, int sms) {
+  const int64_t blocks = 2 * ((n + 127) / 128);
+  int parts = 1;
+  while (parts < kSplitMaxParts && 2 * parts * blocks <= 2 * (int64_t)sms) parts *= 2;
+  return parts;
+}
+// Bytes of EfvArgs::mbuf for n atoms: atoms rounded up to whole tiles of 8.
+inline size_t split_scratch_bytes(int comps, int64_t n, int parts, size_t entry) {
+  return entry * (size_t)comps * (size_t)((n + 7) / 8 * 8) * (size_t)(parts + 1);
+}
 
 using EfvLaunch = int (*)(const EfvArgs&, int precision, bool want_dtheta, cudaStream_t);
 // FP64 basis rows of listed atoms (list == nullptr: atoms atom_begin..), optional FP64 column sums.
@@ -99,7 +126,7 @@ struct LevelEntry {
   BatchLaunch batch;
   TangentLaunch tangent;
   int split_comps;   // components per atom of the EfvArgs::mbuf scratch (0: the level needs none)
-  EfvLaunch team;    // warp-per-atom energy/force kernel (levels without component groups)
+  EfvLaunch team;    // warp-per-atom energy/force kernel (levels with component groups: the split kernels)
 };
 
 const LevelEntry* find_level(int level);

@@ -11,7 +11,7 @@
 #pragma once
 #include <type_traits>
 
-#include "efv_kernel.cuh"
+#include "efv_split.cuh"
 
 namespace mtp {
 
@@ -162,89 +162,130 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs 
     atomicAdd(t.dtheta_tan + S_ + (int64_t)NMU * nq * SS + k, (double)sm.dxi[k]);
 }
 
-// Levels with component groups and a scratch buffer (t.base.mbuf, [2][NCOMP]
-// [atom] dual numbers) run the tangent as three kernels, as the energy does:
-// dual moments per component group, the interpreted contraction at high
-// occupancy, dual adjoint sweeps per group.
-template <class LV, class S>
-__global__ void __launch_bounds__(kEfvThreads) tangent_moments_kernel(const TangentArgs t) {
+// Levels with component groups run the tangent as three kernels, as the
+// energy does: dual moments per component group and share of the neighbours,
+// the tile program on dual numbers, dual adjoint sweeps.
+template <class LV, class S, int G>
+__device__ __forceinline__ void tangent_moments(const TangentArgs& t, const EfvShared<S, LV::NMU, true>& sm,
+                                                const SplitShare& s, int64_t n) {
   using R = Dual<S>;
   constexpr int NMU = LV::NMU;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   const EfvArgs& a = t.base;
-  EfvShared<S, NMU, true> sm;
-  sm.setup(a, smem_raw);
-  __syncthreads();
-  const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= n) return;
-  const int64_t i = a.atom_begin + u;
   TangentGeom<S> geom;
-  geom.load_centre(t, i, cell_of<S>(a));
-  const int zi = species_at(a.z, i, a.n_species);
-  const int64_t beg = __ldg(a.offsets + i), end = __ldg(a.offsets + i + 1);
+  geom.load_centre(t, s.i, cell_of<S>(a));
+  const int zi = species_at(a.z, s.i, a.n_species);
   const R rcut = R(sm.rcut), mid = R(sm.mid), scale = R(sm.scale);
-  R* buf = static_cast<R*>(a.mbuf) + u;
-  auto sweep = [&](auto group) {
-    constexpr int G = decltype(group)::value;
-    R Mg[LV::NCOMP];
+  R Mg[LV::NCOMP];
 #pragma unroll
-    for (int c = 0; c < LV::NCOMP; ++c) Mg[c] = R(0);
-    for (int64_t k = beg; k < end; ++k) {
-      const int32_t j = __ldg(a.nbr_j + k);
-      const int32_t img = __ldg(a.nbr_img + k);
-      const auto l = geom.g.fetch(a, j);
-      R dx, dy, dz;
-      geom.vec(t, j, l, img, dx, dy, dz);
-      const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-      const R rinv = rsqrt_r(r2);
-      const R r = r2 * rinv;
-      R f[NMU];
-      radial<R, NMU, false, false>(sm.c + (zi * sm.S + l.species) * sm.cstride, sm.nq, r, mid, scale, rcut, f,
-                                   (R*)nullptr, (R*)nullptr);
-      LV::template moments_group<G, R>(Mg, f, dx * rinv, dy * rinv, dz * rinv);
-    }
-    LV::template store_group<G, R>(Mg, buf, n);
-  };
-  sweep(std::integral_constant<int, 0>());
-  sweep(std::integral_constant<int, 1>());
+  for (int c = 0; c < LV::NCOMP; ++c) Mg[c] = R(0);
+  for (int64_t k = s.beg; k < s.end; ++k) {
+    const int32_t j = __ldg(a.nbr_j + k);
+    const int32_t img = __ldg(a.nbr_img + k);
+    const auto l = geom.g.fetch(a, j);
+    R dx, dy, dz;
+    geom.vec(t, j, l, img, dx, dy, dz);
+    const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
+    const R rinv = rsqrt_r(r2);
+    const R r = r2 * rinv;
+    R f[NMU];
+    radial<R, NMU, false, false>(sm.c + (zi * sm.S + l.species) * sm.cstride, sm.nq, r, mid, scale, rcut, f,
+                                 (R*)nullptr, (R*)nullptr);
+    LV::template moments_group<G, R>(Mg, f, dx * rinv, dy * rinv, dz * rinv);
+  }
+  if (s.t < tile_padded(n)) {
+    R* buf = static_cast<R*>(a.mbuf) + (int64_t)(blockIdx.y >> 1) * (tile_padded(n) * LV::NCOMP);
+    LV::template store_group<G, R>(Mg, buf + tile_offset<R>(s.t, LV::NCOMP), tile_atoms<R>());
+  }
 }
 
 template <class LV, class S>
-__global__ void __launch_bounds__(kEfvThreads) tangent_contract_kernel(const TangentArgs t) {
-  using R = Dual<S>;
+__global__ void __launch_bounds__(kEfvThreads) tangent_moments_kernel(const TangentArgs t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const EfvArgs& a = t.base;
   EfvShared<S, LV::NMU, true> sm;
-  sm.setup(a, smem_raw);
-  sm.zero_gradients();
+  sm.setup(t.base, smem_raw);
   __syncthreads();
-  const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = u < n;
-  const int lane = threadIdx.x & 31;
-  if (__any_sync(0xffffffffu, active)) {
-    const R* __restrict__ mrow = static_cast<const R*>(a.mbuf) + (active ? u : 0);
-    R* __restrict__ drow = static_cast<R*>(a.mbuf) + (size_t)LV::NCOMP * n + (active ? u : 0);
-    R V[LV::NVALUES], A[LV::NVALUES], B[LV::NBASIS];
-    for (int c = 0; c < LV::NCOMP; ++c) V[c] = active ? mrow[c * n] : R(0);
-    (void)LV::template contract_values<R, true>(V, A, sm.xi, B);
-    if (active)
-      for (int c = 0; c < LV::NCOMP; ++c) drow[c * n] = A[c];
-    for (int k = 0; k < LV::NBASIS; ++k) {
-      const S v = warp_sum_r(active ? B[k].t : S(0));
-      if (lane == 0) atomicAdd(sm.dxi + k, v);
+  const int64_t n = t.base.atom_end - t.base.atom_begin;
+  SplitShare s;
+  if (!s.setup(t.base, n)) return;
+  if ((blockIdx.y & 1) == 0) tangent_moments<LV, S, 0>(t, sm, s, n);
+  else tangent_moments<LV, S, 1>(t, sm, s, n);
+}
+
+template <class LV, class S, int G>
+__device__ __forceinline__ void tangent_adjoint(const TangentArgs& t, const EfvShared<S, LV::NMU, true>& sm,
+                                                const SplitShare& s, int64_t n) {
+  using R = Dual<S>;
+  constexpr int NMU = LV::NMU;
+  constexpr int mu_lo = LV::GROUP_MU_LO[G], mu_hi = LV::GROUP_MU_HI[G];
+  if (!s.active) return;
+  const EfvArgs& a = t.base;
+  TangentGeom<S> geom;
+  geom.load_centre(t, s.i, cell_of<S>(a));
+  const int zi = species_at(a.z, s.i, a.n_species);
+  const R rcut = R(sm.rcut), mid = R(sm.mid), scale = R(sm.scale);
+  S fx = S(0), fy = S(0), fz = S(0);
+  constexpr int kAccS = 4;
+  const bool own_acc = sm.S <= kAccS;
+  S acc[kAccS * NMU * kMaxQ];
+  if (own_acc) {
+    for (int v = 0; v < sm.S * NMU * kMaxQ; ++v) acc[v] = S(0);
+  }
+  R Dg[LV::NCOMP];
+  const R* buf = static_cast<const R*>(a.mbuf) + (int64_t)a.n_parts * (tile_padded(n) * LV::NCOMP);
+  LV::template load_group<G, R>(buf + tile_offset<R>(s.t, LV::NCOMP), tile_atoms<R>(), Dg);
+  for (int64_t k = s.beg; k < s.end; ++k) {
+    const int32_t j = __ldg(a.nbr_j + k);
+    const int32_t img = __ldg(a.nbr_img + k);
+    const auto l = geom.g.fetch(a, j);
+    R dx, dy, dz;
+    geom.vec(t, j, l, img, dx, dy, dz);
+    const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
+    const R rinv = rsqrt_r(r2);
+    const R r = r2 * rinv;
+    R f[NMU], df[NMU], q[kMaxQ];
+    radial<R, NMU, true, true>(sm.c + (zi * sm.S + l.species) * sm.cstride, sm.nq, r, mid, scale, rcut, f, df, q);
+    R gx, gy, gz, Smu[NMU];
+    LV::template pair_adjoint_group<G, R>(Dg, f, df, dx * rinv, dy * rinv, dz * rinv, rinv, gx, gy, gz, Smu);
+    fx += gx.t; fy += gy.t; fz += gz.t;
+    if (t.force_tan) {
+      atomicAdd(t.force_tan + 3 * (int64_t)j, -(double)gx.t);
+      atomicAdd(t.force_tan + 3 * (int64_t)j + 1, -(double)gy.t);
+      atomicAdd(t.force_tan + 3 * (int64_t)j + 2, -(double)gz.t);
+    }
+    if (own_acc) {
+      S* dst = acc + l.species * NMU * kMaxQ;
+#pragma unroll
+      for (int mu = mu_lo; mu < mu_hi; ++mu) {
+#pragma unroll
+        for (int kk = 0; kk < kMaxQ; ++kk)
+          if (kk < sm.nq) dst[mu * kMaxQ + kk] += (q[kk] * Smu[mu]).t;
+      }
+    } else {
+      S* dst = sm.dc + (zi * sm.S + l.species) * NMU * sm.nq;
+#pragma unroll
+      for (int mu = mu_lo; mu < mu_hi; ++mu) {
+#pragma unroll
+        for (int kk = 0; kk < kMaxQ; ++kk)
+          if (kk < sm.nq) atomicAdd(dst + mu * sm.nq + kk, (q[kk] * Smu[mu]).t);
+      }
     }
   }
-  __syncthreads();
-  const int S_ = sm.S, SS = sm.SS, nq = sm.nq;
-  for (int k = threadIdx.x; k < sm.m; k += blockDim.x)
-    atomicAdd(t.dtheta_tan + S_ + (int64_t)LV::NMU * nq * SS + k, (double)sm.dxi[k]);
+  if (own_acc) {
+    for (int zj = 0; zj < sm.S; ++zj) {
+      S* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
+      for (int mu = mu_lo; mu < mu_hi; ++mu)
+        for (int kk = 0; kk < sm.nq; ++kk) atomicAdd(dst + mu * sm.nq + kk, acc[(zj * NMU + mu) * kMaxQ + kk]);
+    }
+  }
+  if (t.force_tan) {
+    atomicAdd(t.force_tan + 3 * s.i, (double)fx);
+    atomicAdd(t.force_tan + 3 * s.i + 1, (double)fy);
+    atomicAdd(t.force_tan + 3 * s.i + 2, (double)fz);
+  }
 }
 
 template <class LV, class S>
 __global__ void __launch_bounds__(kEfvThreads) tangent_adjoint_kernel(const TangentArgs t) {
-  using R = Dual<S>;
   constexpr int NMU = LV::NMU;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EfvArgs& a = t.base;
@@ -253,80 +294,10 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_adjoint_kernel(const Tang
   sm.zero_gradients();
   __syncthreads();
   const int64_t n = a.atom_end - a.atom_begin;
-  const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (u < n) {
-    const int64_t i = a.atom_begin + u;
-    TangentGeom<S> geom;
-    geom.load_centre(t, i, cell_of<S>(a));
-    const int zi = species_at(a.z, i, a.n_species);
-    const int64_t beg = __ldg(a.offsets + i), end = __ldg(a.offsets + i + 1);
-    const R rcut = R(sm.rcut), mid = R(sm.mid), scale = R(sm.scale);
-    const R* buf = static_cast<const R*>(a.mbuf) + (size_t)LV::NCOMP * n + u;
-    S fx = S(0), fy = S(0), fz = S(0);
-    constexpr int kAccS = 4;
-    const bool own_acc = sm.S <= kAccS;
-    S acc[kAccS * NMU * kMaxQ];
-    if (own_acc) {
-      for (int v = 0; v < sm.S * NMU * kMaxQ; ++v) acc[v] = S(0);
-    }
-    auto sweep = [&](auto group) {
-      constexpr int G = decltype(group)::value;
-      R Dg[LV::NCOMP];
-      LV::template load_group<G, R>(buf, n, Dg);
-      for (int64_t k = beg; k < end; ++k) {
-        const int32_t j = __ldg(a.nbr_j + k);
-        const int32_t img = __ldg(a.nbr_img + k);
-        const auto l = geom.g.fetch(a, j);
-        R dx, dy, dz;
-        geom.vec(t, j, l, img, dx, dy, dz);
-        const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-        const R rinv = rsqrt_r(r2);
-        const R r = r2 * rinv;
-        R f[NMU], df[NMU], q[kMaxQ];
-        radial<R, NMU, true, true>(sm.c + (zi * sm.S + l.species) * sm.cstride, sm.nq, r, mid, scale, rcut, f, df,
-                                   q);
-        R gx, gy, gz, Smu[NMU];
-        LV::template pair_adjoint_group<G, R>(Dg, f, df, dx * rinv, dy * rinv, dz * rinv, rinv, gx, gy, gz, Smu);
-        fx += gx.t; fy += gy.t; fz += gz.t;
-        if (t.force_tan) {
-          atomicAdd(t.force_tan + 3 * (int64_t)j, -(double)gx.t);
-          atomicAdd(t.force_tan + 3 * (int64_t)j + 1, -(double)gy.t);
-          atomicAdd(t.force_tan + 3 * (int64_t)j + 2, -(double)gz.t);
-        }
-        constexpr int mu_lo = LV::GROUP_MU_LO[G], mu_hi = LV::GROUP_MU_HI[G];
-        if (own_acc) {
-          S* dst = acc + l.species * NMU * kMaxQ;
-#pragma unroll
-          for (int mu = mu_lo; mu < mu_hi; ++mu) {
-#pragma unroll
-            for (int kk = 0; kk < kMaxQ; ++kk)
-              if (kk < sm.nq) dst[mu * kMaxQ + kk] += (q[kk] * Smu[mu]).t;
-          }
-        } else {
-          S* dst = sm.dc + (zi * sm.S + l.species) * NMU * sm.nq;
-#pragma unroll
-          for (int mu = mu_lo; mu < mu_hi; ++mu) {
-#pragma unroll
-            for (int kk = 0; kk < kMaxQ; ++kk)
-              if (kk < sm.nq) atomicAdd(dst + mu * sm.nq + kk, (q[kk] * Smu[mu]).t);
-          }
-        }
-      }
-    };
-    sweep(std::integral_constant<int, 0>());
-    sweep(std::integral_constant<int, 1>());
-    if (own_acc) {
-      for (int zj = 0; zj < sm.S; ++zj) {
-        S* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-        for (int mu = 0; mu < NMU; ++mu)
-          for (int kk = 0; kk < sm.nq; ++kk) atomicAdd(dst + mu * sm.nq + kk, acc[(zj * NMU + mu) * kMaxQ + kk]);
-      }
-    }
-    if (t.force_tan) {
-      atomicAdd(t.force_tan + 3 * i, (double)fx);
-      atomicAdd(t.force_tan + 3 * i + 1, (double)fy);
-      atomicAdd(t.force_tan + 3 * i + 2, (double)fz);
-    }
+  SplitShare s;
+  if (s.setup(a, n)) {
+    if ((blockIdx.y & 1) == 0) tangent_adjoint<LV, S, 0>(t, sm, s, n);
+    else tangent_adjoint<LV, S, 1>(t, sm, s, n);
   }
   __syncthreads();
   const int S_ = sm.S, SS = sm.SS, nq = sm.nq;
@@ -342,14 +313,13 @@ int tangent_split_launch(const TangentArgs& t, cudaStream_t stream) {
   const EfvArgs& a = t.base;
   const int64_t n = a.atom_end - a.atom_begin;
   const int SS = a.n_species * a.n_species;
-  const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
+  const dim3 grid((unsigned)((n + kEfvThreads - 1) / kEfvThreads), 2 * a.n_parts);
   const size_t bytes = efv_smem_bytes<S, LV::NMU, true>(SS, a.n_q, a.m);
   int rc;
   if ((rc = set_smem(tangent_moments_kernel<LV, S>, bytes)) != MTP_OK) return rc;
-  if ((rc = set_smem(tangent_contract_kernel<LV, S>, bytes)) != MTP_OK) return rc;
   if ((rc = set_smem(tangent_adjoint_kernel<LV, S>, bytes)) != MTP_OK) return rc;
   tangent_moments_kernel<LV, S><<<grid, kEfvThreads, bytes, stream>>>(t);
-  tangent_contract_kernel<LV, S><<<grid, kEfvThreads, bytes, stream>>>(t);
+  if ((rc = tile_contract_launch<LV, Dual<S>, true>(a, t.dtheta_tan, stream)) != MTP_OK) return rc;
   tangent_adjoint_kernel<LV, S><<<grid, kEfvThreads, bytes, stream>>>(t);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -364,31 +334,31 @@ int tangent_launch(const TangentArgs& t, int precision, cudaStream_t stream) {
   const EfvArgs& a = t.base;
   const int64_t n = a.atom_end - a.atom_begin;
   if (n <= 0) return MTP_OK;
-  if constexpr (LV::NGROUPS > 1) {
-    if (a.mbuf)
-      return precision == MTP_MIXED ? tangent_split_launch<LV, float>(t, stream)
-                                    : tangent_split_launch<LV, double>(t, stream);
-  }
-  const int SS = a.n_species * a.n_species;
-  const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
-  cudaError_t e;
-  if (precision == MTP_MIXED) {
-    const size_t bytes = efv_smem_bytes<float, LV::NMU, true>(SS, a.n_q, a.m);
-    auto kern = tangent_kernel<LV, float>;
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+  if constexpr (LV::NGROUPS > 1) {   // the caller always provides the scratch
+    return precision == MTP_MIXED ? tangent_split_launch<LV, float>(t, stream)
+                                  : tangent_split_launch<LV, double>(t, stream);
   } else {
-    const size_t bytes = efv_smem_bytes<double, LV::NMU, true>(SS, a.n_q, a.m);
-    auto kern = tangent_kernel<LV, double>;
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+    const int SS = a.n_species * a.n_species;
+    const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
+    cudaError_t e;
+    if (precision == MTP_MIXED) {
+      const size_t bytes = efv_smem_bytes<float, LV::NMU, true>(SS, a.n_q, a.m);
+      auto kern = tangent_kernel<LV, float>;
+      if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+      kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+    } else {
+      const size_t bytes = efv_smem_bytes<double, LV::NMU, true>(SS, a.n_q, a.m);
+      auto kern = tangent_kernel<LV, double>;
+      if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+      kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      set_error("tangent kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+      return MTP_ERR_CUDA;
+    }
+    return MTP_OK;
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    set_error("tangent kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
-    return MTP_ERR_CUDA;
-  }
-  return MTP_OK;
 }
 
 }  // namespace mtp
