@@ -120,7 +120,7 @@ int tile_contract_launch(const EfvArgs& a, double* theta, cudaStream_t stream) {
   if (rc != MTP_OK) return rc;
   const int64_t n = a.atom_end - a.atom_begin;
   const int64_t tiles = (n + tile_atoms<R>() - 1) / tile_atoms<R>();
-  constexpr int resident = (int)(227 * 1024 / (bytes + 1024)) < 3 ? (int)(227 * 1024 / (bytes + 1024)) : 3;
+  constexpr int resident = (int)(227 * 1024 / (bytes + 1024)) < 2 ? (int)(227 * 1024 / (bytes + 1024)) : 2;
   static_assert(resident >= 1, "a tile's slots fit in the shared memory of an SM");
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)device_sms() * resident);
   kern<<<(unsigned)grid, kTileThreads, bytes, stream>>>(a, theta);

@@ -383,6 +383,7 @@ void mtp_free_nlist(mtp_nlist* nl) {
   nl->bin_start.release();
   nl->bin_atoms.release();
   nl->wrapped.release();
+  nl->columns.release();
   nl->status.release();
   delete nl;
 }

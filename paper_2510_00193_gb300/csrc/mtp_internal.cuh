@@ -170,5 +170,5 @@ struct mtp_nlist {
   double cell[9] = {0};
   int pbc[3] = {0, 0, 0};
   mtp::DevBuf offsets, nbr_j, nbr_img;
-  mtp::DevBuf counts, bins, bin_start, bin_atoms, wrapped, status;
+  mtp::DevBuf counts, bins, bin_start, bin_atoms, wrapped, columns, status;
 };

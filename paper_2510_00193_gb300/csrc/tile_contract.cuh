@@ -26,7 +26,7 @@
 
 namespace mtp {
 
-constexpr int kTileThreads = 512;
+constexpr int kTileThreads = 1024;
 constexpr int kTileRowBytes = 32;
 constexpr int kTileLanes = 16;   // records per warp (two threads each), as the programs are encoded
 
