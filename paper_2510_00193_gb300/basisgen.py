@@ -1033,6 +1033,201 @@ def emit_contract_by_graph(lv: Level, fname="contract"):
     return L
 
 
+CONTRACT_PARTS = 4   # warps that share the contraction of one group of atoms
+
+
+def emit_contract_parts(lv: Level):
+    """The per-graph contraction cut into CONTRACT_PARTS parts for the warps of
+    a block that share the same atoms: part_values<P> forms the values of the
+    part's graphs, part_adjoint<P> (once every part's values are there) its
+    share of the basis values and of E, the adjoints of its graphs and its
+    contribution to D.  Swept moment components are read and D is returned by
+    their position k among the swept ones (M[k], D[k]); G(g) reads and
+    G.put(g, v) stores the value of graph g.  The graphs are dealt to the parts
+    by their operation counts, largest first."""
+    dag = lv.dag
+    ind = "    "
+    pos = {c: k for k, c in enumerate(lv.swept)}
+    exp_order = sorted(lv.expand, key=lambda t: (lv.comps[t][1][2], t))
+
+    def node_ops(n):
+        key, rank = dag.nodes[n]
+        return 3 * n_sym(rank) * n_sym(dag.rank(key[2])) if key[0] == "C" else 0
+
+    closures = [_node_closure(dag, roots) for roots in lv.roots]
+    cost = [8 + sum(node_ops(n) for n in cl) for cl in closures]
+    parts = [[] for _ in range(CONTRACT_PARTS)]
+    for gi in sorted(range(len(cost)), key=lambda g: (-cost[g], g)):
+        min(parts, key=lambda q: (sum(cost[k] for k in q), len(q))).append(gi)
+    parts = [sorted(q) for q in parts]
+    bases = [[] for _ in range(CONTRACT_PARTS)]
+    for a in range(len(lv.bases)):
+        bases[a % CONTRACT_PARTS].append(a)
+
+    def used_comps(nodes):
+        used = set()
+        for n in nodes:
+            key, rank = dag.nodes[n]
+            if key[0] == "M":
+                _, mu, nu, off = key
+                for K in multi_indices(rank):
+                    used.add(lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))])
+        stack = list(used)
+        while stack:
+            for t in lv.expand.get(stack.pop(), ()):
+                if t not in used:
+                    used.add(t)
+                    stack.append(t)
+        return used
+
+    def emit_forward(L, nodes, sfx, barrier):
+        """Moment components and C nodes of `nodes`; returns comp_ref and the weighted operands."""
+        used = used_comps(nodes)
+
+        def mname(c):
+            return ("mx%d%s" % (c, sfx)) if c in lv.expand else ("m%d%s" % (c, sfx))
+
+        for c in sorted(t for t in used if t not in lv.expand):
+            L.append(ind + "R %s = M[%d];" % (mname(c), pos[c]))
+            if barrier:
+                L.append(ind + "opaque(%s);" % mname(c))
+        for c in exp_order:
+            if c in used:
+                s0, s1, s2 = (mname(t) for t in lv.expand[c])
+                L.append(ind + "const R %s = (%s - %s) - %s;" % (mname(c), s0, s1, s2))
+
+        def comp_ref(n, K):
+            key, rank = dag.nodes[n]
+            if key[0] == "M":
+                _, mu, nu, off = key
+                return mname(lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))])
+            return "v%d_%d%s" % (n, multi_indices(rank).index(K), sfx)
+
+        wname = {}
+        for n in sorted(nodes):
+            key, rank = dag.nodes[n]
+            if key[0] != "C":
+                continue
+            _, a, b = key
+            Ps = multi_indices(dag.rank(b))
+            wname[n] = []
+            for j, P in enumerate(Ps):
+                w = multinomial_weight(P)
+                if w == 1:
+                    wname[n].append(comp_ref(b, P))
+                else:
+                    nm = "w%d_%d%s" % (n, j, sfx)
+                    L.append(ind + "const R %s = R(%d) * %s;" % (nm, w, comp_ref(b, P)))
+                    wname[n].append(nm)
+            for ki, K in enumerate(multi_indices(rank)):
+                emit_dot(L, ind, "v%d_%d%s" % (n, ki, sfx),
+                         [(comp_ref(a, tuple(K[d] + P[d] for d in range(3))), wname[n][j]) for j, P in enumerate(Ps)])
+        return comp_ref, wname
+
+    gbar = defaultdict(list)
+    for a, b in enumerate(lv.bases):
+        for j in range(len(b)):
+            gbar[b[j]].append((a, [b[t] for t in range(len(b)) if t != j]))
+    out = ["  static constexpr int NPARTS = %d, NSWEPT = %d;" % (CONTRACT_PARTS, len(lv.swept))]
+    for fn, args, body in (("store_swept", "const R* __restrict__ M, V dst", "dst[%d] = M[%d];"),
+                           ("load_swept", "R* __restrict__ M, V src", "M[%d] = src[%d];")):
+        out.append("  template <class R, class V>")
+        out.append("  __device__ __forceinline__ static void %s(%s) {" % (fn, args))
+        for c in range(len(lv.comps)):
+            if c in pos:
+                out.append(ind + body % ((pos[c], c) if fn == "store_swept" else (c, pos[c])))
+            elif fn == "load_swept":
+                out.append(ind + "M[%d] = R(0);" % c)
+        out.append("  }")
+    for q in range(CONTRACT_PARTS):
+        L = ["  template <class R, class MV, class GV>",
+             "  __device__ __forceinline__ static void part_values_%d(MV M, GV G) {" % q]
+        nodes = set().union(*[closures[g] for g in parts[q]]) if parts[q] else set()
+        cref, _ = emit_forward(L, nodes, "", False)
+        for gi in parts[q]:
+            terms = [cref(n, (0, 0, 0)) if w == 1 else "R(%d) * %s" % (w, cref(n, (0, 0, 0))) for w, n in lv.roots[gi]]
+            L.append(ind + "G.put(%d, %s);" % (gi, tree_sum(terms)))
+        L.append("  }")
+        out += L
+        L = ["  template <class R, bool WANT_B, class MV, class GV, class BV>",
+             "  __device__ __forceinline__ static R part_adjoint_%d(MV M, GV G, const typename ScalarOf<R>::T* "
+             "__restrict__ xi, R* __restrict__ D, BV B) {" % q,
+             ind + "(void)B;"]
+        need = {k for a in bases[q] for k in lv.bases[a]} | {k for g in parts[q] for _, o in gbar[g] for k in o}
+        for k in sorted(need):
+            L.append(ind + "const R G%d = G(%d);" % (k, k))
+        L.append(ind + "R E = R(0);")
+        for a in bases[q]:
+            L.append(ind + "const R B%d = %s;" % (a, " * ".join("G%d" % k for k in lv.bases[a])))
+            L.append(ind + "if (WANT_B) store_basis(B, %d, B%d);" % (a, a))
+            L.append(ind + "E = fmadd(R(xi[%d]), B%d, E);" % (a, a))
+        for gi in parts[q]:
+            L.append(ind + "const R Gb%d = %s;" % (gi, tree_sum(
+                ["R(xi[%d])" % a + "".join(" * G%d" % k for k in o) for a, o in gbar[gi]])))
+        for k in range(len(lv.swept)):
+            L.append(ind + "D[%d] = R(0);" % k)
+        for gi in parts[q]:
+            sfx = "_g%d" % gi
+            nodes = closures[gi]
+            cref, wname = emit_forward(L, nodes, sfx, True)
+            adj, dpos, dneg = defaultdict(list), defaultdict(list), defaultdict(list)
+            for w, node in lv.roots[gi]:
+                adj[(node, 0)].append("Gb%d" % gi if w == 1 else "R(%d) * Gb%d" % (w, gi))
+            for n in sorted(nodes, reverse=True):
+                key, rank = dag.nodes[n]
+                names = []
+                for ki in range(n_sym(rank)):
+                    ex = adj.get((n, ki))
+                    nm = "b%d_%d%s" % (n, ki, sfx) if ex else None
+                    if ex:
+                        L.append(ind + "const R %s = %s;" % (nm, tree_sum(ex)))
+                    names.append(nm)
+                if key[0] == "M":
+                    _, mu, nu, off = key
+                    for ki, K in enumerate(multi_indices(rank)):
+                        if names[ki]:
+                            dpos[lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))]].append(names[ki])
+                    continue
+                _, a, b = key
+                Ps = multi_indices(dag.rank(b))
+                full_idx = multi_indices(dag.rank(a))
+                bacc = defaultdict(list)
+                for ki, K in enumerate(multi_indices(rank)):
+                    if not names[ki]:
+                        continue
+                    for j, P in enumerate(Ps):
+                        full = tuple(K[d] + P[d] for d in range(3))
+                        adj[(a, full_idx.index(full))].append("%s * %s" % (names[ki], wname[n][j]))
+                        bacc[j].append((names[ki], cref(a, full)))
+                for j, lst in bacc.items():
+                    w = multinomial_weight(Ps[j])
+                    nm = "c%d_%d%s" % (n, j, sfx)
+                    emit_dot(L, ind, nm, lst)
+                    adj[(b, j)].append(nm if w == 1 else "R(%d) * %s" % (w, nm))
+            for c in sorted(lv.expand, key=lambda t: (-lv.comps[t][1][2], -t)):
+                if not dpos.get(c) and not dneg.get(c):
+                    continue
+                nm = "dx%d%s" % (c, sfx)
+                val = tree_sum(dpos[c]) if dpos.get(c) else "R(0)"
+                L.append(ind + "const R %s = %s;" % (nm, val if not dneg.get(c) else "%s - %s" % (val, tree_sum(dneg[c]))))
+                s0, s1, s2 = lv.expand[c]
+                dpos[s0].append(nm)
+                dneg[s1].append(nm)
+                dneg[s2].append(nm)
+            for c in sorted(set(dpos) | set(dneg)):
+                if c in lv.expand:
+                    continue
+                ex = "D[%d]" % pos[c]
+                if dpos.get(c):
+                    ex = "%s + %s" % (ex, tree_sum(dpos[c]))
+                if dneg.get(c):
+                    ex = "(%s) - %s" % (ex, tree_sum(dneg[c]))
+                L.append(ind + "D[%d] = %s;" % (pos[c], ex))
+        L += [ind + "return E;", "  }"]
+        out += L
+    return out
+
+
 # Contraction code shape for the straight-line levels in FP32: the reverse
 # pass graph by graph with recomputed nodes (True) or over the whole DAG
 # (False).  FP64 and dual-number code always take the whole-DAG form (the
@@ -1380,6 +1575,7 @@ def emit_header(lv: Level):
         out += (emit_contract_by_graph(lv, "contract_graph") if CONTRACT_BY_GRAPH
                 else emit_contract(lv, "contract_graph"))
         out += emit_contract_dispatch()
+        out += emit_contract_parts(lv)
     out.append("};")
     out.append("}  // namespace mtp")
     return "\n".join(out) + "\n"

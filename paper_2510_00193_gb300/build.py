@@ -59,12 +59,11 @@ def generate_sources(levels=LEVELS):
     basisgen.generate(GEN, levels)
     units = []
     for L in levels:
+        # two units per level, so that the long compilations run side by side
+        head = "// Generated by paper_2510_00193_gb300/build.py.\n#include \"%%s\"\n%%s#include \"mtp_level%d.cuh\"\n" % L
         path = os.path.join(GEN, "efv_level%d.cu" % L)
-        _write(path, (
-            "// Generated by paper_2510_00193_gb300/build.py.\n"
-            "#include \"efv_split.cuh\"\n#include \"grade_kernel.cuh\"\n#include \"batch_kernel.cuh\"\n"
-            "#include \"tangent_kernel.cuh\"\n#include \"efv_team.cuh\"\n"
-            "#include \"mtp_level%d.cuh\"\n"
+        _write(path, head % ("efv_split.cuh", "#include \"grade_kernel.cuh\"\n#include \"batch_kernel.cuh\"\n"
+                                              "#include \"tangent_kernel.cuh\"\n") + (
             "namespace mtp {\nint efv_level%d(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t s) {\n"
             "  return efv_launch<MtpLevel%d>(a, precision, want_dtheta, s);\n}\n"
             "int rows_level%d(const EfvArgs& a, const int32_t* list, int64_t n, double* rows, int64_t ld, double* bsum,"
@@ -74,9 +73,19 @@ def generate_sources(levels=LEVELS):
             "int tangent_level%d(const TangentArgs& t, int precision, cudaStream_t s) {\n"
             "  return tangent_launch<MtpLevel%d>(t, precision, s);\n}\n"
             "int split_level%d() { return MtpLevel%d::NGROUPS > 1 ? MtpLevel%d::NCOMP : 0; }\n"
-            "int team_level%d(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t s) {\n"
-            "  return efv_team_launch<MtpLevel%d>(a, precision, want_dtheta, s);\n}\n"
-            "}  // namespace mtp\n") % (L, L, L, L, L, L, L, L, L, L, L, L, L, L))
+            "}  // namespace mtp\n") % (L, L, L, L, L, L, L, L, L, L, L))
+        units.append(path)
+        path = os.path.join(GEN, "team_level%d.cu" % L)
+        body = ("namespace mtp {\nint efv_level%d(const EfvArgs&, int, bool, cudaStream_t);\n"
+                "int team_level%d(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t s) {\n" % (L, L))
+        if L >= basisgen.INTERPRET_FROM_LEVEL:   # the split kernels cover small systems too
+            head = "// Generated by paper_2510_00193_gb300/build.py.\n#include \"mtp_internal.cuh\"\n"
+            body += "  return efv_level%d(a, precision, want_dtheta, s);\n" % L
+        else:
+            head = head % ("efv_team.cuh", "")
+            body += ("  const int rc = efv_team_launch<MtpLevel%d>(a, precision, want_dtheta, s);\n"
+                     "  return rc == kTeamNoRoom ? efv_level%d(a, precision, want_dtheta, s) : rc;\n" % (L, L))
+        _write(path, head + body + "}\n}  // namespace mtp\n")
         units.append(path)
     decl = "".join("int efv_level%d(const EfvArgs&, int, bool, cudaStream_t);\n"
                    "int rows_level%d(const EfvArgs&, const int32_t*, int64_t, double*, int64_t, double*, cudaStream_t);\n"

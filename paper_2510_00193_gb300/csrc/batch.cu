@@ -52,25 +52,66 @@ __global__ void batch_frac_kernel(const double* __restrict__ x, const int64_t* _
   cfg_of[i] = lo;
 }
 
-// Fixed-point fractional coordinates with each atom's own cell (mixed path).
-__global__ void batch_fixed_point_kernel(const double* __restrict__ s, const int32_t* __restrict__ z, int64_t n,
-                                         int S, long long* __restrict__ out, int* __restrict__ status) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double k = 4294967296.0;
-  const double s0 = s[3 * i], s1 = s[3 * i + 1], s2 = s[3 * i + 2];
-  const int zi = z[i];
-  const bool z_ok = zi >= 0 && zi < S;
-  if (!z_ok) atomicCAS(status, 0, MTP_ERR_ARG);
-  out[4 * i + 3] = z_ok ? (long long)zi : 0ll;   // out-of-range species read as 0 (reported above)
-  if (!(fabs(s0) < 2147483647.0 && fabs(s1) < 2147483647.0 && fabs(s2) < 2147483647.0)) {
-    atomicCAS(status, 0, MTP_ERR_NONFINITE);   // stored as the origin: no kernel reads undefined coordinates
-    out[4 * i] = out[4 * i + 1] = out[4 * i + 2] = 0ll;
+// Everything a batched evaluation needs before its kernel, in one launch: the
+// cleared outputs and work queue and, on the mixed path, the fixed-point
+// fractional coordinates with each atom's own cell.
+struct BatchPrepArgs {
+  const double* x;
+  const int32_t* z;
+  const int64_t* off;
+  const double* hinv;
+  int64_t n;
+  int n_cfg, n_species;
+  double *e_cfg, *virial, *dtheta, *forces;   // forces: FP64 path; dtheta: nullable
+  int64_t n_dtheta;
+  float* forces_f;
+  long long* xq;
+  int32_t* queue;
+  int* status;
+};
+
+template <bool MIXED>
+__global__ void batch_prep_kernel(const BatchPrepArgs a) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  if (i == 0) *a.queue = 0;
+  for (int64_t k = i; k < 6 * (int64_t)a.n_cfg; k += step) {
+    if (k < a.n_cfg) a.e_cfg[k] = 0.0;
+    a.virial[k] = 0.0;
+  }
+  if (a.dtheta)
+    for (int64_t k = i; k < a.n_dtheta; k += step) a.dtheta[k] = 0.0;
+  if (i >= a.n) return;
+  if constexpr (!MIXED) {
+    a.forces[i] = a.forces[a.n + i] = a.forces[2 * a.n + i] = 0.0;
     return;
   }
-  out[4 * i] = __double2ll_rn(s0 * k);
-  out[4 * i + 1] = __double2ll_rn(s1 * k);
-  out[4 * i + 2] = __double2ll_rn(s2 * k);
+  a.forces_f[i] = a.forces_f[a.n + i] = a.forces_f[2 * a.n + i] = 0.f;
+  int lo = 0, hi = a.n_cfg - 1;
+  while (lo < hi) {  // last configuration whose first atom <= i
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.off[mid] <= i) lo = mid; else hi = mid - 1;
+  }
+  const double* h = a.hinv + 9 * (int64_t)lo;
+  const double px = a.x[3 * i], py = a.x[3 * i + 1], pz = a.x[3 * i + 2];
+  const double s0 = px * h[0] + py * h[3] + pz * h[6];
+  const double s1 = px * h[1] + py * h[4] + pz * h[7];
+  const double s2 = px * h[2] + py * h[5] + pz * h[8];
+  const double k = 4294967296.0;
+  const int zi = a.z[i];
+  const bool z_ok = zi >= 0 && zi < a.n_species;
+  if (!z_ok) atomicCAS(a.status, 0, MTP_ERR_ARG);
+  // out-of-range species are read as 0 (reported above); a non-finite position
+  // is stored as the origin: no kernel reads undefined coordinates
+  longlong2 p = make_longlong2(0ll, 0ll), q = make_longlong2(0ll, z_ok ? (long long)zi : 0ll);
+  if (fabs(s0) < 2147483647.0 && fabs(s1) < 2147483647.0 && fabs(s2) < 2147483647.0) {
+    p = make_longlong2(__double2ll_rn(s0 * k), __double2ll_rn(s1 * k));
+    q.x = __double2ll_rn(s2 * k);
+  } else {
+    atomicCAS(a.status, 0, MTP_ERR_NONFINITE);
+  }
+  longlong2* out = reinterpret_cast<longlong2*>(a.xq + 4 * i);
+  out[0] = p;
+  out[1] = q;
 }
 
 struct BatchNbrArgs {
@@ -395,11 +436,11 @@ int mtp_compute_batch(mtp_handle* h, const mtp_batch* b, const double* x, const 
   }
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t n = b->n_atoms;
-  MTP_TRY_CUDA(cudaMemsetAsync(e_cfg, 0, sizeof(double) * b->n_cfg, s));
-  MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6 * b->n_cfg, s));
-  if (dtheta) MTP_TRY_CUDA(cudaMemsetAsync(dtheta, 0, sizeof(double) * h->n_params * b->n_cfg, s));
-  MTP_TRY_CUDA(cudaMemsetAsync(b->queue.ptr, 0, sizeof(int32_t), s));
-  if (precision == MTP_FP64 || n == 0) MTP_TRY_CUDA(cudaMemsetAsync(forces, 0, sizeof(double) * 3 * n, s));
+  if (n == 0) {
+    MTP_TRY_CUDA(cudaMemsetAsync(e_cfg, 0, sizeof(double) * b->n_cfg, s));
+    MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6 * b->n_cfg, s));
+    if (dtheta) MTP_TRY_CUDA(cudaMemsetAsync(dtheta, 0, sizeof(double) * h->n_params * b->n_cfg, s));
+  }
   if (n == 0) return MTP_OK;
   BatchArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -424,19 +465,17 @@ int mtp_compute_batch(mtp_handle* h, const mtp_batch* b, const double* x, const 
   e.forces = forces;
   e.status = h->status.as<int>();
   e.e_atom = e_atom ? e_atom : b->eatom.as<double>();
-  const unsigned blocks = (unsigned)((n + 255) / 256);
   if (precision == MTP_MIXED) {
-    // fractional coordinates of the current positions, then fixed point
-    double* hinv_d = reinterpret_cast<double*>(b->work.ptr);
-    double* sfrac = reinterpret_cast<double*>(b->frac.ptr);
-    int32_t* cfg_of = reinterpret_cast<int32_t*>(sfrac + 3 * n);
-    batch_frac_kernel<<<blocks, 256, 0, s>>>(x, b->off.as<int64_t>(), b->n_cfg, hinv_d, n, sfrac, cfg_of);
-    batch_fixed_point_kernel<<<blocks, 256, 0, s>>>(sfrac, z, n, h->n_species, b->xq.as<long long>(), e.status);
-    MTP_TRY_CUDA(cudaGetLastError());
     e.xq = b->xq.as<long long>();
     e.forces_f = b->forces_f.as<float>();
-    MTP_TRY_CUDA(cudaMemsetAsync(e.forces_f, 0, sizeof(float) * 3 * n, s));
   }
+  BatchPrepArgs pa{x, z, b->off.as<int64_t>(), reinterpret_cast<double*>(b->work.ptr), n, b->n_cfg, h->n_species,
+                   e_cfg, virial, dtheta, forces, (int64_t)h->n_params * b->n_cfg, const_cast<float*>(e.forces_f),
+                   const_cast<long long*>(e.xq), b->queue.as<int32_t>(), e.status};
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  if (precision == MTP_MIXED) batch_prep_kernel<true><<<blocks, 256, 0, s>>>(pa);
+  else batch_prep_kernel<false><<<blocks, 256, 0, s>>>(pa);
+  MTP_TRY_CUDA(cudaGetLastError());
   a.item_cfg = b->items_cfg.as<int32_t>();
   a.item_begin = b->items_begin.as<int64_t>();
   a.item_count = b->items_count.as<int32_t>();

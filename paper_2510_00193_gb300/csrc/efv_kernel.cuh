@@ -733,7 +733,8 @@ __device__ __forceinline__ void efv_atom(const EfvArgs& a, const EfvShared<R, LV
   PairGeom<R> geom;
   geom.load_centre(a, i, cell);
   const int zi = species_at(a.z, i, a.n_species);
-  const int64_t beg = active ? __ldg(a.offsets + i) : 0, end = active ? __ldg(a.offsets + i + 1) : 0;
+  int64_t beg = 0, end = 0;
+  if (active) list_row(a, i, beg, end);
   R M[LV::NCOMP];
 #pragma unroll
   for (int c = 0; c < LV::NCOMP; ++c) M[c] = R(0);

@@ -47,9 +47,6 @@ constexpr int kNoAllocMaxDevices = 64;
 // [4 * kNoAllocMaxAtoms] int64 positions, then [3 * kNoAllocMaxAtoms] floats
 static __device__ __align__(256) long long g_noalloc_scratch[4 * kNoAllocMaxAtoms + 3 * kNoAllocMaxAtoms / 2];
 
-__global__ void fixed_point_kernel(const double* __restrict__ x, const int32_t* __restrict__ z, int64_t n,
-                                   double h0, double h1, double h2, double h3, double h4, double h5, double h6,
-                                   double h7, double h8, int S, long long* __restrict__ out, int* __restrict__ status);
 __global__ void forces_to_fp64_kernel(const float* __restrict__ f, int64_t n3, double* __restrict__ out);
 
 static std::mutex g_noalloc_mutex;
@@ -117,25 +114,25 @@ extern "C" int mtp_compute_efv_noalloc(mtp_handle* h, const mtp_nlist* nl, const
 
   cudaStream_t s = (cudaStream_t)stream;
   float* forces_f = reinterpret_cast<float*>(scratch + 4 * kNoAllocMaxAtoms);
-  MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6, s));
-  MTP_TRY_CUDA(cudaMemsetAsync(e_total, 0, sizeof(double), s));
-  if (n == 0) return MTP_OK;
+  if (n == 0) {
+    MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6, s));
+    MTP_TRY_CUDA(cudaMemsetAsync(e_total, 0, sizeof(double), s));
+    return MTP_OK;
+  }
 
-  double hi[9];
-  hi[0] = (cell[4] * cell[8] - cell[5] * cell[7]) / det;
-  hi[1] = (cell[2] * cell[7] - cell[1] * cell[8]) / det;
-  hi[2] = (cell[1] * cell[5] - cell[2] * cell[4]) / det;
-  hi[3] = (cell[5] * cell[6] - cell[3] * cell[8]) / det;
-  hi[4] = (cell[0] * cell[8] - cell[2] * cell[6]) / det;
-  hi[5] = (cell[2] * cell[3] - cell[0] * cell[5]) / det;
-  hi[6] = (cell[3] * cell[7] - cell[4] * cell[6]) / det;
-  hi[7] = (cell[1] * cell[6] - cell[0] * cell[7]) / det;
-  hi[8] = (cell[0] * cell[4] - cell[1] * cell[3]) / det;
-  fixed_point_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, z, n, hi[0], hi[1], hi[2], hi[3], hi[4], hi[5],
-                                                                 hi[6], hi[7], hi[8], h->n_species, scratch,
-                                                                 h->status.as<int>());
-  MTP_TRY_CUDA(cudaGetLastError());
-  MTP_TRY_CUDA(cudaMemsetAsync(forces_f, 0, sizeof(float) * 3 * (size_t)n, s));
+  PrepArgs pa;
+  std::memset(&pa, 0, sizeof(pa));
+  pa.x = x;
+  pa.z = z;
+  pa.n = n;
+  pa.n_species = h->n_species;
+  pa.xq = scratch;
+  pa.forces_f = forces_f;
+  pa.virial = virial;
+  pa.e_total = e_total;
+  pa.status = h->status.as<int>();
+  inverse_rows(cell, 4294967296.0, pa.h);
+  if ((rc = launch_prep(pa, true, s)) != MTP_OK) return rc;
 
   EfvArgs a;
   std::memset(&a, 0, sizeof(a));

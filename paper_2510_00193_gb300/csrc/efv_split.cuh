@@ -23,7 +23,9 @@ struct SplitShare {
     active = t < n;
     i = a.atom_begin + (active ? t : 0);
     const int part = blockIdx.y >> 1;
-    const int64_t b = __ldg(a.offsets + i), len = __ldg(a.offsets + i + 1) - b;
+    int64_t b, e;
+    list_row(a, i, b, e);
+    const int64_t len = e - b;
     beg = b + len * part / a.n_parts;
     end = active ? b + len * (part + 1) / a.n_parts : beg;
     return __any_sync(0xffffffffu, t < tile_padded(n));

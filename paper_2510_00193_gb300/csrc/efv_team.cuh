@@ -1,197 +1,223 @@
-// Warp-per-atom energy/force kernel: the block-parallel variant for small
-// systems and high levels (the paper keeps a separate GPU pair style that
-// spreads one atom's work over a team of threads for this regime, Sec. 2.1,
-// Table 1, and Sec. 4).  With few atoms the one-thread-per-atom kernel leaves
-// most of the GPU idle and each thread walks all of its ~26-54 neighbours in
-// sequence; here the 32 lanes of a warp share one atom:
-//   sweep 1: lane l takes the pairs l, l + 32, ... and accumulates partial
-//            moments in registers (the generated per-pair code);
-//   reduce:  the partial moments go through a per-warp shared-memory
-//            transpose [c][lane] and lane l sums the components c = l (mod 32);
-//   contract: every lane loads the full moment vector (broadcast reads) and
-//            runs the contraction and its reverse pass redundantly (one
-//            instruction stream for the warp, so this costs the same issue
-//            slots as one lane) and so holds D = dE_i/dM in registers;
-//   sweep 2: lane l takes the same pairs as in sweep 1, scatters F_j -= g and
-//            keeps its share of F_i, W and dE/dc; F_i is summed across the warp.
+// Energy/force kernel in which the W warps of a block share 32 atoms (lane =
+// atom): the block-parallel variant (the paper keeps a separate GPU pair style
+// that spreads one atom's work over a team of threads for small systems, Sec.
+// 2.1, Table 1, and Sec. 4).  With one thread per atom a system of a few
+// thousand atoms leaves most of the GPU idle, and every thread walks ~26-54
+// pairs twice and a contraction of ~10k instructions in sequence.  Here
+//   sweep 1: warp w takes the w-th share of every lane's pairs; the partial
+//            moments meet in shared memory ([w][component][lane], no bank
+//            conflicts) and are added component by component;
+//   contract: warp p runs part p of the generated contraction on all 32
+//            atoms (part_values<p>, then part_adjoint<p> once the graph values
+//            of all parts are there), so the warps execute different code on
+//            the same atoms and no work is repeated but the recomputed nodes;
+//            the parts' shares of D = dE_i/dM are added as the moments were;
+//   sweep 2: warp w takes its share of the pairs again; F_i is added across
+//            the warps in shared memory, F_j -= g is scattered.
+// Taken for systems whose blocks fit in one wave (the rule stands at the call);
+// above that the instruction streams of four different contraction parts on an
+// SM cost more than the idle lanes of one thread per atom.  Level 16, mixed
+// energies and forces, this kernel / one thread per atom (whole call, us):
+// 2,000 atoms 39 / 60, 8,192 45 / 57, 16,000 74 / 57; with dE/dtheta 73 / 190,
+// 79 / 191, 144 / 193; FP64 2,000 atoms 284 / 939, 16,000 1,089 / 963.  The
+// form before (one warp per atom, every lane running the whole contraction)
+// took 59 us at 2,000 atoms.  Bound: instruction fetch (ncu: 3.1 of 6.5 stalled
+// warps per issue wait for instructions at 2,000 atoms).
 // Levels with component groups (18 and 20) run the split kernels at every size.
 #pragma once
-#include "efv_split.cuh"
+#include "efv_kernel.cuh"
 
 namespace mtp {
 
-constexpr int kTeamWarps = 4;   // atoms (warps) per block of 128 threads
+// Many species with a large radial basis: the coefficients leave no room for
+// the shares (the caller takes one thread per atom then).
+constexpr int kTeamNoRoom = 1000;
+constexpr int kTeamWarps = 4;   // 8 measured slower above 2,000 atoms (the extra warps wait through the contraction)
 
-template <class R>
-__host__ __device__ __forceinline__ size_t team_buf_bytes(int ncomp) {
-  return sizeof(R) * (size_t)kTeamWarps * (size_t)ncomp * 33;
+// A lane's column of a [k][32] array in shared memory.
+template <class R> struct LaneColumn {
+  R* p;
+  __device__ __forceinline__ R& operator[](int k) const { return p[k * 32]; }
+};
+template <class R> struct GraphColumn {
+  R* p;
+  __device__ __forceinline__ R operator()(int g) const { return p[g * 32]; }
+  __device__ __forceinline__ void put(int g, R v) const { p[g * 32] = v; }
+};
+
+template <class LV, class R>
+__host__ __device__ __forceinline__ size_t team_buf_bytes(int W) {
+  // partial moments / D shares, their sum, graph values, energies of the parts, forces of the warps
+  const size_t shares = W > LV::NPARTS ? W : LV::NPARTS;
+  return sizeof(R) * 32 * (shares * LV::NSWEPT + LV::NSWEPT + LV::NGRAPH + LV::NPARTS + 3 * (size_t)W);
 }
 
-template <class LV, class R, bool DTHETA, int NQ = 0>
-__global__ void __launch_bounds__(kEfvThreads) efv_team_kernel(const EfvArgs a) {
-  static_assert(LV::NGROUPS == 1, "warp-per-atom kernel: levels with one component group");
-  constexpr int NMU = LV::NMU;
-  const int nq = NQ > 0 ? NQ : a.n_q;
-  constexpr int C = LV::NCOMP;
+template <class LV, class R>
+__device__ __forceinline__ void team_values(int p, LaneColumn<R> M, GraphColumn<R> G) {
+  if (p == 0) LV::template part_values_0<R>(M, G);
+  else if (p == 1) LV::template part_values_1<R>(M, G);
+  else if (p == 2) LV::template part_values_2<R>(M, G);
+  else LV::template part_values_3<R>(M, G);
+}
+
+template <class LV, class R, bool WANT_B, class BV>
+__device__ __forceinline__ R team_adjoint(int p, LaneColumn<R> M, GraphColumn<R> G,
+                                          const typename ScalarOf<R>::T* xi, LaneColumn<R> share, BV B) {
+  auto put = [&](const R (&D)[LV::NSWEPT]) {
+#pragma unroll
+    for (int k = 0; k < LV::NSWEPT; ++k) share[k] = D[k];
+  };
+  R D[LV::NSWEPT];
+  R e;
+  if (p == 0) { e = LV::template part_adjoint_0<R, WANT_B>(M, G, xi, D, B); put(D); }
+  else if (p == 1) { e = LV::template part_adjoint_1<R, WANT_B>(M, G, xi, D, B); put(D); }
+  else if (p == 2) { e = LV::template part_adjoint_2<R, WANT_B>(M, G, xi, D, B); put(D); }
+  else { e = LV::template part_adjoint_3<R, WANT_B>(M, G, xi, D, B); put(D); }
+  return e;
+}
+
+template <class LV, class R, bool DTHETA, int W, int NQ>
+__global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
+  static_assert(LV::NGROUPS == 1, "levels with one component group");
+  static_assert(LV::NPARTS == 4, "four parts");
+  constexpr int NMU = LV::NMU, NSW = LV::NSWEPT, NP = LV::NPARTS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EfvShared<R, NMU, DTHETA> sm;
   sm.setup(a, smem_raw);
   sm.zero_gradients();
   const int SS = a.n_species * a.n_species;
-  R* tbuf = reinterpret_cast<R*>(smem_raw + ((efv_smem_bytes<R, NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)));
-  __syncthreads();
+  constexpr int SHARES = W > NP ? W : NP;
+  R* shares = reinterpret_cast<R*>(smem_raw + ((efv_smem_bytes<R, NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
+                                   efv_acc_bytes<R, NMU, DTHETA>(a.n_species, a.n_q, 32 * W));
+  R* total = shares + SHARES * NSW * 32;
+  R* graphs = total + NSW * 32;
+  R* energy = graphs + LV::NGRAPH * 32;
+  R* force = energy + NP * 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  R* tb = tbuf + (size_t)warp * C * 33;   // [c][33]: 32 lane partials, then the total
-  const int64_t i = a.atom_begin + (int64_t)blockIdx.x * kTeamWarps + warp;
-  const bool active = i < a.atom_end;   // warp-uniform
-  double e_i = 0.0;
-  R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-  if (active) {
-    const R* cell = cell_of<R>(a);
-    PairGeom<R> geom;
-    geom.load_centre(a, i, cell);
-    const int zi = species_at(a.z, i, a.n_species);
-    const int64_t beg = __ldg(a.offsets + i), end = __ldg(a.offsets + i + 1);
-    const R* cz = sm.c + zi * sm.S * sm.cstride;
-    // sweep 1: partial moments of this lane's pairs
-    R M[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) M[c] = R(0);
-    for (int64_t k = beg + lane; k < end; k += 32) {
-      const int32_t j = __ldg(a.nbr_j + k), img = __ldg(a.nbr_img + k);
-      const typename PairGeom<R>::Load lj = geom.fetch(a, j);
-      R dx, dy, dz;
-      geom.vec(a, lj, img, dx, dy, dz);
-      const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-      const R rinv = rsqrt_r(r2);
-      const R r = r2 * rinv;
-      R f[NMU];
-      radial<R, NMU, false, false, NQ>(cz + lj.species * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut, f,
-                                       nullptr, nullptr);
-      LV::template moments<R>(M, f, dx * rinv, dy * rinv, dz * rinv);
+  const int64_t i0 = a.atom_begin + (int64_t)blockIdx.x * 32 + lane;
+  const bool active = i0 < a.atom_end;
+  const int64_t i = active ? i0 : a.atom_begin;
+  __syncthreads();
+  PairGeom<R> geom;
+  geom.load_centre(a, i, cell_of<R>(a));
+  const int zi = species_at(a.z, i, a.n_species);
+  int64_t row, row_end;
+  list_row(a, i, row, row_end);
+  const int len = active ? (int)(row_end - row) : 0;
+  const int64_t beg = row + (int64_t)len * warp / W, end = row + (int64_t)len * (warp + 1) / W;
+  const LaneColumn<R> mine{shares + (size_t)warp * NSW * 32 + lane}, sum{total + lane};
+  // adds the shares of `count` warps, component by component
+  auto add_shares = [&](int count) {
+    for (int k = warp; k < NSW; k += W) {
+      R s = shares[k * 32 + lane];
+      for (int v = 1; v < count; ++v) s += shares[(v * NSW + k) * 32 + lane];
+      sum[k] = s;
     }
-    // reduce across the warp through the transpose buffer
+  };
+  {
+    R M[LV::NCOMP];
 #pragma unroll
-    for (int c = 0; c < C; ++c) tb[c * 33 + lane] = M[c];
-    __syncwarp();
-    for (int c = lane; c < C; c += 32) {
-      R s = R(0);
-#pragma unroll 8
-      for (int t = 0; t < 32; ++t) s += tb[c * 33 + t];
-      tb[c * 33 + 32] = s;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int c = 0; c < C; ++c) M[c] = tb[c * 33 + 32];
-    // contraction (every lane, the same values)
-    R D[C];
-    R Bv[DTHETA ? LV::NBASIS : 1];
-    R ei;
+    for (int c = 0; c < LV::NCOMP; ++c) M[c] = R(0);
+    moment_sweep<LV, R, DTHETA, -1, false, NQ>(a, sm, geom, a.cell, zi, beg, end, M);
+    LV::template store_swept<R>(M, mine);
+  }
+  __syncthreads();
+  add_shares(W);
+  __syncthreads();
+  const GraphColumn<R> G{graphs + lane};
+  for (int p = warp; p < NP; p += W) team_values<LV, R>(p, sum, G);
+  __syncthreads();
+  for (int p = warp; p < NP; p += W) {
+    const LaneColumn<R> share{shares + (size_t)p * NSW * 32 + lane};
+    R e;
     if constexpr (DTHETA)
-      ei = LV::template contract<R, true>(M, sm.xi, D, Bv);
+      e = team_adjoint<LV, R, true>(p, sum, G, sm.xi, share, WarpBasisSink<R>{sm.dxi, lane, active});
     else
-      ei = LV::template contract<R, true, const R*, DiscardBasisSink<R>>(
-          M, sm.xi, D, DiscardBasisSink<R>{sm.discard + warp, lane == 0});
-    if (lane == 0) {
-      e_i = a.species_energy[zi] + (double)ei;
-      a.e_atom[i] = e_i;
-      if (DTHETA) {
-        for (int t = 0; t < (DTHETA ? LV::NBASIS : 1); ++t) atomicAdd(sm.dxi + t, Bv[t]);
-        atomicAdd(sm.cnt + zi, 1);
-      }
-    }
-    // sweep 2: this lane's pairs
-    R fx = R(0), fy = R(0), fz = R(0);
-    constexpr int kAccS = 4;
-    const bool own_acc = DTHETA && sm.S <= kAccS;
-    R acc[DTHETA ? kAccS * NMU * kMaxQ : 1];
-    if (own_acc) {
-      for (int t = 0; t < sm.S * NMU * nq; ++t) acc[t] = R(0);
-    }
-    for (int64_t k = beg + lane; k < end; k += 32) {
-      const int32_t j = __ldg(a.nbr_j + k), img = __ldg(a.nbr_img + k);
-      const typename PairGeom<R>::Load lj = geom.fetch(a, j);
-      const int zj = lj.species;
-      R dx, dy, dz;
-      geom.vec(a, lj, img, dx, dy, dz);
-      const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-      const R rinv = rsqrt_r(r2);
-      const R r = r2 * rinv;
-      R f[NMU], df[NMU], q[DTHETA ? kMaxQ : 1];
-      radial<R, NMU, true, DTHETA, NQ>(cz + zj * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut, f, df, q);
-      R gx, gy, gz, Smu[NMU];
-      LV::template pair_adjoint<R>(D, f, df, dx * rinv, dy * rinv, dz * rinv, rinv, gx, gy, gz, Smu);
-      fx += gx;
-      fy += gy;
-      fz += gz;
-      scatter_force(a, j, -gx, -gy, -gz);
-      w[0] = fmadd(-gx, dx, w[0]);
-      w[1] = fmadd(-gy, dy, w[1]);
-      w[2] = fmadd(-gz, dz, w[2]);
-      w[3] = fmadd(R(-0.5), fmadd(gx, dy, gy * dx), w[3]);
-      w[4] = fmadd(R(-0.5), fmadd(gx, dz, gz * dx), w[4]);
-      w[5] = fmadd(R(-0.5), fmadd(gy, dz, gz * dy), w[5]);
-      if (DTHETA) {
-        if (own_acc) {
-          R* dst = acc + zj * NMU * nq;
-#pragma unroll
-          for (int mu = 0; mu < NMU; ++mu)
-#pragma unroll
-            for (int kk = 0; kk < kMaxQ; ++kk)
-              if (kk < nq) dst[mu * nq + kk] = fmadd(q[kk], Smu[mu], dst[mu * nq + kk]);
-        } else {
-          R* dst = sm.dc + (zi * sm.S + zj) * NMU * nq;
-#pragma unroll
-          for (int mu = 0; mu < NMU; ++mu)
-#pragma unroll
-            for (int kk = 0; kk < kMaxQ; ++kk)
-              if (kk < nq) atomicAdd(dst + mu * nq + kk, q[kk] * Smu[mu]);
+      e = team_adjoint<LV, R, false>(p, sum, G, sm.xi, share, (R*)nullptr);
+    energy[p * 32 + lane] = e;
+  }
+  __syncthreads();
+  add_shares(NP);
+  double e_i = 0.0;
+  if (warp == 0 && active) {
+    for (int p = 0; p < NP; ++p) e_i += (double)energy[p * 32 + lane];
+    e_i += a.species_energy[zi];
+    a.e_atom[i] = e_i;
+    if (DTHETA) atomicAdd(sm.cnt + zi, 1);
+  }
+  __syncthreads();
+  R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+  R fx = R(0), fy = R(0), fz = R(0);
+  // dE/dc of this thread's pairs, per neighbour species (as in efv_atom)
+  constexpr int kAccS = 4;
+  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccS * NMU * kMaxQ : 1];
+  const AccView<R> acc = (sizeof(R) == 4) ? AccView<R>{sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x}
+                                          : AccView<R>{acc_local, 1};
+  const bool own_acc = DTHETA && sm.S <= kAccS && acc.p != nullptr;
+  if (own_acc) {
+    for (int t = 0; t < sm.S * NMU * sm.nq; ++t) acc[t] = R(0);
+  }
+  {
+    R D[LV::NCOMP];
+    LV::template load_swept<R>(D, sum);
+    adjoint_sweep<LV, R, DTHETA, -1, false, NQ>(a, sm, geom, a.cell, zi, beg, end, D, fx, fy, fz, w, acc, own_acc);
+  }
+  force[(warp * 3 + 0) * 32 + lane] = fx;
+  force[(warp * 3 + 1) * 32 + lane] = fy;
+  force[(warp * 3 + 2) * 32 + lane] = fz;
+  __syncthreads();
+  if (own_acc) {
+    if constexpr (sizeof(R) == 4) {
+      // the warps' accumulators of one atom side by side: added, then one atomic per atom and entry
+      const int per = NMU * sm.nq;
+      if (active)
+        for (int t = warp; t < sm.S * per; t += W) {
+          R s = R(0);
+          for (int v = 0; v < W; ++v) s += sm.acc[t * (32 * W) + v * 32 + lane];
+          atomicAdd(sm.dc + (zi * sm.S + t / per) * per + t % per, s);
         }
-      }
-    }
-    if (own_acc) {
+    } else if (active) {
       for (int zj = 0; zj < sm.S; ++zj) {
         R* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
         for (int t = 0; t < NMU * sm.nq; ++t) atomicAdd(dst + t, acc[zj * NMU * sm.nq + t]);
       }
     }
-    fx = warp_sum_r(fx);
-    fy = warp_sum_r(fy);
-    fz = warp_sum_r(fz);
-    if (lane == 0) {
-      scatter_force(a, i, fx, fy, fz);
-      if (!isfinite(e_i) || !isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
-        flag_status(a.status, MTP_ERR_NONFINITE);
+  }
+  if (warp == 0 && active) {
+    for (int v = 1; v < W; ++v) {
+      fx += force[(v * 3 + 0) * 32 + lane];
+      fy += force[(v * 3 + 1) * 32 + lane];
+      fz += force[(v * 3 + 2) * 32 + lane];
     }
+    scatter_force(a, i, fx, fy, fz);
+    if (!isfinite(e_i) || !isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
+      flag_status(a.status, MTP_ERR_NONFINITE);
   }
   efv_block_flush<LV, R, DTHETA>(sm, e_i, w, a.e_total, a.virial, a.dtheta);
 }
 
 template <class LV, class R, bool DTHETA>
 int efv_team_launch_typed(const EfvArgs& a, cudaStream_t stream) {
-  if constexpr (LV::NGROUPS > 1) {
-    return efv_launch_typed<LV, R, DTHETA>(a, stream);   // the split kernels cut small systems into shares themselves
-  } else {
-    const int SS = a.n_species * a.n_species;
-    const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                         team_buf_bytes<R>(LV::NCOMP);
-    auto kern = efv_team_kernel<LV, R, DTHETA>;
-    if constexpr (std::is_same<R, float>::value) {
-      if (a.n_q == kFixedQ) kern = efv_team_kernel<LV, R, DTHETA, kFixedQ>;
-    }
-    int rc = set_smem(kern, bytes);
-    if (rc != MTP_OK) return rc;
-    const int64_t n = a.atom_end - a.atom_begin;
-    if (n <= 0) return MTP_OK;
-    const unsigned grid = (unsigned)((n + kTeamWarps - 1) / kTeamWarps);
-    kern<<<grid, kEfvThreads, bytes, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      set_error("warp-per-atom kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-    return MTP_OK;
+  const int SS = a.n_species * a.n_species;
+  const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
+                       efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, 32 * kTeamWarps) +
+                       team_buf_bytes<LV, R>(kTeamWarps);
+  if (bytes > 227 * 1024) return kTeamNoRoom;
+  auto kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, 0>;
+  if constexpr (std::is_same<R, float>::value) {
+    if (a.n_q == kFixedQ) kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, kFixedQ>;
   }
+  int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
+  const int64_t n = a.atom_end - a.atom_begin;
+  if (n <= 0) return MTP_OK;
+  kern<<<(unsigned)((n + 31) / 32), 32 * kTeamWarps, bytes, stream>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("team kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+    return MTP_ERR_CUDA;
+  }
+  return MTP_OK;
 }
 
 template <class LV>

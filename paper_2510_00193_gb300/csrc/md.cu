@@ -7,9 +7,13 @@
 // Fig. 3), and its examples run 1 fs MD (Sec. 3); the pair style receives a
 // neighbour list from the MD engine (Sec. 2.3).  Here one step is
 //   v += (dt/2) F/m;  x += dt v            (md_kick_drift_kernel)
-//   exact list of x from the skin list     (md_filter_kernel, scan, md_compact_kernel)
+//   exact rows of x from the skin list     (md_filter_kernel)
 //   F, E_pot = MTP(x)                      (the energy/force kernels)
 //   v += (dt/2) F/m;  E_kin = sum m v^2/2  (md_kick_kernel)
+// The energy/force kernels read the rows where the filter leaves them, at the
+// start of each atom's skin-list segment; only the last rows of a run are moved
+// to a contiguous list (scan, md_compact_kernel), which is what mtp_md_nlist
+// returns and the in-run grade reads.
 // The skin list holds every pair within R_cut + skin of the positions at its
 // last build; while no atom has moved more than skin/2 since then, it holds
 // every pair within R_cut now.  The filter decides each listed pair with the
@@ -50,8 +54,9 @@ struct MdFilterGeom {
 __global__ void md_kick_drift_kernel(double* __restrict__ x, double* __restrict__ v, const double* __restrict__ f,
                                      const int32_t* __restrict__ z, MdMass mm, double dt, int64_t n,
                                      const double* __restrict__ xref, double half_skin2, float4* __restrict__ xf,
-                                     int* __restrict__ flags) {
+                                     int* __restrict__ flags, double* __restrict__ e_kin) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && e_kin) *e_kin = 0.0;   // md_kick_kernel adds this step's
   if (i >= n) return;
   const double a = mm.inv_m[min(max(z[i], 0), kMaxSpecies - 1)] * 0.5 * dt;   // species checked by the force pass
   double p[3];
@@ -240,6 +245,9 @@ struct mtp_md {
   mtp::DevBuf xf;                   // FP32 positions and max |x| [N] float4
   mtp::DevBuf counts;               // int64 [N + 1] and the scan's temporary storage
   mtp::DevBuf tmp;                  // kept pairs at their skin-list positions: j, then image [2][P_skin]
+  bool compact = true;              // `exact` holds the kept pairs of the last filter pass
+  int* host_flag = nullptr;         // pinned copy of the displacement flag, and the event after the copy
+  cudaEvent_t flag_read = nullptr;
   size_t scan_bytes = 0;
   mtp::DevBuf e_atom, small;        // site energies [N]; virial [6], E_pot [1], flags [1]
   mtp::MdFilterGeom geom;
@@ -285,28 +293,59 @@ void md_set_cell(mtp_md* md, const double* cell) {
     for (int k = 0; k < 9; ++k) md->exact->cell[k] = cell[k];
 }
 
+// Exact rows of x at the start of the skin-list segments (md->tmp, counts).
 int md_filter(mtp_md* md, const double* x, cudaStream_t s) {
   using namespace mtp;
   const int64_t n = md->n_atoms;
   if (n == 0) return MTP_OK;
-  const int T = 256;   // 8 atoms (warps) per block; n + 1 warps for the filter pass
+  const int T = 256;   // 8 atoms (warps) per block; n + 1 warps
+  const unsigned blocks = (unsigned)((32 * (n + 1) + T - 1) / T);
+  mtp_nlist* sl = md->skin_list;
+  int32_t* tmp_j = md->tmp.as<int32_t>();
+  int32_t* tmp_img = tmp_j + std::max<int64_t>(sl->n_pairs, 1);
+  md_filter_kernel<<<blocks, T, 0, s>>>(x, md->xf.as<float4>(), n, md->geom, sl->offsets.as<int64_t>(),
+                                        sl->nbr_j.as<int32_t>(), sl->nbr_img.as<int32_t>(),
+                                        md->counts.as<int64_t>(), tmp_j, tmp_img);
+  MTP_TRY_CUDA(cudaGetLastError());
+  md->compact = false;
+  return MTP_OK;
+}
+
+// The rows of the last filter pass as the contiguous list md->exact.
+int md_compact(mtp_md* md, cudaStream_t s) {
+  using namespace mtp;
+  const int64_t n = md->n_atoms;
+  if (n == 0 || md->compact) return MTP_OK;
+  const int T = 256;
   const unsigned blocks = (unsigned)((32 * (n + 1) + T - 1) / T);
   int64_t* counts = md->counts.as<int64_t>();
   void* tmp = reinterpret_cast<char*>(md->counts.ptr) + ((sizeof(int64_t) * (n + 1) + 255) & ~size_t(255));
   mtp_nlist* sl = md->skin_list;
   mtp_nlist* ex = md->exact;
-  const int64_t cap = std::max<int64_t>(sl->n_pairs, 1);
   int32_t* tmp_j = md->tmp.as<int32_t>();
-  int32_t* tmp_img = tmp_j + cap;
-  md_filter_kernel<<<blocks, T, 0, s>>>(x, md->xf.as<float4>(), n, md->geom, sl->offsets.as<int64_t>(),
-                                        sl->nbr_j.as<int32_t>(), sl->nbr_img.as<int32_t>(), counts, tmp_j, tmp_img);
-  MTP_TRY_CUDA(cudaGetLastError());
+  int32_t* tmp_img = tmp_j + std::max<int64_t>(sl->n_pairs, 1);
   size_t tb = md->scan_bytes;
   MTP_TRY_CUDA(cub::DeviceScan::ExclusiveSum(tmp, tb, counts, ex->offsets.as<int64_t>(), (int)(n + 1), s));
   md_compact_kernel<<<blocks, T, 0, s>>>(n, sl->offsets.as<int64_t>(), ex->offsets.as<int64_t>(), tmp_j, tmp_img,
                                          ex->nbr_j.as<int32_t>(), ex->nbr_img.as<int32_t>());
   MTP_TRY_CUDA(cudaGetLastError());
+  md->compact = true;
   return MTP_OK;
+}
+
+// The rows of the last filter pass as a list for the energy/force kernels.
+mtp_nlist md_rows(const mtp_md* md) {
+  mtp_nlist v;
+  v.device = md->device;
+  v.n_atoms = md->n_atoms;
+  v.n_pairs = -1;
+  v.r_cut = md->r_cut;
+  v.offsets = md->skin_list->offsets;
+  v.row_counts = md->counts.as<int64_t>();
+  v.nbr_j = md->tmp;
+  v.nbr_img = md->tmp;
+  v.nbr_img.ptr = md->tmp.as<int32_t>() + std::max<int64_t>(md->skin_list->n_pairs, 1);
+  return v;
 }
 
 int md_read_flags(mtp_md* md, cudaStream_t s, int* flags) {
@@ -345,6 +384,23 @@ int md_rebuild(mtp_handle* h, mtp_md* md, const double* x, cudaStream_t s) {
   md->scale_since_build = 1.0;
   (void)h;
   return md_filter(md, x, s);
+}
+
+// The displacement flag of the last drift, read while the GPU goes on with
+// what is queued behind it: md_flag_queue copies it to pinned memory, and
+// md_flag_wait waits for that copy alone.
+int md_flag_queue(mtp_md* md, cudaStream_t s) {
+  if (!md->host_flag) MTP_TRY_CUDA(cudaHostAlloc((void**)&md->host_flag, sizeof(int), cudaHostAllocDefault));
+  if (!md->flag_read) MTP_TRY_CUDA(cudaEventCreateWithFlags(&md->flag_read, cudaEventDisableTiming));
+  int* dflags = reinterpret_cast<int*>(md->small.as<double>() + 7);
+  MTP_TRY_CUDA(cudaMemcpyAsync(md->host_flag, dflags, sizeof(int), cudaMemcpyDeviceToHost, s));
+  MTP_TRY_CUDA(cudaEventRecord(md->flag_read, s));
+  return MTP_OK;
+}
+int md_flag_wait(mtp_md* md, int* flags) {
+  MTP_TRY_CUDA(cudaEventSynchronize(md->flag_read));
+  *flags = *md->host_flag;
+  return MTP_OK;
 }
 
 }  // namespace
@@ -413,7 +469,7 @@ int mtp_md_create(mtp_handle* h, const double* x, int64_t n, const double* cell,
     mtp_md_free(md);
     return rc;
   }
-  if ((rc = md_rebuild(h, md, x, s)) != MTP_OK) {
+  if ((rc = md_rebuild(h, md, x, s)) != MTP_OK || (rc = md_compact(md, s)) != MTP_OK) {
     mtp_md_free(md);
     return rc;
   }
@@ -426,7 +482,8 @@ int mtp_md_rebuild(mtp_handle* h, mtp_md* md, const double* x, void* stream) {
     mtp::set_error("mtp_md_rebuild: invalid argument");
     return MTP_ERR_ARG;
   }
-  return md_rebuild(h, md, x, (cudaStream_t)stream);
+  const int rc = md_rebuild(h, md, x, (cudaStream_t)stream);
+  return rc != MTP_OK ? rc : md_compact(md, (cudaStream_t)stream);
 }
 
 int mtp_md_nlist(mtp_md* md, const mtp_nlist** nl, void* stream) {
@@ -464,9 +521,22 @@ int mtp_md_status(mtp_md* md, int64_t* steps_since_build, int64_t* rebuilds, voi
   return MTP_OK;
 }
 
+static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z, const double* mass,
+                        double dt, int32_t n_steps, int32_t rebuild_every, int32_t precision, double* forces,
+                        double* e_pot, double* e_kin, void* stream);
+
 int mtp_md_run(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z, const double* mass, double dt,
                int32_t n_steps, int32_t rebuild_every, int32_t precision, double* forces, double* e_pot,
                double* e_kin, void* stream) {
+  const int rc = md_run_steps(h, md, x, v, z, mass, dt, n_steps, rebuild_every, precision, forces, e_pot, e_kin, stream);
+  if (!md) return rc;
+  const int rc2 = md_compact(md, (cudaStream_t)stream);   // also after a run that stopped early
+  return rc != MTP_OK ? rc : rc2;
+}
+
+static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z, const double* mass,
+                        double dt, int32_t n_steps, int32_t rebuild_every, int32_t precision, double* forces,
+                        double* e_pot, double* e_kin, void* stream) {
   using namespace mtp;
   if (!h || !md || !mass || n_steps < 0 ||
       (md->n_atoms > 0 && (!x || !v || !z || !forces))) {
@@ -512,28 +582,31 @@ int mtp_md_run(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z
       if (flags) return mtp_md_status(md, nullptr, nullptr, stream);
       if ((rc = md_rebuild(h, md, x, s)) != MTP_OK) return rc;
     }
+    double* ep = e_pot ? e_pot + step : small + 6;
+    double* ek = e_kin ? e_kin + step : (npt ? small + 8 : nullptr);
+    auto evaluate = [&]() {
+      const mtp_nlist rows = md_rows(md);
+      return mtp_compute_efv(h, &rows, x, z, n, md->cell, precision, 0, md->e_atom.as<double>(), forces, small, ep,
+                             nullptr, stream);
+    };
     if (n > 0) {
       md_kick_drift_kernel<<<blocks, 256, 0, s>>>(x, v, forces, z, mm, dt, n, md->xref.as<double>(), half_skin2,
-                                                  md->xf.as<float4>(), dflags);
+                                                  md->xf.as<float4>(), dflags, ek);
       MTP_TRY_CUDA(cudaGetLastError());
+    } else if (ek) {
+      MTP_TRY_CUDA(cudaMemsetAsync(ek, 0, sizeof(double), s));
     }
-    bool rebuilt = false;
+    if (rebuild_every < 0 && (rc = md_flag_queue(md, s)) != MTP_OK) return rc;
+    if ((rc = md_filter(md, x, s)) != MTP_OK || (rc = evaluate()) != MTP_OK) return rc;
     if (rebuild_every < 0) {
-      // displacement check of this step's positions: rebuild before the list is used
+      // displacement check of this step's positions.  The evaluation is queued
+      // before the flag is known, so that the GPU does not wait for the host; in
+      // the rare step whose list may be incomplete it is done again (every
+      // output is overwritten) on a fresh list before anything uses it
       int flags = 0;
-      if ((rc = md_read_flags(md, s, &flags)) != MTP_OK) return rc;
-      if (flags) {
-        if ((rc = md_rebuild(h, md, x, s)) != MTP_OK) return rc;   // filters too
-        rebuilt = true;
-      }
+      if ((rc = md_flag_wait(md, &flags)) != MTP_OK) return rc;
+      if (flags && ((rc = md_rebuild(h, md, x, s)) != MTP_OK || (rc = evaluate()) != MTP_OK)) return rc;
     }
-    if (!rebuilt && (rc = md_filter(md, x, s)) != MTP_OK) return rc;
-    double* ep = e_pot ? e_pot + step : small + 6;
-    rc = mtp_compute_efv(h, md->exact, x, z, n, md->cell, precision, 0, md->e_atom.as<double>(), forces, small, ep,
-                         nullptr, stream);
-    if (rc != MTP_OK) return rc;
-    double* ek = e_kin ? e_kin + step : (npt ? small + 8 : nullptr);
-    if (ek) MTP_TRY_CUDA(cudaMemsetAsync(ek, 0, sizeof(double), s));
     if (n > 0) {
       md_kick_kernel<<<blocks, 256, 0, s>>>(v, forces, z, mm, dt, n, ek);
       MTP_TRY_CUDA(cudaGetLastError());
@@ -544,6 +617,7 @@ int mtp_md_run(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z
     if (graded && md->steps_total % md->grade_every == 0) {
       // extrapolation grade of this step's configuration (the positions and
       // exact list the forces were computed with), before any cell scaling
+      if ((rc = md_compact(md, s)) != MTP_OK) return rc;
       double gmax = 0.0;
       rc = mtp_compute_grade(h, md->exact, x, z, n, md->cell, md->a_inv, nullptr, md->tau_sel, md->tau_brk, 0,
                              md->grade_method, md->gamma.as<double>(), md->flags.as<uint8_t>(), &gmax, nullptr,
@@ -680,6 +754,8 @@ void mtp_md_free(mtp_md* md) {
   md->gamma.release();
   md->flags.release();
   md->sel_count.release();
+  if (md->host_flag) cudaFreeHost(md->host_flag);
+  if (md->flag_read) cudaEventDestroy(md->flag_read);
   delete md;
 }
 

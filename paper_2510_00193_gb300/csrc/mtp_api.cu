@@ -51,33 +51,67 @@ static const tables::LevelTable* find_table(int level) {
 int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cell, const int32_t* pbc, double r_cut,
                     cudaStream_t stream);
 
-// x (FP64) -> 32.32 fixed-point fractional coordinates s = x H^-1 (not
-// wrapped: the pair difference plus the image is then exact), species in slot 3.
-__global__ void fixed_point_kernel(const double* __restrict__ x, const int32_t* __restrict__ z, int64_t n,
-                                   double h0, double h1, double h2, double h3, double h4, double h5, double h6,
-                                   double h7, double h8, int S, long long* __restrict__ out, int* __restrict__ status) {
+template <bool MIXED>
+__global__ void efv_prep_kernel(const PrepArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-  const double s0 = px * h0 + py * h3 + pz * h6;
-  const double s1 = px * h1 + py * h4 + pz * h7;
-  const double s2 = px * h2 + py * h5 + pz * h8;
-  const double k = 4294967296.0;
-  const double lim = 2147483647.0;
-  const int zi = z[i];
-  const bool z_ok = zi >= 0 && zi < S;
-  if (!z_ok) atomicCAS(status, 0, MTP_ERR_ARG);
-  out[4 * i + 3] = z_ok ? (long long)zi : 0ll;   // out-of-range species read as 0 (reported above)
-  if (!(fabs(s0) < lim && fabs(s1) < lim && fabs(s2) < lim)) {
-    // non-finite (or absurdly far) position: reported, stored as the origin so
-    // that no kernel reads undefined coordinates
-    atomicCAS(status, 0, MTP_ERR_NONFINITE);
-    out[4 * i] = out[4 * i + 1] = out[4 * i + 2] = 0ll;
+  if (a.virial && i < 6) a.virial[i] = 0.0;
+  if (a.e_total && i == 6) *a.e_total = 0.0;   // blocks have more than 6 threads
+  if (a.dtheta)
+    for (int64_t k = i; k < a.n_params; k += (int64_t)gridDim.x * blockDim.x) a.dtheta[k] = 0.0;
+  if (i >= a.n) return;
+  const int zi = a.z[i];
+  const bool z_ok = zi >= 0 && zi < a.n_species;
+  if (!z_ok && a.status) atomicCAS(a.status, 0, MTP_ERR_ARG);
+  if constexpr (!MIXED) {
+    if (a.forces) a.forces[i] = a.forces[a.n + i] = a.forces[2 * a.n + i] = 0.0;
     return;
   }
-  out[4 * i] = __double2ll_rn(s0 * k);
-  out[4 * i + 1] = __double2ll_rn(s1 * k);
-  out[4 * i + 2] = __double2ll_rn(s2 * k);
+  if (a.forces_f) a.forces_f[i] = a.forces_f[a.n + i] = a.forces_f[2 * a.n + i] = 0.f;
+  const double px = a.x[3 * i], py = a.x[3 * i + 1], pz = a.x[3 * i + 2];
+  const double s0 = px * a.h[0] + py * a.h[3] + pz * a.h[6];
+  const double s1 = px * a.h[1] + py * a.h[4] + pz * a.h[7];
+  const double s2 = px * a.h[2] + py * a.h[5] + pz * a.h[8];
+  const double lim = 2147483647.0 * 4294967296.0;
+  longlong2 lo = make_longlong2(0ll, 0ll), hi = make_longlong2(0ll, z_ok ? (long long)zi : 0ll);
+  // out-of-range species are read as 0 (reported above); a non-finite (or
+  // absurdly far) position is reported and stored as the origin, so that no
+  // kernel reads undefined coordinates
+  if (fabs(s0) < lim && fabs(s1) < lim && fabs(s2) < lim) {
+    lo = make_longlong2(__double2ll_rn(s0), __double2ll_rn(s1));
+    hi.x = __double2ll_rn(s2);
+  } else {
+    atomicCAS(a.status, 0, MTP_ERR_NONFINITE);
+  }
+  longlong2* out = reinterpret_cast<longlong2*>(a.xq + 4 * i);
+  out[0] = lo;
+  out[1] = hi;
+}
+
+int launch_prep(const PrepArgs& a, bool mixed, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((a.n + 255) / 256);
+  if (mixed) efv_prep_kernel<true><<<blocks, 256, 0, s>>>(a);
+  else efv_prep_kernel<false><<<blocks, 256, 0, s>>>(a);
+  MTP_TRY_CUDA(cudaGetLastError());
+  return MTP_OK;
+}
+
+static double cell_det(const double* c) {
+  return c[0] * (c[4] * c[8] - c[5] * c[7]) - c[1] * (c[3] * c[8] - c[5] * c[6]) + c[2] * (c[3] * c[7] - c[4] * c[6]);
+}
+static bool cell_ok(const double* c) { return std::fabs(cell_det(c)) > 0.0; }
+// H^-1 of the cell rows, times `scale`.
+void inverse_rows(const double* c, double scale, double* hi) {
+  const double det = cell_det(c);
+  hi[0] = (c[4] * c[8] - c[5] * c[7]) / det;
+  hi[1] = (c[2] * c[7] - c[1] * c[8]) / det;
+  hi[2] = (c[1] * c[5] - c[2] * c[4]) / det;
+  hi[3] = (c[5] * c[6] - c[3] * c[8]) / det;
+  hi[4] = (c[0] * c[8] - c[2] * c[6]) / det;
+  hi[5] = (c[2] * c[3] - c[0] * c[5]) / det;
+  hi[6] = (c[3] * c[7] - c[4] * c[6]) / det;
+  hi[7] = (c[1] * c[6] - c[0] * c[7]) / det;
+  hi[8] = (c[0] * c[4] - c[1] * c[3]) / det;
+  for (int k = 0; k < 9; ++k) hi[k] *= scale;
 }
 
 // Mixed path: the FP32 force accumulator converted to the FP64 output.
@@ -86,18 +120,16 @@ __global__ void forces_to_fp64_kernel(const float* __restrict__ f, int64_t n3, d
   if (k < n3) out[k] = (double)f[k];
 }
 
-__global__ void species_check_kernel(const int32_t* __restrict__ z, int64_t n, int S, int* __restrict__ status) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && (z[i] < 0 || z[i] >= S)) atomicCAS(status, 0, MTP_ERR_ARG);
-}
-
 }  // namespace mtp
 
 using namespace mtp;
 
 namespace mtp {
-// Below this many atoms an untuned handle takes the warp-per-atom kernel.
-constexpr int64_t kTeamDefaultAtoms = 2048;
+// Up to this many atoms an untuned handle takes the team kernel: one wave of
+// its blocks (32 atoms, two blocks per SM).  On the mixed path with dE/dtheta
+// two waves: one thread per atom then carries the gradient accumulators too
+// (level 16: 144 against 193 us at 16,000 atoms, 809 against 687 at 128,000).
+static int64_t team_atoms(bool mixed, bool dtheta) { return 64 * (int64_t)device_sms() * (mixed && dtheta ? 2 : 1); }
 }  // namespace mtp
 
 extern "C" {
@@ -417,11 +449,12 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
     }
   }
   cudaStream_t s = (cudaStream_t)stream;
-  if (precision == MTP_FP64 || n == 0) MTP_TRY_CUDA(cudaMemsetAsync(forces, 0, sizeof(double) * 3 * (size_t)n, s));
-  MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6, s));
-  MTP_TRY_CUDA(cudaMemsetAsync(e_total, 0, sizeof(double), s));
-  if (dtheta) MTP_TRY_CUDA(cudaMemsetAsync(dtheta, 0, sizeof(double) * h->n_params, s));
-  if (n == 0) return MTP_OK;
+  if (n == 0) {
+    MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6, s));
+    MTP_TRY_CUDA(cudaMemsetAsync(e_total, 0, sizeof(double), s));
+    if (dtheta) MTP_TRY_CUDA(cudaMemsetAsync(dtheta, 0, sizeof(double) * h->n_params, s));
+    return MTP_OK;
+  }
 
   EfvArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -429,6 +462,7 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   a.offsets = nl->offsets.as<int64_t>();
   a.nbr_j = nl->nbr_j.as<int32_t>();
   a.nbr_img = nl->nbr_img.as<int32_t>();
+  a.row_counts = nl->row_counts;
   a.x = x;
   a.z = z;
   for (int k = 0; k < 9; ++k) {
@@ -452,36 +486,30 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   a.e_total = e_total;
   a.dtheta = dtheta;
   a.status = h->status.as<int>();
-  const unsigned blocks = (unsigned)((n + 255) / 256);
+  PrepArgs pa;
+  std::memset(&pa, 0, sizeof(pa));
+  pa.x = x;
+  pa.z = z;
+  pa.n = n;
+  pa.n_params = h->n_params;
+  pa.n_species = h->n_species;
+  pa.virial = virial;
+  pa.e_total = e_total;
+  pa.dtheta = dtheta;
+  pa.status = a.status;
   if (precision == MTP_MIXED) {
     int rc = h->xq.ensure(sizeof(long long) * 4 * (size_t)n);
     if (rc != MTP_OK) return rc;
-    double det = cell[0] * (cell[4] * cell[8] - cell[5] * cell[7]) - cell[1] * (cell[3] * cell[8] - cell[5] * cell[6]) +
-                 cell[2] * (cell[3] * cell[7] - cell[4] * cell[6]);
-    if (!(std::fabs(det) > 0.0)) {
-      set_error("mtp_compute_efv: singular cell");
-      return MTP_ERR_ARG;
-    }
-    double hi[9];
-    hi[0] = (cell[4] * cell[8] - cell[5] * cell[7]) / det;
-    hi[1] = (cell[2] * cell[7] - cell[1] * cell[8]) / det;
-    hi[2] = (cell[1] * cell[5] - cell[2] * cell[4]) / det;
-    hi[3] = (cell[5] * cell[6] - cell[3] * cell[8]) / det;
-    hi[4] = (cell[0] * cell[8] - cell[2] * cell[6]) / det;
-    hi[5] = (cell[2] * cell[3] - cell[0] * cell[5]) / det;
-    hi[6] = (cell[3] * cell[7] - cell[4] * cell[6]) / det;
-    hi[7] = (cell[1] * cell[6] - cell[0] * cell[7]) / det;
-    hi[8] = (cell[0] * cell[4] - cell[1] * cell[3]) / det;
-    fixed_point_kernel<<<blocks, 256, 0, s>>>(x, z, n, hi[0], hi[1], hi[2], hi[3], hi[4], hi[5], hi[6], hi[7], hi[8],
-                                              h->n_species, h->xq.as<long long>(), a.status);
-    MTP_TRY_CUDA(cudaGetLastError());
-    a.xq = h->xq.as<long long>();
     if ((rc = h->forces_f.ensure(sizeof(float) * 3 * (size_t)n)) != MTP_OK) return rc;
-    a.forces_f = h->forces_f.as<float>();
-    MTP_TRY_CUDA(cudaMemsetAsync(a.forces_f, 0, sizeof(float) * 3 * (size_t)n, s));
+    a.xq = pa.xq = h->xq.as<long long>();
+    a.forces_f = pa.forces_f = h->forces_f.as<float>();
+    inverse_rows(cell, 4294967296.0, pa.h);
   } else {
-    species_check_kernel<<<blocks, 256, 0, s>>>(z, n, h->n_species, a.status);
-    MTP_TRY_CUDA(cudaGetLastError());
+    pa.forces = forces;
+  }
+  {
+    const int rc = launch_prep(pa, precision == MTP_MIXED, s);
+    if (rc != MTP_OK) return rc;
   }
   const int64_t chunk = chunk_atoms > 0 ? chunk_atoms : n;
   // energy/force kernel: one thread per atom, or one warp per atom (small
@@ -491,7 +519,7 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   if (variant == 0) {
     const int bucket = std::min(63, (int)std::floor(std::log2((double)std::max<int64_t>(n, 1))));
     variant = h->tuned[precision == MTP_MIXED ? 1 : 0][bucket];
-    if (variant == 0) variant = n <= kTeamDefaultAtoms ? 2 : 1;
+    if (variant == 0) variant = n <= team_atoms(precision == MTP_MIXED, dtheta != nullptr) ? 2 : 1;
   }
   if (h->ops->split_comps > 0 && n > 0) {
     // moment/adjoint scratch of the split kernels (levels with component
@@ -602,6 +630,7 @@ static int fill_efv_args(mtp_handle* h, const mtp_nlist* nl, const double* x, co
   a.offsets = nl->offsets.as<int64_t>();
   a.nbr_j = nl->nbr_j.as<int32_t>();
   a.nbr_img = nl->nbr_img.as<int32_t>();
+  a.row_counts = nl->row_counts;
   a.x = x;
   a.z = z;
   for (int k = 0; k < 9; ++k) {
@@ -645,39 +674,42 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
     return MTP_ERR_UNSUPPORTED;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  MTP_TRY_CUDA(cudaMemsetAsync(dtheta_tan, 0, sizeof(double) * h->n_params, s));
-  if (force_tan) MTP_TRY_CUDA(cudaMemsetAsync(force_tan, 0, sizeof(double) * 3 * (size_t)n, s));
-  if (n == 0) return MTP_OK;
+  if (n == 0) {
+    MTP_TRY_CUDA(cudaMemsetAsync(dtheta_tan, 0, sizeof(double) * h->n_params, s));
+    return MTP_OK;
+  }
   TangentArgs t;
   std::memset(&t, 0, sizeof(t));
   fill_efv_args(h, nl, x, z, n, cell, t.base);
   t.v = v;
   t.dtheta_tan = dtheta_tan;
   t.force_tan = force_tan;
+  PrepArgs pa;
+  std::memset(&pa, 0, sizeof(pa));
+  pa.x = x;
+  pa.z = z;
+  pa.n = n;
+  pa.n_params = h->n_params;
+  pa.n_species = h->n_species;
+  pa.dtheta = dtheta_tan;
+  pa.status = t.base.status;
   if (precision == MTP_MIXED) {
     int rc = h->xq.ensure(sizeof(long long) * 4 * (size_t)n);
     if (rc != MTP_OK) return rc;
-    double det = cell[0] * (cell[4] * cell[8] - cell[5] * cell[7]) - cell[1] * (cell[3] * cell[8] - cell[5] * cell[6]) +
-                 cell[2] * (cell[3] * cell[7] - cell[4] * cell[6]);
-    if (!(std::fabs(det) > 0.0)) {
+    if (!cell_ok(cell)) {
       set_error("mtp_compute_efv_tangent: singular cell");
       return MTP_ERR_ARG;
     }
-    double hi[9];
-    hi[0] = (cell[4] * cell[8] - cell[5] * cell[7]) / det;
-    hi[1] = (cell[2] * cell[7] - cell[1] * cell[8]) / det;
-    hi[2] = (cell[1] * cell[5] - cell[2] * cell[4]) / det;
-    hi[3] = (cell[5] * cell[6] - cell[3] * cell[8]) / det;
-    hi[4] = (cell[0] * cell[8] - cell[2] * cell[6]) / det;
-    hi[5] = (cell[2] * cell[3] - cell[0] * cell[5]) / det;
-    hi[6] = (cell[3] * cell[7] - cell[4] * cell[6]) / det;
-    hi[7] = (cell[1] * cell[6] - cell[0] * cell[7]) / det;
-    hi[8] = (cell[0] * cell[4] - cell[1] * cell[3]) / det;
-    fixed_point_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, z, n, hi[0], hi[1], hi[2], hi[3], hi[4], hi[5],
-                                                                   hi[6], hi[7], hi[8], h->n_species,
-                                                                   h->xq.as<long long>(), t.base.status);
-    MTP_TRY_CUDA(cudaGetLastError());
-    t.base.xq = h->xq.as<long long>();
+    t.base.xq = pa.xq = h->xq.as<long long>();
+    inverse_rows(cell, 4294967296.0, pa.h);
+    if (force_tan) MTP_TRY_CUDA(cudaMemsetAsync(force_tan, 0, sizeof(double) * 3 * (size_t)n, s));
+  } else {
+    pa.forces = force_tan;
+    pa.status = nullptr;   // FP64 tangents read an out-of-range species as 0 without a report
+  }
+  {
+    const int rc = launch_prep(pa, precision == MTP_MIXED, s);
+    if (rc != MTP_OK) return rc;
   }
   t.base.atom_begin = 0;
   t.base.atom_end = n;

@@ -57,6 +57,7 @@ __device__ __forceinline__ int species_at(const int32_t* z, int64_t i, int S) {
 struct EfvArgs {
   int64_t atom_begin, atom_end, n_atoms;
   const int64_t* offsets;
+  const int64_t* row_counts;   // nullptr: row i is offsets[i] .. offsets[i + 1]; else offsets[i] .. + row_counts[i]
   const int32_t* nbr_j;
   const int32_t* nbr_img;
   const double* x;          // FP64 path
@@ -82,6 +83,37 @@ struct EfvArgs {
                             // n_parts buffers of partial moments, then the adjoints (nullptr: one fused kernel)
   int n_parts;              // shares into which the split kernels cut each atom's neighbours
 };
+
+// List row of atom i.
+__device__ __forceinline__ void list_row(const EfvArgs& a, int64_t i, int64_t& beg, int64_t& end) {
+  beg = __ldg(a.offsets + i);
+  end = a.row_counts ? beg + __ldg(a.row_counts + i) : __ldg(a.offsets + i + 1);
+}
+
+// Everything an evaluation needs before its own kernels, in one launch (a
+// call on a few hundred atoms is bound by launches: separate clears of the
+// energy, virial, gradient and force arrays cost more than its kernels):
+// the outputs that the kernels add to are cleared and every species index is
+// checked; MIXED: x (FP64) -> 32.32 fixed-point fractional coordinates
+// s = x H^-1 (not wrapped: the pair difference plus the image is then exact),
+// species in slot 3.
+struct PrepArgs {
+  const double* x;
+  const int32_t* z;
+  int64_t n, n_params;
+  double h[9];          // H^-1, MIXED: times 2^32 (exact)
+  int n_species;
+  long long* xq;        // MIXED
+  float* forces_f;      // MIXED, nullable
+  double* forces;       // FP64 path, nullable
+  double* virial;       // [6], nullable
+  double* e_total;      // nullable
+  double* dtheta;       // [n_params], nullable
+  int* status;
+};
+int launch_prep(const PrepArgs& a, bool mixed, cudaStream_t s);
+// H^-1 of the cell rows, times `scale`.
+void inverse_rows(const double* cell, double scale, double* hi);
 
 // Shares of each atom's neighbours in the split sweeps (levels with component
 // groups) of n atoms.  One thread per atom, component group and share: at 255
@@ -170,5 +202,6 @@ struct mtp_nlist {
   double cell[9] = {0};
   int pbc[3] = {0, 0, 0};
   mtp::DevBuf offsets, nbr_j, nbr_img;
+  const int64_t* row_counts = nullptr;   // entries of row i from offsets[i] on (nullptr: up to offsets[i + 1])
   mtp::DevBuf counts, bins, bin_start, bin_atoms, wrapped, columns, status;
 };
