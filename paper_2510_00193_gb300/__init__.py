@@ -28,16 +28,31 @@ def library_path() -> str:
     return _lib.LIB_PATH
 
 
+# Marshalling: small calls are bound by it (the interpreter code between two
+# launches runs from cold caches), so addresses travel as plain integers, the
+# raw stream handle is read without building a Stream object, and host arrays
+# of FP64 values pass as views of their own memory.
+
 def _stream_ptr(stream):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _dptr(t, dtype=None, n=None, name="array"):
-    import torch
     if t is None:
         return None
+    try:
+        if t.is_cuda and (dtype is None or t.dtype is dtype) and (n is None or t.numel() == n) and t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:
+        pass
+    return _dptr_error(t, dtype, n, name)
+
+
+def _dptr_error(t, dtype, n, name):
+    import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
     if dtype is not None and t.dtype != dtype:
@@ -46,7 +61,19 @@ def _dptr(t, dtype=None, n=None, name="array"):
         raise ValueError("%s must be contiguous" % name)
     if n is not None and t.numel() != n:
         raise ValueError("%s must have %d elements (got %d)" % (name, n, t.numel()))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_C_DOUBLE = ctypes.c_double
+_C_DOUBLE_P = ctypes.POINTER(ctypes.c_double)
+
+
+def _hptr(a):
+    """A contiguous FP64 host array as a ctypes argument (keeps the array's memory alive)."""
+    try:
+        return (_C_DOUBLE * a.size).from_buffer(a)
+    except (TypeError, ValueError, BufferError):   # a read-only array
+        return a.ctypes.data_as(_C_DOUBLE_P)
 
 
 def _host_d(a, n):
@@ -205,7 +232,7 @@ def mtp_build_neighbors(potential: Potential, x, cell, pbc=(1, 1, 1), nlist: Nei
     c = _host_d(cell, 9)
     p = np.ascontiguousarray(np.asarray(pbc, dtype=np.int32).reshape(3))
     check(_lib.load().mtp_build_neighbors(
-        potential.handle, _dptr(x, torch.float64, 3 * n, "x"), n, c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+        potential.handle, _dptr(x, torch.float64, 3 * n, "x"), n, _hptr(c),
         p.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), ctypes.byref(nl.handle), _stream_ptr(stream)))
     return nl
 
@@ -231,7 +258,7 @@ def mtp_compute_efv(potential: Potential, nlist: NeighborList, x, z, cell, preci
     c = _host_d(cell, 9)
     check(_lib.load().mtp_compute_efv(
         potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"), _dptr(z, torch.int32, n, "z"), n,
-        c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), int(precision), int(chunk_atoms),
+        _hptr(c), int(precision), int(chunk_atoms),
         _dptr(out["e_atom"], torch.float64, n, "e_atom"), _dptr(out["forces"], torch.float64, 3 * n, "forces"),
         _dptr(out["virial"], torch.float64, 6, "virial"), _dptr(out["e_total"], torch.float64, 1, "e_total"),
         _dptr(out["dtheta"], torch.float64, potential.n_params, "dtheta") if dtheta else None, _stream_ptr(stream)))
@@ -255,7 +282,7 @@ def mtp_efv_tune(potential: Potential, nlist: NeighborList, x, z, cell, precisio
     ch = ctypes.c_int32()
     ms = (ctypes.c_float * 2)()
     check(_lib.load().mtp_efv_tune(potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"),
-                                   _dptr(z, torch.int32, n, "z"), n, c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                   _dptr(z, torch.int32, n, "z"), n, _hptr(c),
                                    int(precision), ctypes.byref(ch), ms, _stream_ptr(stream)))
     return {"chosen": ch.value, "ms": [ms[0], ms[1]]}
 
@@ -270,7 +297,7 @@ def mtp_compute_efv_noalloc(potential: Potential, nlist: NeighborList, x, z, cel
     c = _host_d(cell, 9)
     check(_lib.load().mtp_compute_efv_noalloc(
         potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"), _dptr(z, torch.int32, n, "z"), n,
-        c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), int(chunk_atoms),
+        _hptr(c), int(chunk_atoms),
         _dptr(out["e_atom"], torch.float64, n, "e_atom"), _dptr(out["forces"], torch.float64, 3 * n, "forces"),
         _dptr(out["virial"], torch.float64, 6, "virial"), _dptr(out["e_total"], torch.float64, 1, "e_total"),
         _stream_ptr(stream)))
@@ -300,7 +327,7 @@ def mtp_compute_grade(potential: Potential, nlist: NeighborList, x, z, cell, a_i
     amb, rchk = ctypes.c_int64(), ctypes.c_int64()
     rc = check(_lib.load().mtp_compute_grade(
         potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"), _dptr(z, torch.int32, n, "z"), n,
-        c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+        _hptr(c),
         _dptr(a_inv, torch.float64, m * m, "a_inv") if a_inv is not None else None,
         _dptr(a_inv_cfg, torch.float64, m * m, "a_inv_cfg") if a_inv_cfg is not None else None,
         float(tau_sel), float(tau_brk), int(chunk_atoms), int(method),
@@ -365,7 +392,7 @@ class Batch:
         self._b = ctypes.c_void_p()
         self._pot = potential
         check(lib.mtp_batch_create(potential.handle, self.n_cfg, off.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)),
-                                   cl.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                   _hptr(cl),
                                    p.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)),
                                    _dptr(x, torch.float64, 3 * self.n_atoms, "x"), int(atoms_per_block),
                                    ctypes.byref(self._b), _stream_ptr(stream)))
@@ -452,7 +479,7 @@ def mtp_compute_efv_tangent(potential: Potential, nlist: NeighborList, x, z, cel
     c = _host_d(cell, 9)
     check(_lib.load().mtp_compute_efv_tangent(
         potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"), _dptr(z, torch.int32, n, "z"), n,
-        c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), int(precision), _dptr(v, torch.float64, 3 * n, "v"),
+        _hptr(c), int(precision), _dptr(v, torch.float64, 3 * n, "v"),
         _dptr(out["dtheta_tan"], torch.float64, potential.n_params, "dtheta_tan"),
         _dptr(out["force_tan"], torch.float64, 3 * n, "force_tan") if force_tan else None, _stream_ptr(stream)))
     return out
@@ -480,7 +507,7 @@ def mtp_compute_basis_rows(potential: Potential, nlist: NeighborList, x, z, cell
     c = _host_d(cell, 9)
     check(_lib.load().mtp_compute_basis_rows(
         potential.handle, nlist.handle, _dptr(x, torch.float64, 3 * n, "x"), _dptr(z, torch.int32, n, "z"), n,
-        c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _dptr(out, torch.float64, n * potential.m, "rows"),
+        _hptr(c), _dptr(out, torch.float64, n * potential.m, "rows"),
         _stream_ptr(stream)))
     return out
 
@@ -516,7 +543,7 @@ class MD:
         self._pot = potential
         self._md = ctypes.c_void_p()
         check(_lib.load().mtp_md_create(
-            potential.handle, _dptr(x, torch.float64, 3 * n, "x"), n, c.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+            potential.handle, _dptr(x, torch.float64, 3 * n, "x"), n, _hptr(c),
             p.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), float(skin), ctypes.byref(self._md), _stream_ptr(stream)))
 
     @property
@@ -565,7 +592,7 @@ class MD:
         m = _host_d(masses, self._pot.n_species)
         return check(_lib.load().mtp_md_run(
             self._pot.handle, self._md, _dptr(x, torch.float64, 3 * n, "x"), _dptr(v, torch.float64, 3 * n, "v"),
-            _dptr(z, torch.int32, n, "z"), m.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), float(dt), int(n_steps),
+            _dptr(z, torch.int32, n, "z"), _hptr(m), float(dt), int(n_steps),
             int(rebuild_every), int(precision), _dptr(forces, torch.float64, 3 * n, "forces"),
             _dptr(e_pot, torch.float64, n_steps, "e_pot") if e_pot is not None else None,
             _dptr(e_kin, torch.float64, n_steps, "e_kin") if e_kin is not None else None, _stream_ptr(stream)))
