@@ -1033,41 +1033,29 @@ def emit_contract_by_graph(lv: Level, fname="contract"):
     return L
 
 
-CONTRACT_PARTS = 4   # warps that share the contraction of one group of atoms
+class GraphCode:
+    """Straight-line code of single graphs: the forward values of their nodes
+    and the reverse pass into the swept moment components.  mload(c) is the
+    expression that reads swept component c."""
 
+    def __init__(self, lv, mload):
+        self.lv, self.mload = lv, mload
+        self.exp_order = sorted(lv.expand, key=lambda t: (lv.comps[t][1][2], t))
+        self.closures = [_node_closure(lv.dag, roots) for roots in lv.roots]
+        self.gbar = defaultdict(list)               # graph -> [(basis function, the other factors)]
+        for a, b in enumerate(lv.bases):
+            for j in range(len(b)):
+                self.gbar[b[j]].append((a, [b[t] for t in range(len(b)) if t != j]))
 
-def emit_contract_parts(lv: Level):
-    """The per-graph contraction cut into CONTRACT_PARTS parts for the warps of
-    a block that share the same atoms: part_values<P> forms the values of the
-    part's graphs, part_adjoint<P> (once every part's values are there) its
-    share of the basis values and of E, the adjoints of its graphs and its
-    contribution to D.  Swept moment components are read and D is returned by
-    their position k among the swept ones (M[k], D[k]); G(g) reads and
-    G.put(g, v) stores the value of graph g.  The graphs are dealt to the parts
-    by their operation counts, largest first."""
-    dag = lv.dag
-    ind = "    "
-    pos = {c: k for k, c in enumerate(lv.swept)}
-    exp_order = sorted(lv.expand, key=lambda t: (lv.comps[t][1][2], t))
+    def node_terms(self, n):
+        key, rank = self.lv.dag.nodes[n]
+        return n_sym(rank) * n_sym(self.lv.dag.rank(key[2])) if key[0] == "C" else 0
 
-    def node_ops(n):
-        key, rank = dag.nodes[n]
-        return 3 * n_sym(rank) * n_sym(dag.rank(key[2])) if key[0] == "C" else 0
-
-    closures = [_node_closure(dag, roots) for roots in lv.roots]
-    cost = [8 + sum(node_ops(n) for n in cl) for cl in closures]
-    parts = [[] for _ in range(CONTRACT_PARTS)]
-    for gi in sorted(range(len(cost)), key=lambda g: (-cost[g], g)):
-        min(parts, key=lambda q: (sum(cost[k] for k in q), len(q))).append(gi)
-    parts = [sorted(q) for q in parts]
-    bases = [[] for _ in range(CONTRACT_PARTS)]
-    for a in range(len(lv.bases)):
-        bases[a % CONTRACT_PARTS].append(a)
-
-    def used_comps(nodes):
-        used = set()
+    def comps(self, nodes, with_sources=True):
+        """Moment components that the nodes read (and the swept ones they are formed from)."""
+        lv, used = self.lv, set()
         for n in nodes:
-            key, rank = dag.nodes[n]
+            key, rank = lv.dag.nodes[n]
             if key[0] == "M":
                 _, mu, nu, off = key
                 for K in multi_indices(rank):
@@ -1080,18 +1068,20 @@ def emit_contract_parts(lv: Level):
                     stack.append(t)
         return used
 
-    def emit_forward(L, nodes, sfx, barrier):
-        """Moment components and C nodes of `nodes`; returns comp_ref and the weighted operands."""
-        used = used_comps(nodes)
+    def forward(self, L, nodes, sfx, barrier):
+        """Moment components and C nodes of `nodes`; returns comp_ref and the weighted operands.  With
+        `barrier` the components are read through opaque(), so that nothing is kept from another graph."""
+        lv, dag, ind = self.lv, self.lv.dag, "    "
+        used = self.comps(nodes)
 
         def mname(c):
             return ("mx%d%s" % (c, sfx)) if c in lv.expand else ("m%d%s" % (c, sfx))
 
         for c in sorted(t for t in used if t not in lv.expand):
-            L.append(ind + "R %s = M[%d];" % (mname(c), pos[c]))
+            L.append(ind + "R %s = %s;" % (mname(c), self.mload(c)))
             if barrier:
                 L.append(ind + "opaque(%s);" % mname(c))
-        for c in exp_order:
+        for c in self.exp_order:
             if c in used:
                 s0, s1, s2 = (mname(t) for t in lv.expand[c])
                 L.append(ind + "const R %s = (%s - %s) - %s;" % (mname(c), s0, s1, s2))
@@ -1124,10 +1114,108 @@ def emit_contract_parts(lv: Level):
                          [(comp_ref(a, tuple(K[d] + P[d] for d in range(3))), wname[n][j]) for j, P in enumerate(Ps)])
         return comp_ref, wname
 
-    gbar = defaultdict(list)
-    for a, b in enumerate(lv.bases):
-        for j in range(len(b)):
-            gbar[b[j]].append((a, [b[t] for t in range(len(b)) if t != j]))
+    def value(self, gi, cref):
+        return tree_sum([cref(n, (0, 0, 0)) if w == 1 else "R(%d) * %s" % (w, cref(n, (0, 0, 0)))
+                         for w, n in self.lv.roots[gi]])
+
+    def bar(self, gi):
+        """The graph's adjoint dE/dG from xi and the values G<k> of the other factors."""
+        return tree_sum(["R(xi[%d])" % a + "".join(" * G%d" % k for k in o) for a, o in self.gbar[gi]])
+
+    def fold(self, L, dpos, dneg, sfx):
+        """Adjoints of formed components go to the swept ones they came from, in decreasing z-exponent."""
+        lv = self.lv
+        for c in sorted(lv.expand, key=lambda t: (-lv.comps[t][1][2], -t)):
+            if not dpos.get(c) and not dneg.get(c):
+                continue
+            nm = "dx%d%s" % (c, sfx)
+            val = tree_sum(dpos[c]) if dpos.get(c) else "R(0)"
+            L.append("    const R %s = %s;" % (nm, val if not dneg.get(c) else "%s - %s" % (val, tree_sum(dneg[c]))))
+            s0, s1, s2 = lv.expand[c]
+            dpos[s0].append(nm)
+            dneg[s1].append(nm)
+            dneg[s2].append(nm)
+
+    def add(self, L, dpos, dneg, dname, comps):
+        for c in comps:
+            ex = dname(c)
+            if dpos.get(c):
+                ex = "%s + %s" % (ex, tree_sum(dpos[c]))
+            if dneg.get(c):
+                ex = "(%s) - %s" % (ex, tree_sum(dneg[c]))
+            L.append("    %s = %s;" % (dname(c), ex))
+
+    def reverse(self, L, gi, gbar_name, dname, fold=True):
+        """Forward values of graph gi again and its reverse pass: dname(c) += its share for the swept components
+        (without `fold` for every component it reads); returns the components it added to."""
+        lv, dag, ind = self.lv, self.lv.dag, "    "
+        sfx = "_g%d" % gi
+        nodes = self.closures[gi]
+        cref, wname = self.forward(L, nodes, sfx, True)
+        adj, dpos, dneg = defaultdict(list), defaultdict(list), defaultdict(list)
+        for w, node in lv.roots[gi]:
+            adj[(node, 0)].append(gbar_name if w == 1 else "R(%d) * %s" % (w, gbar_name))
+        for n in sorted(nodes, reverse=True):
+            key, rank = dag.nodes[n]
+            names = []
+            for ki in range(n_sym(rank)):
+                ex = adj.get((n, ki))
+                nm = "b%d_%d%s" % (n, ki, sfx) if ex else None
+                if ex:
+                    L.append(ind + "const R %s = %s;" % (nm, tree_sum(ex)))
+                names.append(nm)
+            if key[0] == "M":
+                _, mu, nu, off = key
+                for ki, K in enumerate(multi_indices(rank)):
+                    if names[ki]:
+                        dpos[lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))]].append(names[ki])
+                continue
+            _, a, b = key
+            Ps = multi_indices(dag.rank(b))
+            full_idx = multi_indices(dag.rank(a))
+            bacc = defaultdict(list)
+            for ki, K in enumerate(multi_indices(rank)):
+                if not names[ki]:
+                    continue
+                for j, P in enumerate(Ps):
+                    full = tuple(K[d] + P[d] for d in range(3))
+                    adj[(a, full_idx.index(full))].append("%s * %s" % (names[ki], wname[n][j]))
+                    bacc[j].append((names[ki], cref(a, full)))
+            for j, lst in bacc.items():
+                w = multinomial_weight(Ps[j])
+                nm = "c%d_%d%s" % (n, j, sfx)
+                emit_dot(L, ind, nm, lst)
+                adj[(b, j)].append(nm if w == 1 else "R(%d) * %s" % (w, nm))
+        if fold:
+            self.fold(L, dpos, dneg, sfx)
+        touched = sorted(c for c in set(dpos) | set(dneg) if not fold or c not in lv.expand)
+        self.add(L, dpos, dneg, dname, touched)
+        return touched
+
+
+CONTRACT_PARTS = 4   # warps that share the contraction of one group of atoms
+
+
+def emit_contract_parts(lv: Level):
+    """The per-graph contraction cut into CONTRACT_PARTS parts for the warps of
+    a block that share the same atoms: part_values<P> forms the values of the
+    part's graphs, part_adjoint<P> (once every part's values are there) its
+    share of the basis values and of E, the adjoints of its graphs and its
+    contribution to D.  Swept moment components are read and D is returned by
+    their position k among the swept ones (M[k], D[k]); G(g) reads and
+    G.put(g, v) stores the value of graph g.  The graphs are dealt to the parts
+    by their operation counts, largest first."""
+    ind = "    "
+    pos = {c: k for k, c in enumerate(lv.swept)}
+    gc = GraphCode(lv, lambda c: "M[%d]" % pos[c])
+    cost = [8 + 3 * sum(gc.node_terms(n) for n in cl) for cl in gc.closures]
+    parts = [[] for _ in range(CONTRACT_PARTS)]
+    for gi in sorted(range(len(cost)), key=lambda g: (-cost[g], g)):
+        min(parts, key=lambda q: (sum(cost[k] for k in q), len(q))).append(gi)
+    parts = [sorted(q) for q in parts]
+    bases = [[] for _ in range(CONTRACT_PARTS)]
+    for a in range(len(lv.bases)):
+        bases[a % CONTRACT_PARTS].append(a)
     out = ["  static constexpr int NPARTS = %d, NSWEPT = %d;" % (CONTRACT_PARTS, len(lv.swept))]
     for fn, args, body in (("store_swept", "const R* __restrict__ M, V dst", "dst[%d] = M[%d];"),
                            ("load_swept", "R* __restrict__ M, V src", "M[%d] = src[%d];")):
@@ -1142,18 +1230,17 @@ def emit_contract_parts(lv: Level):
     for q in range(CONTRACT_PARTS):
         L = ["  template <class R, class MV, class GV>",
              "  __device__ __forceinline__ static void part_values_%d(MV M, GV G) {" % q]
-        nodes = set().union(*[closures[g] for g in parts[q]]) if parts[q] else set()
-        cref, _ = emit_forward(L, nodes, "", False)
+        nodes = set().union(*[gc.closures[g] for g in parts[q]]) if parts[q] else set()
+        cref, _ = gc.forward(L, nodes, "", False)
         for gi in parts[q]:
-            terms = [cref(n, (0, 0, 0)) if w == 1 else "R(%d) * %s" % (w, cref(n, (0, 0, 0))) for w, n in lv.roots[gi]]
-            L.append(ind + "G.put(%d, %s);" % (gi, tree_sum(terms)))
+            L.append(ind + "G.put(%d, %s);" % (gi, gc.value(gi, cref)))
         L.append("  }")
         out += L
         L = ["  template <class R, bool WANT_B, class MV, class GV, class BV>",
              "  __device__ __forceinline__ static R part_adjoint_%d(MV M, GV G, const typename ScalarOf<R>::T* "
              "__restrict__ xi, R* __restrict__ D, BV B) {" % q,
              ind + "(void)B;"]
-        need = {k for a in bases[q] for k in lv.bases[a]} | {k for g in parts[q] for _, o in gbar[g] for k in o}
+        need = {k for a in bases[q] for k in lv.bases[a]} | {k for g in parts[q] for _, o in gc.gbar[g] for k in o}
         for k in sorted(need):
             L.append(ind + "const R G%d = G(%d);" % (k, k))
         L.append(ind + "R E = R(0);")
@@ -1162,70 +1249,110 @@ def emit_contract_parts(lv: Level):
             L.append(ind + "if (WANT_B) store_basis(B, %d, B%d);" % (a, a))
             L.append(ind + "E = fmadd(R(xi[%d]), B%d, E);" % (a, a))
         for gi in parts[q]:
-            L.append(ind + "const R Gb%d = %s;" % (gi, tree_sum(
-                ["R(xi[%d])" % a + "".join(" * G%d" % k for k in o) for a, o in gbar[gi]])))
+            L.append(ind + "const R Gb%d = %s;" % (gi, gc.bar(gi)))
         for k in range(len(lv.swept)):
             L.append(ind + "D[%d] = R(0);" % k)
         for gi in parts[q]:
-            sfx = "_g%d" % gi
-            nodes = closures[gi]
-            cref, wname = emit_forward(L, nodes, sfx, True)
-            adj, dpos, dneg = defaultdict(list), defaultdict(list), defaultdict(list)
-            for w, node in lv.roots[gi]:
-                adj[(node, 0)].append("Gb%d" % gi if w == 1 else "R(%d) * Gb%d" % (w, gi))
-            for n in sorted(nodes, reverse=True):
-                key, rank = dag.nodes[n]
-                names = []
-                for ki in range(n_sym(rank)):
-                    ex = adj.get((n, ki))
-                    nm = "b%d_%d%s" % (n, ki, sfx) if ex else None
-                    if ex:
-                        L.append(ind + "const R %s = %s;" % (nm, tree_sum(ex)))
-                    names.append(nm)
-                if key[0] == "M":
-                    _, mu, nu, off = key
-                    for ki, K in enumerate(multi_indices(rank)):
-                        if names[ki]:
-                            dpos[lv.comp_index[(mu, tuple(off[d] + K[d] for d in range(3)))]].append(names[ki])
-                    continue
-                _, a, b = key
-                Ps = multi_indices(dag.rank(b))
-                full_idx = multi_indices(dag.rank(a))
-                bacc = defaultdict(list)
-                for ki, K in enumerate(multi_indices(rank)):
-                    if not names[ki]:
-                        continue
-                    for j, P in enumerate(Ps):
-                        full = tuple(K[d] + P[d] for d in range(3))
-                        adj[(a, full_idx.index(full))].append("%s * %s" % (names[ki], wname[n][j]))
-                        bacc[j].append((names[ki], cref(a, full)))
-                for j, lst in bacc.items():
-                    w = multinomial_weight(Ps[j])
-                    nm = "c%d_%d%s" % (n, j, sfx)
-                    emit_dot(L, ind, nm, lst)
-                    adj[(b, j)].append(nm if w == 1 else "R(%d) * %s" % (w, nm))
-            for c in sorted(lv.expand, key=lambda t: (-lv.comps[t][1][2], -t)):
-                if not dpos.get(c) and not dneg.get(c):
-                    continue
-                nm = "dx%d%s" % (c, sfx)
-                val = tree_sum(dpos[c]) if dpos.get(c) else "R(0)"
-                L.append(ind + "const R %s = %s;" % (nm, val if not dneg.get(c) else "%s - %s" % (val, tree_sum(dneg[c]))))
-                s0, s1, s2 = lv.expand[c]
-                dpos[s0].append(nm)
-                dneg[s1].append(nm)
-                dneg[s2].append(nm)
-            for c in sorted(set(dpos) | set(dneg)):
-                if c in lv.expand:
-                    continue
-                ex = "D[%d]" % pos[c]
-                if dpos.get(c):
-                    ex = "%s + %s" % (ex, tree_sum(dpos[c]))
-                if dneg.get(c):
-                    ex = "(%s) - %s" % (ex, tree_sum(dneg[c]))
-                L.append(ind + "D[%d] = %s;" % (pos[c], ex))
+            gc.reverse(L, gi, "Gb%d" % gi, lambda c: "D[%d]" % pos[c])
         L += [ind + "return E;", "  }"]
         out += L
     return out
+
+
+GROUP_TERMS = 1500    # terms of a graph group's nodes: the group's reverse pass stays inside the instruction cache
+VALUE_TERMS = 3000    # the same for the forward passes
+
+
+def graph_groups(lv, gc, cap):
+    """Graphs in groups of at most `cap` node terms, each graph where most of its nodes are already."""
+    terms = [sum(gc.node_terms(n) for n in cl) for cl in gc.closures]
+    groups = []
+    for g in sorted(range(len(terms)), key=lambda g: (-terms[g], g)):
+        best = None
+        for q in groups:
+            add = sum(gc.node_terms(n) for n in gc.closures[g] - q[0])
+            if q[1] + add <= cap and (best is None or (terms[g] - add, q[1]) > best[0]):
+                best = ((terms[g] - add, q[1]), q, add)
+        if best is None:
+            groups.append([set(gc.closures[g]), terms[g], [g]])
+        else:
+            q = best[1]
+            q[0] |= gc.closures[g]
+            q[1] += best[2]
+            q[2].append(g)
+    return [sorted(q[2]) for q in groups]
+
+
+def emit_graph_groups(lv: Level):
+    """The contraction of a level with component groups as straight-line FP32 code, cut into groups of graphs that
+    are kernels of their own: values_<k> (graph values), products (basis values, E and graph adjoints) and
+    adjoint_<k> (each group's contribution to D).  M and D are one atom's columns (component c at c * ld), G and GB
+    the graph values and adjoints (graph g at g * gld)."""
+    ind = "    "
+    gc = GraphCode(lv, lambda c: "M[%d * ld]" % c)
+    vals = graph_groups(lv, gc, VALUE_TERMS)
+    adjs = graph_groups(lv, gc, GROUP_TERMS)
+    name = "MtpGraphs%d" % lv.level
+    out = ["// Generated by paper_2510_00193_gb300/basisgen.py for MTP level %d. Do not edit." % lv.level,
+           "#pragma once", "#include \"mtp_math.cuh\"", "namespace mtp {", "struct %s {" % name,
+           "  using R = float;",
+           "  static constexpr int VALUE_GROUPS = %d, ADJOINT_GROUPS = %d;" % (len(vals), len(adjs))]
+    for q, graphs in enumerate(vals):
+        L = ["  __device__ __forceinline__ static void values_%d(const R* __restrict__ M, int64_t ld, R* __restrict__ G, "
+             "int64_t gld) {" % q]
+        for gi in graphs:
+            cref, _ = gc.forward(L, gc.closures[gi], "_g%d" % gi, True)
+            L.append(ind + "G[%d * gld] = %s;" % (gi, gc.value(gi, cref)))
+        out += L + ["  }"]
+    L = ["  template <bool WANT_B, class BV>",
+         "  __device__ __forceinline__ static R products(const R* __restrict__ G, int64_t gld, const R* __restrict__ xi, "
+         "R* __restrict__ GB, BV B) {", ind + "(void)B;"]
+    for g in range(len(lv.graphs)):
+        L.append(ind + "const R G%d = G[%d * gld];" % (g, g))
+    # one basis function at a time: few partial sums, each a short chain
+    L.append(ind + "R E0 = R(0), E1 = R(0), E2 = R(0), E3 = R(0);")
+    for a, b in enumerate(lv.bases):
+        L.append(ind + "const R B%d = %s;" % (a, " * ".join("G%d" % k for k in b)))
+        L.append(ind + "if (WANT_B) store_basis(B, %d, B%d);" % (a, a))
+        L.append(ind + "E%d = fmadd(xi[%d], B%d, E%d);" % (a % 4, a, a, a % 4))
+    for g in range(len(lv.graphs)):
+        L.append(ind + "GB[%d * gld] = %s;" % (g, gc.bar(g)))
+    out += L + [ind + "return (E0 + E1) + (E2 + E3);", "  }"]
+    written = set()
+    for q, graphs in enumerate(adjs):
+        L = []
+        touched = set()
+        for gi in graphs:
+            L.append(ind + "const R gb%d = GB[%d * gld];" % (gi, gi))
+            touched |= set(gc.reverse(L, gi, "gb%d" % gi, lambda c: "d%d" % c, False))
+        # the formed components' adjoints fold into the swept ones once per group: they are sums of terms
+        # that partly cancel, and folding each graph's share by itself doubled the FP32 force error
+        dpos, dneg = defaultdict(list), defaultdict(list)
+        for c in touched:
+            if c in lv.expand:
+                dpos[c].append("d%d" % c)
+        gc.fold(L, dpos, dneg, "")
+        into = sorted(c for c in set(dpos) | set(dneg) if c not in lv.expand)
+        gc.add(L, dpos, dneg, lambda c: "d%d" % c, into)
+        touched |= set(into)
+        head = ["  __device__ __forceinline__ static void adjoint_%d(const R* __restrict__ M, int64_t ld, "
+                "const R* __restrict__ GB, int64_t gld, R* __restrict__ D) {" % q]
+        head += [ind + "R d%d = R(0);" % c for c in sorted(touched)]
+        # the first group that touches a component stores, the later ones add
+        out_c = sorted(c for c in touched if c not in lv.expand)
+        tail = [ind + ("D[%d * ld] = d%d;" if c not in written else "D[%d * ld] += d%d;") % (c, c) for c in out_c]
+        written |= set(out_c)
+        if q == len(adjs) - 1:
+            tail += [ind + "D[%d * ld] = R(0);" % c for c in lv.swept if c not in written]
+        out += head + L + tail + ["  }"]
+    for fn, args, call, n in (
+            ("values", "const R* M, int64_t ld, R* G, int64_t gld", "(M, ld, G, gld)", len(vals)),
+            ("adjoint", "const R* M, int64_t ld, const R* GB, int64_t gld, R* D", "(M, ld, GB, gld, D)", len(adjs))):
+        out += ["  template <int K>", "  __device__ __forceinline__ static void %s(%s) {" % (fn, args)]
+        out += [ind + "%sif constexpr (K == %d) %s_%d%s;" % ("" if k == 0 else "else ", k, fn, k, call) for k in range(n)]
+        out.append("  }")
+    out += ["};", "}  // namespace mtp"]
+    return "\n".join(out) + "\n"
 
 
 # Contraction code shape for the straight-line levels in FP32: the reverse
@@ -1635,6 +1762,10 @@ def generate(outdir, levels=LEVELS):
         path = os.path.join(outdir, "mtp_level%d.cuh" % lv.level)
         _write_if_changed(path, emit_header(lv))
         written.append(path)
+        if lv.level >= INTERPRET_FROM_LEVEL:
+            path = os.path.join(outdir, "mtp_graphs_level%d.cuh" % lv.level)
+            _write_if_changed(path, emit_graph_groups(lv))
+            written.append(path)
     path = os.path.join(outdir, "mtp_tables.h")
     _write_if_changed(path, emit_tables(lvs))
     written.append(path)

@@ -73,8 +73,16 @@ def generate_sources(levels=LEVELS):
             "int tangent_level%d(const TangentArgs& t, int precision, cudaStream_t s) {\n"
             "  return tangent_launch<MtpLevel%d>(t, precision, s);\n}\n"
             "int split_level%d() { return MtpLevel%d::NGROUPS > 1 ? MtpLevel%d::NCOMP : 0; }\n"
-            "}  // namespace mtp\n") % (L, L, L, L, L, L, L, L, L, L, L))
+            "int graphs_level%d() { return MtpLevel%d::NGROUPS > 1 ? MtpLevel%d::NGRAPH : 0; }\n"
+            "}  // namespace mtp\n") % (L, L, L, L, L, L, L, L, L, L, L, L, L, L))
         units.append(path)
+        if L >= basisgen.INTERPRET_FROM_LEVEL:
+            path = os.path.join(GEN, "graphs_level%d.cu" % L)
+            _write(path, head % ("efv_graphs.cuh", "#include \"mtp_graphs_level%d.cuh\"\n" % L) + (
+                "namespace mtp {\ntemplate <> int graphs_launch<%d>(const EfvArgs& a, bool want_dtheta, cudaStream_t s) {\n"
+                "  return graphs_launch_typed<MtpGraphs%d, MtpLevel%d>(a, want_dtheta, s);\n}\n}  // namespace mtp\n"
+                ) % (L, L, L))
+            units.append(path)
         path = os.path.join(GEN, "team_level%d.cu" % L)
         body = ("namespace mtp {\nint efv_level%d(const EfvArgs&, int, bool, cudaStream_t);\n"
                 "int team_level%d(const EfvArgs& a, int precision, bool want_dtheta, cudaStream_t s) {\n" % (L, L))
@@ -92,10 +100,11 @@ def generate_sources(levels=LEVELS):
                    "int batch_level%d(const BatchArgs&, int, bool, int, cudaStream_t);\n"
                    "int tangent_level%d(const TangentArgs&, int, cudaStream_t);\n"
                    "int split_level%d();\n"
+                   "int graphs_level%d();\n"
                    "int team_level%d(const EfvArgs&, int, bool, cudaStream_t);\n"
-                   % (L, L, L, L, L, L) for L in levels)
-    table = ",\n".join("  {%d, efv_level%d, rows_level%d, batch_level%d, tangent_level%d, split_level%d(), team_level%d}"
-                        % (L, L, L, L, L, L, L) for L in levels)
+                   % (L, L, L, L, L, L, L) for L in levels)
+    table = ",\n".join("  {%d, efv_level%d, rows_level%d, batch_level%d, tangent_level%d, split_level%d(), graphs_level%d(), team_level%d}"
+                        % (L, L, L, L, L, L, L, L) for L in levels)
     reg = os.path.join(GEN, "levels.cu")
     _write(reg, (
         "// Generated by paper_2510_00193_gb300/build.py.\n#include \"mtp_internal.cuh\"\nnamespace mtp {\n%s"

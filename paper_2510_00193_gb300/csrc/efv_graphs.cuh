@@ -1,0 +1,121 @@
+// Contraction of the levels with component groups (18 and 20) in FP32 for
+// large systems: one thread per atom, straight-line code.  The whole
+// contraction is far larger than the instruction cache (level 20: some 50,000
+// instructions), so it is cut into groups of graphs, each a kernel of its own
+// whose code fits: the values of the graphs, then the basis products with E
+// and the graph adjoints, then per group its graphs' nodes again and their
+// reverse pass.  Operands stay in registers, where the tile program
+// (tile_contract.cuh) reads each of its ~31,000 terms' operands from shared
+// memory; moments and the D accumulators pass between the kernels through
+// memory (about 12 KB per atom at level 20), and so do the graph values
+// (G[graph][atom]).
+//
+// Measured, level 20, 108,000 atoms, mixed: contraction 3.60 ms (tile program)
+// -> 0.59 ms (values 104, products 48, adjoints 435 us); the whole evaluation
+// 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays: at 2,016 atoms it
+// takes 0.11 ms, and these kernels would run on less than half a wave each.
+// Bound: instruction issue at 8 warps per SM (255 registers); the groups that
+// touch many components (281 of 295 in one) also wait for their D columns.
+#pragma once
+#include <utility>
+
+#include "efv_kernel.cuh"
+#include "tile_contract.cuh"
+
+namespace mtp {
+
+// Partial moments of the neighbour sweep's shares added into the first.
+template <class GR>
+__global__ void __launch_bounds__(256) sum_shares_kernel(float* __restrict__ mom, int64_t part, int n_parts) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= part) return;
+  float s = mom[k];
+  for (int p = 1; p < n_parts; ++p) s += mom[p * part + k];
+  mom[k] = s;
+}
+
+template <class GR, int NCOMP, int K>
+__global__ void __launch_bounds__(kEfvThreads) graph_values_kernel(const float* __restrict__ mom, int64_t n,
+                                                                   float* __restrict__ G, int64_t gld) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  GR::template values<K>(mom + tile_offset<float>(t, NCOMP), tile_atoms<float>(), G + t, gld);
+}
+
+template <class GR, class LV, bool DTHETA>
+__global__ void __launch_bounds__(kEfvThreads) graph_products_kernel(const EfvArgs a, const float* __restrict__ G,
+                                                                     float* __restrict__ GB, int64_t gld) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  EfvShared<float, LV::NMU, DTHETA> sm;
+  sm.setup(a, smem_raw);
+  sm.zero_gradients();
+  __syncthreads();
+  const int64_t n = a.atom_end - a.atom_begin;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool active = t < n;
+  double e_i = 0.0;
+  const float w[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // lanes without an atom run along on the first one (the basis values are summed across the warp)
+  const int64_t u = active ? t : 0;
+  if (__any_sync(0xffffffffu, active)) {
+    // the scratch has room for the padding atoms of the last block's warps: see split_scratch_bytes
+    const float e = GR::template products<DTHETA>(G + u, gld, sm.xi, GB + t,
+                                                  WarpBasisSink<float>{sm.dxi, (int)(threadIdx.x & 31), active});
+    if (active) {
+      const int64_t i = a.atom_begin + t;
+      const int zi = species_at(a.z, i, a.n_species);
+      e_i = a.species_energy[zi] + (double)e;
+      a.e_atom[i] = e_i;
+      if (!isfinite(e_i)) flag_status(a.status, MTP_ERR_NONFINITE);
+      if (DTHETA) atomicAdd(sm.cnt + zi, 1);
+    }
+  }
+  efv_block_flush<LV, float, DTHETA>(sm, e_i, w, a.e_total, a.virial, a.dtheta, kFlushEW | kFlushDxi);
+}
+
+template <class GR, int NCOMP, int K>
+__global__ void __launch_bounds__(kEfvThreads) graph_adjoint_kernel(const float* __restrict__ mom, int64_t n,
+                                                                    const float* __restrict__ GB, int64_t gld,
+                                                                    float* __restrict__ D) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int64_t at = tile_offset<float>(t, NCOMP);
+  GR::template adjoint<K>(mom + at, tile_atoms<float>(), GB + t, gld, D + at);
+}
+
+template <class GR, class LV, bool DTHETA, int... V, int... A>
+int graphs_launch_seq(const EfvArgs& a, cudaStream_t stream, std::integer_sequence<int, V...>,
+                      std::integer_sequence<int, A...>) {
+  const int64_t n = a.atom_end - a.atom_begin;
+  if (n <= 0) return MTP_OK;
+  const int64_t part = tile_padded(n) * LV::NCOMP, gld = graph_padded(n);
+  float* mom = static_cast<float*>(a.mbuf);
+  float* D = mom + part * a.n_parts;
+  float* G = D + part;
+  float* GB = G + gld * LV::NGRAPH;
+  const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
+  const size_t bytes = efv_smem_bytes<float, LV::NMU, DTHETA>(a.n_species * a.n_species, a.n_q, a.m);
+  int rc = set_smem(graph_products_kernel<GR, LV, DTHETA>, bytes);
+  if (rc != MTP_OK) return rc;
+  if (a.n_parts > 1)
+    sum_shares_kernel<GR><<<(unsigned)((part + 255) / 256), 256, 0, stream>>>(mom, part, a.n_parts);
+  (graph_values_kernel<GR, LV::NCOMP, V><<<grid, kEfvThreads, 0, stream>>>(mom, n, G, gld), ...);
+  graph_products_kernel<GR, LV, DTHETA><<<grid, kEfvThreads, bytes, stream>>>(a, G, GB, gld);
+  (graph_adjoint_kernel<GR, LV::NCOMP, A><<<grid, kEfvThreads, 0, stream>>>(mom, n, GB, gld, D), ...);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("graph kernels (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+    return MTP_ERR_CUDA;
+  }
+  return MTP_OK;
+}
+
+template <class GR, class LV>
+int graphs_launch_typed(const EfvArgs& a, bool want_dtheta, cudaStream_t stream) {
+  using Vs = std::make_integer_sequence<int, GR::VALUE_GROUPS>;
+  using As = std::make_integer_sequence<int, GR::ADJOINT_GROUPS>;
+  return want_dtheta ? graphs_launch_seq<GR, LV, true>(a, stream, Vs(), As())
+                     : graphs_launch_seq<GR, LV, false>(a, stream, Vs(), As());
+}
+
+}  // namespace mtp

@@ -494,7 +494,13 @@ struct EfvShared {
 
 // First neighbour sweep: M[c] += f_mu(r_ij) rhat^K for the components of
 // group G (G < 0: all components; G >= 0: the level's component group G).
-// CLOSE64 (mixed path only): pairs closer than R_min take close_pair_fp64.
+// CLOSE64 (mixed path only): pairs closer than R_min take close_pair_fp64, in
+// a second pass over the row.  Their terms are orders of magnitude larger than
+// the others (the radial functions are extrapolated there), so every term added
+// after one of them rounds at its size; added last, each costs one rounding.
+// (256,000 level-20 atoms, eight orientations of the box: force RMS error
+// 5.7e-5 eV/A; in list order 1.0e-4 with the straight-line contraction, 6.2e-5
+// with one thread per atom interpreting the program.)
 // Which sweeps are software-pipelined when DTHETA is set (without it both are).
 constexpr bool kPipeMomentsDtheta = true;
 constexpr bool kPipeAdjointDtheta = false;
@@ -569,26 +575,39 @@ __device__ __forceinline__ void moment_sweep(const EfvArgs& a, const EfvShared<R
     }
     return;
   }
-  while (ps.next(a, geom, j, img, lj)) {
-    R dx, dy, dz;
-    geom.vec(a, lj, img, dx, dy, dz);
-    const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-    R rinv = rsqrt_r(r2);
-    const R r = r2 * rinv;
-    R f[NMU];
-    if constexpr (CLOSE64 && std::is_same<R, float>::value) {
-      if (r < sm.rmin)
-        close_pair_fp64<NMU, false, false>(a, cell64, geom.ci, j, img, zi, lj.species, dx, dy,
-                                           dz, rinv, f, nullptr, nullptr);
-      else
-        radial<R, NMU, false, false, NQ>(sm.c + (zi * sm.S + lj.species) * sm.cstride, sm.nq, r, sm.mid,
-                                         sm.scale, sm.rcut, f, nullptr, nullptr);
-    } else {
-      radial<R, NMU, false, false, NQ>(sm.c + (zi * sm.S + lj.species) * sm.cstride, sm.nq, r, sm.mid, sm.scale,
-                                       sm.rcut, f, nullptr, nullptr);
+  constexpr bool kClose = CLOSE64 && std::is_same<R, float>::value;
+  int64_t first = end, last = beg;   // the row's entries from its first to its last pair below R_min
+  for (bool second = false;; second = true, ps.start(a, geom, first, last)) {
+    while (ps.next(a, geom, j, img, lj)) {
+      R dx, dy, dz;
+      geom.vec(a, lj, img, dx, dy, dz);
+      const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
+      R rinv = rsqrt_r(r2);
+      const R r = r2 * rinv;
+      if constexpr (kClose) {
+        const bool close = r < sm.rmin;
+        if (close && !second) {
+          first = min(first, ps.k - 1);
+          last = ps.k;
+        }
+        if (close != second) continue;
+      }
+      R f[NMU];
+      if constexpr (CLOSE64 && std::is_same<R, float>::value) {
+        if (r < sm.rmin)
+          close_pair_fp64<NMU, false, false>(a, cell64, geom.ci, j, img, zi, lj.species, dx, dy,
+                                             dz, rinv, f, nullptr, nullptr);
+        else
+          radial<R, NMU, false, false, NQ>(sm.c + (zi * sm.S + lj.species) * sm.cstride, sm.nq, r, sm.mid,
+                                           sm.scale, sm.rcut, f, nullptr, nullptr);
+      } else {
+        radial<R, NMU, false, false, NQ>(sm.c + (zi * sm.S + lj.species) * sm.cstride, sm.nq, r, sm.mid, sm.scale,
+                                         sm.rcut, f, nullptr, nullptr);
+      }
+      if constexpr (G < 0) LV::template moments<R>(M, f, dx * rinv, dy * rinv, dz * rinv);
+      else LV::template moments_group<G, R>(M, f, dx * rinv, dy * rinv, dz * rinv);
     }
-    if constexpr (G < 0) LV::template moments<R>(M, f, dx * rinv, dy * rinv, dz * rinv);
-    else LV::template moments_group<G, R>(M, f, dx * rinv, dy * rinv, dz * rinv);
+    if (!kClose || second || first >= last) break;
   }
 }
 
@@ -679,25 +698,38 @@ __device__ __forceinline__ void adjoint_sweep(const EfvArgs& a, const EfvShared<
     }
     return;
   }
-  while (ps.next(a, geom, j, img, lj)) {
-    const int zj = lj.species;
-    R dx, dy, dz;
-    geom.vec(a, lj, img, dx, dy, dz);
-    const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
-    R rinv = rsqrt_r(r2);
-    const R r = r2 * rinv;
-    R f[NMU], df[NMU], q[DTHETA ? kMaxQ : 1];
-    if constexpr (std::is_same<R, float>::value) {
-      if (r < sm.rmin)
-        close_pair_fp64<NMU, true, DTHETA>(a, cell64, geom.ci, j, img, zi, zj, dx, dy, dz, rinv, f, df, q);
-      else
-        radial<R, NMU, true, DTHETA, NQ>(sm.c + (zi * sm.S + zj) * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut,
-                                         f, df, q);
-    } else {
-      radial<R, NMU, true, DTHETA, NQ>(sm.c + (zi * sm.S + zj) * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut, f,
-                                       df, q);
+  constexpr bool kClose = CLOSE64 && std::is_same<R, float>::value;
+  int64_t first = end, last = beg;   // as in moment_sweep
+  for (bool second = false;; second = true, ps.start(a, geom, first, last)) {
+    while (ps.next(a, geom, j, img, lj)) {
+      const int zj = lj.species;
+      R dx, dy, dz;
+      geom.vec(a, lj, img, dx, dy, dz);
+      const R r2 = fmadd(dz, dz, fmadd(dy, dy, dx * dx));
+      R rinv = rsqrt_r(r2);
+      const R r = r2 * rinv;
+      if constexpr (kClose) {
+        const bool close = r < sm.rmin;
+        if (close && !second) {
+          first = min(first, ps.k - 1);
+          last = ps.k;
+        }
+        if (close != second) continue;
+      }
+      R f[NMU], df[NMU], q[DTHETA ? kMaxQ : 1];
+      if constexpr (std::is_same<R, float>::value) {
+        if (r < sm.rmin)
+          close_pair_fp64<NMU, true, DTHETA>(a, cell64, geom.ci, j, img, zi, zj, dx, dy, dz, rinv, f, df, q);
+        else
+          radial<R, NMU, true, DTHETA, NQ>(sm.c + (zi * sm.S + zj) * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut,
+                                           f, df, q);
+      } else {
+        radial<R, NMU, true, DTHETA, NQ>(sm.c + (zi * sm.S + zj) * sm.cstride, sm.nq, r, sm.mid, sm.scale, sm.rcut, f,
+                                         df, q);
+      }
+      adjoint_pair<LV, R, DTHETA, G, NQ>(a, sm, zi, j, zj, dx, dy, dz, rinv, f, df, q, D, fx, fy, fz, w, acc, own_acc);
     }
-    adjoint_pair<LV, R, DTHETA, G, NQ>(a, sm, zi, j, zj, dx, dy, dz, rinv, f, df, q, D, fx, fy, fz, w, acc, own_acc);
+    if (!kClose || second || first >= last) break;
   }
 }
 

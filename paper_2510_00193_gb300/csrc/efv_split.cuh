@@ -143,7 +143,14 @@ int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
   if ((rc = set_smem(split_moments_kernel<LV, R>, b0)) != MTP_OK) return rc;
   if ((rc = set_smem(split_adjoint_kernel<LV, R, DTHETA>, b1)) != MTP_OK) return rc;
   split_moments_kernel<LV, R><<<grid, kEfvThreads, b0, stream>>>(a);
-  if ((rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream)) != MTP_OK) return rc;
+  if constexpr (std::is_same<R, float>::value) {
+    // the scratch of a chunked call is sized for its first, largest range
+    if (n >= kGraphAtoms) rc = graphs_launch<LV::LEVEL>(a, DTHETA, stream);
+    else rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream);
+  } else {
+    rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream);
+  }
+  if (rc != MTP_OK) return rc;
   split_adjoint_kernel<LV, R, DTHETA><<<grid, kEfvThreads, b1, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -527,7 +527,8 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
     const int64_t range = std::min<int64_t>(chunk, n);
     a.n_parts = split_parts(range, device_sms());
     int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, range, a.n_parts,
-                                                precision == MTP_MIXED ? sizeof(float) : sizeof(double)));
+                                                precision == MTP_MIXED ? sizeof(float) : sizeof(double),
+                                                precision == MTP_MIXED && range >= kGraphAtoms ? h->ops->split_graphs : 0));
     if (rc != MTP_OK) return rc;
     a.mbuf = h->mbuf.ptr;
   }
@@ -717,7 +718,7 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
     // dual moments and adjoints of the split tangent kernels: (value, tangent) pairs
     t.base.n_parts = split_parts(n, device_sms());
     int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, n, t.base.n_parts,
-                                                2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double))));
+                                                2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double)), 0));
     if (rc != MTP_OK) return rc;
     t.base.mbuf = h->mbuf.ptr;
   }

@@ -136,10 +136,20 @@ inline int split_parts(int64_t n, int sms) {
   while (parts < kSplitMaxParts && 2 * parts * blocks <= 2 * (int64_t)sms) parts *= 2;
   return parts;
 }
-// Bytes of EfvArgs::mbuf for n atoms: atoms rounded up to whole tiles of 8.
-inline size_t split_scratch_bytes(int comps, int64_t n, int parts, size_t entry) {
-  return entry * (size_t)comps * (size_t)((n + 7) / 8 * 8) * (size_t)(parts + 1);
+// Row length of the graph values G[graph][atom]: whole blocks of 128 threads.
+__host__ __device__ inline int64_t graph_padded(int64_t n) { return (n + 127) / 128 * 128; }
+// Bytes of EfvArgs::mbuf for n atoms: the shares' moments and the adjoints, with
+// the atoms rounded up to whole tiles of 8, then the values and adjoints of the
+// graphs (the straight-line contraction; graphs = 0 without it).
+inline size_t split_scratch_bytes(int comps, int64_t n, int parts, size_t entry, int graphs) {
+  return entry * ((size_t)comps * (size_t)((n + 7) / 8 * 8) * (size_t)(parts + 1) +
+                  2 * (size_t)graphs * (size_t)graph_padded(n));
 }
+// From this many atoms of a range on, the mixed path of the levels with
+// component groups contracts with the straight-line graph kernels.
+constexpr int64_t kGraphAtoms = 4096;
+// The straight-line contraction of level LEVEL (generated).
+template <int LEVEL> int graphs_launch(const EfvArgs& a, bool want_dtheta, cudaStream_t s);
 
 using EfvLaunch = int (*)(const EfvArgs&, int precision, bool want_dtheta, cudaStream_t);
 // FP64 basis rows of listed atoms (list == nullptr: atoms atom_begin..), optional FP64 column sums.
@@ -158,6 +168,7 @@ struct LevelEntry {
   BatchLaunch batch;
   TangentLaunch tangent;
   int split_comps;   // components per atom of the EfvArgs::mbuf scratch (0: the level needs none)
+  int split_graphs;  // graphs per atom of that scratch (0: the level needs none)
   EfvLaunch team;    // warp-per-atom energy/force kernel (levels with component groups: the split kernels)
 };
 

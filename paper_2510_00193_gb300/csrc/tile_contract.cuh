@@ -12,9 +12,9 @@
 //
 // Measured (whole evaluation, FCC level 20, against one thread per atom
 // interpreting the program on local-memory arrays, or one warp per atom with
-// shared-memory atomics for small systems): 108,000 atoms mixed 10.5 -> 4.4 ms,
-// 2,016 atoms mixed 2.38 -> 0.154 ms, one FP64 force-matching step of 4,000
-// atoms 41.3 -> 6.6 ms.
+// shared-memory atomics for small systems): 2,016 atoms mixed 2.38 -> 0.140 ms,
+// 108,000 atoms mixed 10.4 -> 4.2 ms (there the graph kernels of efv_graphs.cuh
+// now take 1.41), one FP64 force-matching step of 4,000 atoms 41.3 -> 6.5 ms.
 //
 // Bound: shared-memory bandwidth on the FP32 path (two 16-byte reads per term
 // and thread; the four rows that a quarter warp reads lie in random bank
