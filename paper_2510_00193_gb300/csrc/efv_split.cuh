@@ -70,11 +70,9 @@ __device__ __forceinline__ void split_adjoint(const EfvArgs& a, const EfvShared<
   geom.load_centre(a, s.i, cell_of<R>(a));
   const int zi = species_at(a.z, s.i, a.n_species);
   R fx = R(0), fy = R(0), fz = R(0);
-  constexpr int kAccS = 4;
-  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccS * NMU * kMaxQ : 1];
-  const AccView<R> acc = (sizeof(R) == 4) ? AccView<R>{sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x}
-                                          : AccView<R>{acc_local, 1};
-  const bool own_acc = DTHETA && sm.S <= kAccS && acc.p != nullptr;
+  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccSpecies * NMU * kMaxQ : 1];
+  const AccView<R> acc = own_accumulators<R, 0>(sm.acc, acc_local);
+  const bool own_acc = DTHETA && sm.S <= kAccSpecies && acc.p != nullptr;
   if (own_acc) {
     for (int u = 0; u < sm.S * NMU * sm.nq; ++u) acc[u] = R(0);
   }
@@ -82,14 +80,10 @@ __device__ __forceinline__ void split_adjoint(const EfvArgs& a, const EfvShared<
   const R* buf = static_cast<const R*>(a.mbuf) + (int64_t)a.n_parts * (tile_padded(n) * LV::NCOMP);
   LV::template load_group<G, R>(buf + tile_offset<R>(s.active ? s.t : 0, LV::NCOMP), tile_atoms<R>(), Dg);
   adjoint_sweep<LV, R, DTHETA, G, true>(a, sm, geom, a.cell, zi, s.beg, s.end, Dg, fx, fy, fz, w, acc, own_acc);
+  if (own_acc)
+    add_warp_gradients(sm, LV::GROUP_MU_LO[G] * sm.nq, LV::GROUP_MU_HI[G] * sm.nq, zi, s.active,
+                       [&](int t) { return acc[t]; });
   if (!s.active) return;
-  if (own_acc) {
-    constexpr int lo = LV::GROUP_MU_LO[G], hi = LV::GROUP_MU_HI[G];
-    for (int zj = 0; zj < sm.S; ++zj) {
-      R* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-      for (int u = lo * sm.nq; u < hi * sm.nq; ++u) atomicAdd(dst + u, acc[zj * NMU * sm.nq + u]);
-    }
-  }
   scatter_force(a, s.i, fx, fy, fz);
   if (!isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
     flag_status(a.status, MTP_ERR_NONFINITE);
@@ -134,15 +128,16 @@ int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
   const int SS = a.n_species * a.n_species;
   const int64_t n = a.atom_end - a.atom_begin;
   if (n <= 0) return MTP_OK;
-  // every thread of the last block that pads a tile must exist: 128 is a multiple of the tile's atoms
-  const dim3 grid((unsigned)((n + kEfvThreads - 1) / kEfvThreads), 2 * a.n_parts);
+  // every thread of the last block that pads a tile must exist: a block's threads are whole tiles
+  const int threads = sizeof(R) == 8 ? fp64_threads(n, 2 * a.n_parts) : kEfvThreads;
+  const dim3 grid((unsigned)((n + threads - 1) / threads), 2 * a.n_parts);
   const size_t b0 = efv_smem_bytes<R, LV::NMU, false>(SS, a.n_q, a.m);
-  const size_t b1 = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                    efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvThreads);
+  const size_t base = (efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15);
+  const size_t b1 = base + efv_acc_bytes<R, LV::NMU, DTHETA>(base, a.n_species, a.n_q, threads);
   int rc;
   if ((rc = set_smem(split_moments_kernel<LV, R>, b0)) != MTP_OK) return rc;
   if ((rc = set_smem(split_adjoint_kernel<LV, R, DTHETA>, b1)) != MTP_OK) return rc;
-  split_moments_kernel<LV, R><<<grid, kEfvThreads, b0, stream>>>(a);
+  split_moments_kernel<LV, R><<<grid, threads, b0, stream>>>(a);
   if constexpr (std::is_same<R, float>::value) {
     // the scratch of a chunked call is sized for its first, largest range
     if (n >= kGraphAtoms) rc = graphs_launch<LV::LEVEL>(a, DTHETA, stream);
@@ -151,7 +146,7 @@ int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
     rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream);
   }
   if (rc != MTP_OK) return rc;
-  split_adjoint_kernel<LV, R, DTHETA><<<grid, kEfvThreads, b1, stream>>>(a);
+  split_adjoint_kernel<LV, R, DTHETA><<<grid, threads, b1, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("efv split kernels (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
@@ -166,12 +161,17 @@ int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
     if (a.mbuf) return efv_split_launch<LV, R, DTHETA>(a, stream);
   }
   const int SS = a.n_species * a.n_species;
-  const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                       efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, kEfvFusedThreads);
+  const int64_t n = a.atom_end - a.atom_begin;
+  if (n <= 0) return MTP_OK;
+  const int threads = sizeof(R) == 8 ? fp64_threads(n, 1) : kEfvFusedThreads;
+  const size_t base = (efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15);
+  const size_t bytes = base + efv_acc_bytes<R, LV::NMU, DTHETA>(base, a.n_species, a.n_q, threads);
   auto kern = efv_kernel<LV, R, DTHETA>;
-  // the mixed path of the single-group levels with the common radial basis
-  // size n_q = 8 runs with n_q fixed at compile time
-  if constexpr (std::is_same<R, float>::value && LV::NGROUPS == 1) {
+  // the single-group levels with the common radial basis size n_q = 8 run with
+  // n_q fixed at compile time on the mixed path and with dE/dtheta (FP64, 48,546
+  // atoms: 3.5 -> 2.9 ms; loops up to kMaxQ predicate FP64 operations away that
+  // still take their turn in the pipe)
+  if constexpr ((std::is_same<R, float>::value || DTHETA) && LV::NGROUPS == 1) {
     if (a.n_q == kFixedQ) kern = efv_kernel<LV, R, DTHETA, kFixedQ>;
   }
   if (bytes > 48 * 1024) {
@@ -181,10 +181,7 @@ int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
       return MTP_ERR_CUDA;
     }
   }
-  const int64_t n = a.atom_end - a.atom_begin;
-  if (n <= 0) return MTP_OK;
-  const unsigned grid = (unsigned)((n + kEfvFusedThreads - 1) / kEfvFusedThreads);
-  kern<<<grid, kEfvFusedThreads, bytes, stream>>>(a);
+  kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("efv kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));

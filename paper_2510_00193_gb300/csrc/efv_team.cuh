@@ -18,9 +18,9 @@
 // above that the instruction streams of four different contraction parts on an
 // SM cost more than the idle lanes of one thread per atom.  Level 16, mixed
 // energies and forces, this kernel / one thread per atom (whole call, us):
-// 2,000 atoms 39 / 60, 8,192 45 / 57, 16,000 74 / 57; with dE/dtheta 73 / 190,
-// 79 / 191, 144 / 193; FP64 2,000 atoms 284 / 939, 16,000 1,089 / 963.  The
-// form before (one warp per atom, every lane running the whole contraction)
+// 2,000 atoms 39 / 60, 8,192 45 / 57, 16,000 74 / 57; with dE/dtheta 2,000 atoms
+// 49 / 108, 16,000 171 / 111; FP64 2,000 atoms 278 / 879, 16,000 1,081 / 953.
+// The form before (one warp per atom, every lane running the whole contraction)
 // took 59 us at 2,000 atoms.  Bound: instruction fetch (ncu: 3.1 of 6.5 stalled
 // warps per issue wait for instructions at 2,000 atoms).
 // Levels with component groups (18 and 20) run the split kernels at every size.
@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   const int SS = a.n_species * a.n_species;
   constexpr int SHARES = W > NP ? W : NP;
   R* shares = reinterpret_cast<R*>(smem_raw + ((efv_smem_bytes<R, NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                                   efv_acc_bytes<R, NMU, DTHETA>(a.n_species, a.n_q, 32 * W));
+                                   efv_own_bytes<R, NMU, DTHETA>(a.n_species, a.n_q, 32 * W) +
+                                   efv_stage_bytes<R, DTHETA>(a.n_species, 32 * W));
   R* total = shares + SHARES * NSW * 32;
   R* graphs = total + NSW * 32;
   R* energy = graphs + LV::NGRAPH * 32;
@@ -149,11 +150,9 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
   R fx = R(0), fy = R(0), fz = R(0);
   // dE/dc of this thread's pairs, per neighbour species (as in efv_atom)
-  constexpr int kAccS = 4;
-  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccS * NMU * kMaxQ : 1];
-  const AccView<R> acc = (sizeof(R) == 4) ? AccView<R>{sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x}
-                                          : AccView<R>{acc_local, 1};
-  const bool own_acc = DTHETA && sm.S <= kAccS && acc.p != nullptr;
+  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccSpecies * NMU * kMaxQ : 1];
+  const AccView<R> acc = own_accumulators<R, NQ>(sm.acc, acc_local);
+  const bool own_acc = DTHETA && sm.S <= kAccSpecies && acc.p != nullptr;
   if (own_acc) {
     for (int t = 0; t < sm.S * NMU * sm.nq; ++t) acc[t] = R(0);
   }
@@ -166,23 +165,7 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   force[(warp * 3 + 1) * 32 + lane] = fy;
   force[(warp * 3 + 2) * 32 + lane] = fz;
   __syncthreads();
-  if (own_acc) {
-    if constexpr (sizeof(R) == 4) {
-      // the warps' accumulators of one atom side by side: added, then one atomic per atom and entry
-      const int per = NMU * sm.nq;
-      if (active)
-        for (int t = warp; t < sm.S * per; t += W) {
-          R s = R(0);
-          for (int v = 0; v < W; ++v) s += sm.acc[t * (32 * W) + v * 32 + lane];
-          atomicAdd(sm.dc + (zi * sm.S + t / per) * per + t % per, s);
-        }
-    } else if (active) {
-      for (int zj = 0; zj < sm.S; ++zj) {
-        R* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-        for (int t = 0; t < NMU * sm.nq; ++t) atomicAdd(dst + t, acc[zj * NMU * sm.nq + t]);
-      }
-    }
-  }
+  if (own_acc) add_warp_gradients(sm, 0, NMU * sm.nq, zi, active, [&](int t) { return acc[t]; });
   if (warp == 0 && active) {
     for (int v = 1; v < W; ++v) {
       fx += force[(v * 3 + 0) * 32 + lane];
@@ -200,9 +183,10 @@ template <class LV, class R, bool DTHETA>
 int efv_team_launch_typed(const EfvArgs& a, cudaStream_t stream) {
   const int SS = a.n_species * a.n_species;
   const size_t bytes = ((efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15)) +
-                       efv_acc_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, 32 * kTeamWarps) +
+                       efv_own_bytes<R, LV::NMU, DTHETA>(a.n_species, a.n_q, 32 * kTeamWarps) +
+                       efv_stage_bytes<R, DTHETA>(a.n_species, 32 * kTeamWarps) +
                        team_buf_bytes<LV, R>(kTeamWarps);
-  if (bytes > 227 * 1024) return kTeamNoRoom;
+  if (bytes > kMaxBlockSmem) return kTeamNoRoom;
   auto kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, 0>;
   if constexpr (std::is_same<R, float>::value) {
     if (a.n_q == kFixedQ) kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, kFixedQ>;

@@ -93,8 +93,8 @@ int basis_rows_launch(const EfvArgs& a, const int32_t* list, int64_t n_rows, dou
       return MTP_ERR_CUDA;
     }
   }
-  kern<<<(unsigned)((n_rows + kRowsThreads - 1) / kRowsThreads), kRowsThreads, bytes, stream>>>(a, list, n_rows,
-                                                                                                  rows, ld, bsum);
+  const int threads = fp64_threads(n_rows, 1);
+  kern<<<(unsigned)((n_rows + threads - 1) / threads), threads, bytes, stream>>>(a, list, n_rows, rows, ld, bsum);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("basis_rows kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));

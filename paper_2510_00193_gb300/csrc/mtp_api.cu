@@ -126,10 +126,8 @@ using namespace mtp;
 
 namespace mtp {
 // Up to this many atoms an untuned handle takes the team kernel: one wave of
-// its blocks (32 atoms, two blocks per SM).  On the mixed path with dE/dtheta
-// two waves: one thread per atom then carries the gradient accumulators too
-// (level 16: 144 against 193 us at 16,000 atoms, 809 against 687 at 128,000).
-static int64_t team_atoms(bool mixed, bool dtheta) { return 64 * (int64_t)device_sms() * (mixed && dtheta ? 2 : 1); }
+// its blocks (32 atoms, two blocks per SM); times on both sides stand at the kernel.
+static int64_t team_atoms() { return 64 * (int64_t)device_sms(); }
 }  // namespace mtp
 
 extern "C" {
@@ -519,7 +517,7 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   if (variant == 0) {
     const int bucket = std::min(63, (int)std::floor(std::log2((double)std::max<int64_t>(n, 1))));
     variant = h->tuned[precision == MTP_MIXED ? 1 : 0][bucket];
-    if (variant == 0) variant = n <= team_atoms(precision == MTP_MIXED, dtheta != nullptr) ? 2 : 1;
+    if (variant == 0) variant = n <= team_atoms() ? 2 : 1;
   }
   if (h->ops->split_comps > 0 && n > 0) {
     // moment/adjoint scratch of the split kernels (levels with component

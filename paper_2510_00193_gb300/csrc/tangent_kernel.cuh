@@ -54,18 +54,20 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EfvArgs& a = t.base;
   EfvShared<S, NMU, true> sm;     // coefficients and (tangent) accumulators in S
-  sm.setup(a, smem_raw);
+  sm.template setup<false>(a, smem_raw);
   sm.zero_gradients();
   __syncthreads();
-  const int64_t i = a.atom_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i0 = a.atom_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool active = i0 < a.atom_end;
+  const int64_t i = active ? i0 : a.atom_begin;   // a lane without an atom runs no pairs
   S Bt[LV::NBASIS];
 #pragma unroll
   for (int k = 0; k < LV::NBASIS; ++k) Bt[k] = S(0);
-  if (i < a.atom_end) {
+  {
     TangentGeom<S> geom;
     geom.load_centre(t, i, cell_of<S>(a));
     const int zi = species_at(a.z, i, a.n_species);
-    const int64_t beg = __ldg(a.offsets + i), end = __ldg(a.offsets + i + 1);
+    const int64_t beg = __ldg(a.offsets + i), end = active ? __ldg(a.offsets + i + 1) : beg;
     R M[LV::NCOMP];
 #pragma unroll
     for (int c = 0; c < LV::NCOMP; ++c) M[c] = R(0);
@@ -89,11 +91,10 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs 
 #pragma unroll
     for (int k = 0; k < LV::NBASIS; ++k) Bt[k] = B[k].t;
     S fx = S(0), fy = S(0), fz = S(0);
-    constexpr int kAccS = 4;
-    const bool own_acc = sm.S <= kAccS;
-    S acc[kAccS * NMU * kMaxQ];
+    const bool own_acc = sm.S <= kAccSpecies;
+    S acc[kAccSpecies * NMU * kMaxQ];
     if (own_acc) {
-      for (int u = 0; u < sm.S * NMU * kMaxQ; ++u) acc[u] = S(0);
+      for (int u = 0; u < sm.S * NMU * sm.nq; ++u) acc[u] = S(0);
     }
     for (int64_t k = beg; k < end; ++k) {
       const int32_t j = __ldg(a.nbr_j + k);
@@ -115,12 +116,12 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs 
         atomicAdd(t.force_tan + 3 * (int64_t)j + 2, -(double)gz.t);
       }
       if (own_acc) {
-        S* dst = acc + l.species * NMU * kMaxQ;
+        S* dst = acc + l.species * NMU * sm.nq;
 #pragma unroll
         for (int mu = 0; mu < NMU; ++mu) {
 #pragma unroll
           for (int kk = 0; kk < kMaxQ; ++kk)
-            if (kk < sm.nq) dst[mu * kMaxQ + kk] += (q[kk] * Smu[mu]).t;
+            if (kk < sm.nq) dst[mu * sm.nq + kk] += (q[kk] * Smu[mu]).t;
         }
       } else {
         S* dst = sm.dc + (zi * sm.S + l.species) * NMU * sm.nq;
@@ -132,14 +133,8 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs 
         }
       }
     }
-    if (own_acc) {
-      for (int zj = 0; zj < sm.S; ++zj) {
-        S* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-        for (int mu = 0; mu < NMU; ++mu)
-          for (int kk = 0; kk < sm.nq; ++kk) atomicAdd(dst + mu * sm.nq + kk, acc[(zj * NMU + mu) * kMaxQ + kk]);
-      }
-    }
-    if (t.force_tan) {
+    if (own_acc) add_warp_gradients(sm, 0, NMU * sm.nq, zi, active, [&](int u) { return acc[u]; });
+    if (t.force_tan && active) {
       atomicAdd(t.force_tan + 3 * i, (double)fx);
       atomicAdd(t.force_tan + 3 * i + 1, (double)fy);
       atomicAdd(t.force_tan + 3 * i + 2, (double)fz);
@@ -202,7 +197,7 @@ template <class LV, class S>
 __global__ void __launch_bounds__(kEfvThreads) tangent_moments_kernel(const TangentArgs t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EfvShared<S, LV::NMU, true> sm;
-  sm.setup(t.base, smem_raw);
+  sm.template setup<false>(t.base, smem_raw);
   __syncthreads();
   const int64_t n = t.base.atom_end - t.base.atom_begin;
   SplitShare s;
@@ -217,22 +212,20 @@ __device__ __forceinline__ void tangent_adjoint(const TangentArgs& t, const EfvS
   using R = Dual<S>;
   constexpr int NMU = LV::NMU;
   constexpr int mu_lo = LV::GROUP_MU_LO[G], mu_hi = LV::GROUP_MU_HI[G];
-  if (!s.active) return;
   const EfvArgs& a = t.base;
   TangentGeom<S> geom;
   geom.load_centre(t, s.i, cell_of<S>(a));
   const int zi = species_at(a.z, s.i, a.n_species);
   const R rcut = R(sm.rcut), mid = R(sm.mid), scale = R(sm.scale);
   S fx = S(0), fy = S(0), fz = S(0);
-  constexpr int kAccS = 4;
-  const bool own_acc = sm.S <= kAccS;
-  S acc[kAccS * NMU * kMaxQ];
+  const bool own_acc = sm.S <= kAccSpecies;
+  S acc[kAccSpecies * NMU * kMaxQ];
   if (own_acc) {
-    for (int v = 0; v < sm.S * NMU * kMaxQ; ++v) acc[v] = S(0);
+    for (int v = 0; v < sm.S * NMU * sm.nq; ++v) acc[v] = S(0);
   }
   R Dg[LV::NCOMP];
   const R* buf = static_cast<const R*>(a.mbuf) + (int64_t)a.n_parts * (tile_padded(n) * LV::NCOMP);
-  LV::template load_group<G, R>(buf + tile_offset<R>(s.t, LV::NCOMP), tile_atoms<R>(), Dg);
+  LV::template load_group<G, R>(buf + tile_offset<R>(s.active ? s.t : 0, LV::NCOMP), tile_atoms<R>(), Dg);
   for (int64_t k = s.beg; k < s.end; ++k) {
     const int32_t j = __ldg(a.nbr_j + k);
     const int32_t img = __ldg(a.nbr_img + k);
@@ -253,12 +246,12 @@ __device__ __forceinline__ void tangent_adjoint(const TangentArgs& t, const EfvS
       atomicAdd(t.force_tan + 3 * (int64_t)j + 2, -(double)gz.t);
     }
     if (own_acc) {
-      S* dst = acc + l.species * NMU * kMaxQ;
+      S* dst = acc + l.species * NMU * sm.nq;
 #pragma unroll
       for (int mu = mu_lo; mu < mu_hi; ++mu) {
 #pragma unroll
         for (int kk = 0; kk < kMaxQ; ++kk)
-          if (kk < sm.nq) dst[mu * kMaxQ + kk] += (q[kk] * Smu[mu]).t;
+          if (kk < sm.nq) dst[mu * sm.nq + kk] += (q[kk] * Smu[mu]).t;
       }
     } else {
       S* dst = sm.dc + (zi * sm.S + l.species) * NMU * sm.nq;
@@ -270,14 +263,9 @@ __device__ __forceinline__ void tangent_adjoint(const TangentArgs& t, const EfvS
       }
     }
   }
-  if (own_acc) {
-    for (int zj = 0; zj < sm.S; ++zj) {
-      S* dst = sm.dc + (zi * sm.S + zj) * NMU * sm.nq;
-      for (int mu = mu_lo; mu < mu_hi; ++mu)
-        for (int kk = 0; kk < sm.nq; ++kk) atomicAdd(dst + mu * sm.nq + kk, acc[(zj * NMU + mu) * kMaxQ + kk]);
-    }
-  }
-  if (t.force_tan) {
+  if (own_acc)
+    add_warp_gradients(sm, mu_lo * sm.nq, mu_hi * sm.nq, zi, s.active, [&](int u) { return acc[u]; });
+  if (t.force_tan && s.active) {
     atomicAdd(t.force_tan + 3 * s.i, (double)fx);
     atomicAdd(t.force_tan + 3 * s.i + 1, (double)fy);
     atomicAdd(t.force_tan + 3 * s.i + 2, (double)fz);
@@ -290,7 +278,7 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_adjoint_kernel(const Tang
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EfvArgs& a = t.base;
   EfvShared<S, NMU, true> sm;
-  sm.setup(a, smem_raw);
+  sm.template setup<false>(a, smem_raw);
   sm.zero_gradients();
   __syncthreads();
   const int64_t n = a.atom_end - a.atom_begin;
@@ -308,19 +296,27 @@ __global__ void __launch_bounds__(kEfvThreads) tangent_adjoint_kernel(const Tang
   }
 }
 
+// The tangent's accumulators are thread-private in either precision: staging only.
+template <class S, int NMU>
+size_t tangent_smem(const EfvArgs& a, int threads) {
+  const size_t base = (efv_smem_bytes<S, NMU, true>(a.n_species * a.n_species, a.n_q, a.m) + 15) & ~size_t(15);
+  const size_t stage = efv_stage_bytes<S, true>(a.n_species, threads);
+  return base + stage <= kMaxBlockSmem ? base + stage : base;
+}
+
 template <class LV, class S>
 int tangent_split_launch(const TangentArgs& t, cudaStream_t stream) {
   const EfvArgs& a = t.base;
   const int64_t n = a.atom_end - a.atom_begin;
-  const int SS = a.n_species * a.n_species;
-  const dim3 grid((unsigned)((n + kEfvThreads - 1) / kEfvThreads), 2 * a.n_parts);
-  const size_t bytes = efv_smem_bytes<S, LV::NMU, true>(SS, a.n_q, a.m);
+  const int threads = sizeof(S) == 8 ? fp64_threads(n, 2 * a.n_parts) : kEfvThreads;
+  const dim3 grid((unsigned)((n + threads - 1) / threads), 2 * a.n_parts);
+  const size_t bytes = tangent_smem<S, LV::NMU>(a, threads);
   int rc;
   if ((rc = set_smem(tangent_moments_kernel<LV, S>, bytes)) != MTP_OK) return rc;
   if ((rc = set_smem(tangent_adjoint_kernel<LV, S>, bytes)) != MTP_OK) return rc;
-  tangent_moments_kernel<LV, S><<<grid, kEfvThreads, bytes, stream>>>(t);
+  tangent_moments_kernel<LV, S><<<grid, threads, bytes, stream>>>(t);
   if ((rc = tile_contract_launch<LV, Dual<S>, true>(a, t.dtheta_tan, stream)) != MTP_OK) return rc;
-  tangent_adjoint_kernel<LV, S><<<grid, kEfvThreads, bytes, stream>>>(t);
+  tangent_adjoint_kernel<LV, S><<<grid, threads, bytes, stream>>>(t);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("tangent split kernels (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
@@ -338,19 +334,21 @@ int tangent_launch(const TangentArgs& t, int precision, cudaStream_t stream) {
     return precision == MTP_MIXED ? tangent_split_launch<LV, float>(t, stream)
                                   : tangent_split_launch<LV, double>(t, stream);
   } else {
-    const int SS = a.n_species * a.n_species;
-    const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
     cudaError_t e;
     if (precision == MTP_MIXED) {
-      const size_t bytes = efv_smem_bytes<float, LV::NMU, true>(SS, a.n_q, a.m);
+      const int threads = kEfvThreads;
+      const size_t bytes = tangent_smem<float, LV::NMU>(a, threads);
       auto kern = tangent_kernel<LV, float>;
-      if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+      const int rc = set_smem(kern, bytes);
+      if (rc != MTP_OK) return rc;
+      kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(t);
     } else {
-      const size_t bytes = efv_smem_bytes<double, LV::NMU, true>(SS, a.n_q, a.m);
+      const int threads = fp64_threads(n, 1);
+      const size_t bytes = tangent_smem<double, LV::NMU>(a, threads);
       auto kern = tangent_kernel<LV, double>;
-      if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      kern<<<grid, kEfvThreads, bytes, stream>>>(t);
+      const int rc = set_smem(kern, bytes);
+      if (rc != MTP_OK) return rc;
+      kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(t);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) {
