@@ -268,7 +268,7 @@ int mtp_set_wait_limit(int64_t ns);
  * c per configuration); pbc (HOST, 3, for all); x_dev the positions used to
  * build the per-configuration neighbour lists (same definition and order as
  * mtp_build_neighbors, indices global).  atoms_per_block: 32..256 (multiple
- * of 32) or 0 for 64; mtp_batch_tune can pick it by timing.  Synchronises. */
+ * of 32) or 0 for 32; mtp_batch_tune can pick it by timing.  Synchronises. */
 typedef struct mtp_batch mtp_batch;
 int mtp_batch_create(mtp_handle* h, int32_t n_cfg, const int64_t* atom_off, const double* cells,
                      const int32_t* pbc, const double* x_dev, int32_t atoms_per_block, mtp_batch** out,

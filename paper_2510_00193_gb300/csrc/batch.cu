@@ -23,7 +23,7 @@ struct mtp_batch {
   int device = 0;
   int32_t n_cfg = 0;
   int64_t n_atoms = 0;
-  int threads = 64;            // atoms per block of the persistent launch
+  int threads = 32;            // atoms per block of the persistent launch
   int32_t n_items = 0;
   std::vector<int64_t> h_off;
   std::vector<double> h_cells;
@@ -403,7 +403,7 @@ int mtp_batch_create(mtp_handle* h, int32_t n_cfg, const int64_t* atom_off, cons
   }
   if ((rc = b->xq.ensure(sizeof(long long) * 4 * nn)) || (rc = b->forces_f.ensure(sizeof(float) * 3 * nn)) ||
       (rc = b->eatom.ensure(sizeof(double) * nn)) ||
-      (rc = build_items(b, atoms_per_block ? atoms_per_block : 64))) {
+      (rc = build_items(b, atoms_per_block ? atoms_per_block : 32))) {
     mtp_batch_free(b);
     return rc;
   }

@@ -68,7 +68,7 @@ int batch_launch_typed(const BatchArgs& b, int threads, cudaStream_t stream) {
   const size_t base = (efv_smem_bytes<R, LV::NMU, DTHETA>(SS, b.base.n_q, b.base.m) + 15) & ~size_t(15);
   const size_t bytes = base + efv_acc_bytes<R, LV::NMU, DTHETA>(base, b.base.n_species, b.base.n_q, threads);
   auto kern = batch_kernel<LV, R, DTHETA>;
-  if constexpr (std::is_same<R, float>::value && LV::NGROUPS == 1) {
+  if constexpr (LV::NGROUPS == 1) {
     if (b.base.n_q == kFixedQ) kern = batch_kernel<LV, R, DTHETA, kFixedQ>;
   }
   if (bytes > 48 * 1024) {

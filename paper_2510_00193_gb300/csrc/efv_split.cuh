@@ -168,10 +168,10 @@ int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
   const size_t bytes = base + efv_acc_bytes<R, LV::NMU, DTHETA>(base, a.n_species, a.n_q, threads);
   auto kern = efv_kernel<LV, R, DTHETA>;
   // the single-group levels with the common radial basis size n_q = 8 run with
-  // n_q fixed at compile time on the mixed path and with dE/dtheta (FP64, 48,546
-  // atoms: 3.5 -> 2.9 ms; loops up to kMaxQ predicate FP64 operations away that
-  // still take their turn in the pipe)
-  if constexpr ((std::is_same<R, float>::value || DTHETA) && LV::NGROUPS == 1) {
+  // n_q fixed at compile time (FP64, 48,546 atoms with dE/dtheta: 3.5 -> 2.9 ms;
+  // loops up to kMaxQ predicate FP64 operations away that still take their turn
+  // in the pipe)
+  if constexpr (LV::NGROUPS == 1) {
     if (a.n_q == kFixedQ) kern = efv_kernel<LV, R, DTHETA, kFixedQ>;
   }
   if (bytes > 48 * 1024) {

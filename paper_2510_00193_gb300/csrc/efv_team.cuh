@@ -1,5 +1,5 @@
 // Energy/force kernel in which the W warps of a block share 32 atoms (lane =
-// atom): the block-parallel variant (the paper keeps a separate GPU pair style
+// atom; fewer in small systems, with several lanes per atom): the block-parallel variant (the paper keeps a separate GPU pair style
 // that spreads one atom's work over a team of threads for small systems, Sec.
 // 2.1, Table 1, and Sec. 4).  With one thread per atom a system of a few
 // thousand atoms leaves most of the GPU idle, and every thread walks ~26-54
@@ -19,7 +19,9 @@
 // SM cost more than the idle lanes of one thread per atom.  Level 16, mixed
 // energies and forces, this kernel / one thread per atom (whole call, us):
 // 2,000 atoms 39 / 60, 8,192 45 / 57, 16,000 74 / 57; with dE/dtheta 2,000 atoms
-// 49 / 108, 16,000 171 / 111; FP64 2,000 atoms 278 / 879, 16,000 1,081 / 953.
+// 49 / 108, 16,000 171 / 111; FP64 128 atoms 115 / 224 (the form before), 1,152
+// 137 / 464, 3,432 272 / 959, 8,704 558 / 941, 16,000 1,081 / 953.  With 32 atoms
+// per block always, FP64 at 128 atoms took 269 us: four SMs' FP64 pipes.
 // The form before (one warp per atom, every lane running the whole contraction)
 // took 59 us at 2,000 atoms.  Bound: instruction fetch (ncu: 3.1 of 6.5 stalled
 // warps per issue wait for instructions at 2,000 atoms).
@@ -32,6 +34,7 @@ namespace mtp {
 // Many species with a large radial basis: the coefficients leave no room for
 // the shares (the caller takes one thread per atom then).
 constexpr int kTeamNoRoom = 1000;
+constexpr int kTeamMinAtoms = 2;
 constexpr int kTeamWarps = 4;   // 8 measured slower above 2,000 atoms (the extra warps wait through the contraction)
 
 // A lane's column of a [k][32] array in shared memory.
@@ -77,7 +80,7 @@ __device__ __forceinline__ R team_adjoint(int p, LaneColumn<R> M, GraphColumn<R>
 }
 
 template <class LV, class R, bool DTHETA, int W, int NQ>
-__global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
+__global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a, const int atoms) {
   static_assert(LV::NGROUPS == 1, "levels with one component group");
   static_assert(LV::NPARTS == 4, "four parts");
   constexpr int NMU = LV::NMU, NSW = LV::NSWEPT, NP = LV::NPARTS;
@@ -95,8 +98,11 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   R* energy = graphs + LV::NGRAPH * 32;
   R* force = energy + NP * 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t i0 = a.atom_begin + (int64_t)blockIdx.x * 32 + lane;
-  const bool active = i0 < a.atom_end;
+  // lane = atom + atoms * sub: the lanes of an atom take shares of its pairs too,
+  // and run the contraction on the same values
+  const int subs = 32 / atoms, sub = lane / atoms;
+  const int64_t i0 = a.atom_begin + (int64_t)blockIdx.x * atoms + (lane & (atoms - 1));
+  const bool active = i0 < a.atom_end, owner = active && sub == 0;
   const int64_t i = active ? i0 : a.atom_begin;
   __syncthreads();
   PairGeom<R> geom;
@@ -105,14 +111,20 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   int64_t row, row_end;
   list_row(a, i, row, row_end);
   const int len = active ? (int)(row_end - row) : 0;
-  const int64_t beg = row + (int64_t)len * warp / W, end = row + (int64_t)len * (warp + 1) / W;
+  const int share = warp * subs + sub, all = W * subs;
+  const int64_t beg = row + (int64_t)len * share / all, end = row + (int64_t)len * (share + 1) / all;
   const LaneColumn<R> mine{shares + (size_t)warp * NSW * 32 + lane}, sum{total + lane};
+  // sum over the lanes of one atom (every one of them receives it)
+  auto add_subs = [&](R v) {
+    for (int o = atoms; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
   // adds the shares of `count` warps, component by component
-  auto add_shares = [&](int count) {
+  auto add_shares = [&](int count, bool across) {
     for (int k = warp; k < NSW; k += W) {
       R s = shares[k * 32 + lane];
       for (int v = 1; v < count; ++v) s += shares[(v * NSW + k) * 32 + lane];
-      sum[k] = s;
+      sum[k] = across ? add_subs(s) : s;
     }
   };
   {
@@ -123,7 +135,7 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
     LV::template store_swept<R>(M, mine);
   }
   __syncthreads();
-  add_shares(W);
+  add_shares(W, true);
   __syncthreads();
   const GraphColumn<R> G{graphs + lane};
   for (int p = warp; p < NP; p += W) team_values<LV, R>(p, sum, G);
@@ -132,15 +144,15 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
     const LaneColumn<R> share{shares + (size_t)p * NSW * 32 + lane};
     R e;
     if constexpr (DTHETA)
-      e = team_adjoint<LV, R, true>(p, sum, G, sm.xi, share, WarpBasisSink<R>{sm.dxi, lane, active});
+      e = team_adjoint<LV, R, true>(p, sum, G, sm.xi, share, WarpBasisSink<R>{sm.dxi, lane, owner});
     else
       e = team_adjoint<LV, R, false>(p, sum, G, sm.xi, share, (R*)nullptr);
     energy[p * 32 + lane] = e;
   }
   __syncthreads();
-  add_shares(NP);
+  add_shares(NP, false);
   double e_i = 0.0;
-  if (warp == 0 && active) {
+  if (warp == 0 && owner) {
     for (int p = 0; p < NP; ++p) e_i += (double)energy[p * 32 + lane];
     e_i += a.species_energy[zi];
     a.e_atom[i] = e_i;
@@ -166,12 +178,17 @@ __global__ void __launch_bounds__(32 * W, 2) efv_team_kernel(const EfvArgs a) {
   force[(warp * 3 + 2) * 32 + lane] = fz;
   __syncthreads();
   if (own_acc) add_warp_gradients(sm, 0, NMU * sm.nq, zi, active, [&](int t) { return acc[t]; });
-  if (warp == 0 && active) {
+  if (warp == 0) {
     for (int v = 1; v < W; ++v) {
       fx += force[(v * 3 + 0) * 32 + lane];
       fy += force[(v * 3 + 1) * 32 + lane];
       fz += force[(v * 3 + 2) * 32 + lane];
     }
+    fx = add_subs(fx);
+    fy = add_subs(fy);
+    fz = add_subs(fz);
+  }
+  if (warp == 0 && owner) {
     scatter_force(a, i, fx, fy, fz);
     if (!isfinite(e_i) || !isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
       flag_status(a.status, MTP_ERR_NONFINITE);
@@ -188,14 +205,17 @@ int efv_team_launch_typed(const EfvArgs& a, cudaStream_t stream) {
                        team_buf_bytes<LV, R>(kTeamWarps);
   if (bytes > kMaxBlockSmem) return kTeamNoRoom;
   auto kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, 0>;
-  if constexpr (std::is_same<R, float>::value) {
-    if (a.n_q == kFixedQ) kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, kFixedQ>;
-  }
+  if (a.n_q == kFixedQ) kern = efv_team_kernel<LV, R, DTHETA, kTeamWarps, kFixedQ>;
   int rc = set_smem(kern, bytes);
   if (rc != MTP_OK) return rc;
   const int64_t n = a.atom_end - a.atom_begin;
   if (n <= 0) return MTP_OK;
-  kern<<<(unsigned)((n + 31) / 32), 32 * kTeamWarps, bytes, stream>>>(a);
+  // fewer atoms per block while the blocks still fit one to an SM: the lanes of
+  // an atom share its pairs, and the pipes of more SMs take part
+  int atoms = 32;
+  const int64_t sms = device_sms();
+  while (atoms > kTeamMinAtoms && (n + atoms / 2 - 1) / (atoms / 2) <= sms) atoms /= 2;
+  kern<<<(unsigned)((n + atoms - 1) / atoms), 32 * kTeamWarps, bytes, stream>>>(a, atoms);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error("team kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));

@@ -15,7 +15,7 @@ namespace mtp {
 
 constexpr int kRowsThreads = 128;
 
-template <class LV>
+template <class LV, int NQ>
 __global__ void __launch_bounds__(kRowsThreads) basis_rows_kernel(const EfvArgs a, const int32_t* __restrict__ list,
                                                                   int64_t n_rows, double* __restrict__ rows,
                                                                   int64_t ld, double* __restrict__ bsum) {
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kRowsThreads) basis_rows_kernel(const EfvArgs 
       const R rinv = rsqrt_r(r2);
       const R rr = r2 * rinv;
       R f[NMU];
-      radial<R, NMU, false, false>(s_c + (zi * S + lj.species) * cstride, nq, rr, mid, scale, rcut, f, nullptr,
+      radial<R, NMU, false, false, NQ>(s_c + (zi * S + lj.species) * cstride, nq, rr, mid, scale, rcut, f, nullptr,
                                    nullptr);
       LV::template moments<R>(M, f, dx * rinv, dy * rinv, dz * rinv);
     }
@@ -85,7 +85,10 @@ int basis_rows_launch(const EfvArgs& a, const int32_t* list, int64_t n_rows, dou
   if (n_rows <= 0) return MTP_OK;
   const int SS = a.n_species * a.n_species;
   const size_t bytes = sizeof(double) * ((size_t)SS * CoefLayout<double, LV::NMU>::cstride(a.n_q) + a.m);
-  auto kern = basis_rows_kernel<LV>;
+  auto kern = basis_rows_kernel<LV, 0>;
+  if constexpr (LV::NGROUPS == 1) {
+    if (a.n_q == kFixedQ) kern = basis_rows_kernel<LV, kFixedQ>;
+  }
   if (bytes > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) {

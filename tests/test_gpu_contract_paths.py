@@ -72,3 +72,18 @@ def test_tile_edges(P, n):
             scale = np.abs(b[k]).max()
             assert np.abs(a[k] - b[k]).max() <= 1e-10 * max(1.0, scale)
             assert np.abs(m[k] - b[k]).max() <= 2e-3 * max(1.0, scale)
+
+
+@pytest.mark.parametrize("cells", [(1, 1, 1), (3, 3, 3), (6, 5, 5), (7, 7, 7), (10, 10, 10), (17, 16, 16)])
+def test_team_lanes_per_atom(P, cells):
+    """2 to 8,704 atoms: 16 to 1 lanes per atom in the team kernel, against one thread per atom (level 16)."""
+    pot = P.Potential.from_dict(pot_dict("bcc-l16-s3"))
+    st = synth.crystal("bcc", cells, 3.16, 0.08, 3, 2)
+    P.mtp_set_efv_variant(pot, 1)
+    ref, mixed_ref = run(P, pot, st, P.MTP_FP64), run(P, pot, st, P.MTP_MIXED)
+    P.mtp_set_efv_variant(pot, 2)
+    got, mixed = run(P, pot, st, P.MTP_FP64), run(P, pot, st, P.MTP_MIXED)
+    for k in ("e_atom", "forces", "virial", "dtheta"):
+        scale = max(1.0, np.abs(ref[k]).max())
+        assert np.abs(got[k] - ref[k]).max() <= 1e-11 * scale
+        assert np.abs(mixed[k] - ref[k]).max() <= 4 * np.abs(mixed_ref[k] - ref[k]).max() + 1e-6 * scale
