@@ -996,14 +996,15 @@ __global__ void __launch_bounds__(kEfvFusedThreads) efv_kernel(const EfvArgs a) 
   sm.setup(a, smem_raw);
   sm.zero_gradients();
   __syncthreads();
-  const int64_t i = a.atom_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double e_i = 0.0;
   R w[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-  const bool active = i < a.atom_end;
+  const bool active = t < a.atom_end - a.atom_begin;
+  const int64_t i = active ? thread_atom(a, t) : a.atom_begin;
   // the block's warps meet between the neighbour sweeps and the contraction,
   // so that they run the same code at the same time (instruction cache); a
   // warp without atoms runs the phases on zero pairs
-  efv_atom<LV, R, DTHETA, true, NQ>(a, sm, active ? i : a.atom_begin, active, cell_of<R>(a), a.cell, e_i, w);
+  efv_atom<LV, R, DTHETA, true, NQ>(a, sm, i, active, cell_of<R>(a), a.cell, e_i, w);
   efv_block_flush<LV, R, DTHETA>(sm, e_i, w, a.e_total, a.virial, a.dtheta);
 }
 

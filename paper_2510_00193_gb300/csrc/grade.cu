@@ -16,11 +16,13 @@
 // sum_j |b_ij| max_k |A_jk|; a row whose FP64 grade lies within eps_i of a
 // threshold is counted as ambiguous (its flag is still the FP64 comparison).
 //
-// gemm_grade_kernel: 64 rows x all m columns per block of 256 threads (in
-// column blocks of 128), K in blocks of 16 staged in shared memory, 4 x 8
-// FP64 accumulators per thread,
-// fused row maximum, bound, flags and the running maximum grade; rows come
-// either contiguously or from an index list.
+// gemm_grade_kernel: 16 RPT rows x all m columns per block of 256 threads (in
+// column blocks of 128), K in blocks of 16 staged in shared memory, RPT x 8
+// FP64 accumulators per thread, fused row maximum, bound, flags and the running
+// maximum grade.  Contiguous rows: RPT = 4.  Rows from an index list (the
+// re-check, a few percent of a chunk): RPT = 1 and a fixed grid, blocks taking
+// every gridDim-th group of 16 rows, so that some 11,000 rows spread evenly over
+// the SMs' FP64 pipes (groups of 64 were two on some SMs and one on others).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -31,11 +33,12 @@
 namespace mtp {
 
 constexpr double kGradeRelErr = 1e-12;
-constexpr int kGemmBM = 64, kGemmBK = 16, kGemmBN = 128;
+constexpr int kGemmBK = 16, kGemmBN = 128;
 
 // Row r of the product is row `src` of `rows` (stride ld), entry j read at
 // column cols[j] when cols is given (else j): the configuration mode over the
 // parameter gradient grades a subset of its columns.
+template <int RPT>
 __global__ void __launch_bounds__(256) gemm_grade_kernel(const double* __restrict__ rows, int64_t ld,
                                                          const int32_t* __restrict__ cols, int64_t n, int m,
                                                          const double* __restrict__ ainv,
@@ -46,76 +49,79 @@ __global__ void __launch_bounds__(256) gemm_grade_kernel(const double* __restric
                                                          unsigned long long* __restrict__ n_ambiguous,
                                                          const int32_t* __restrict__ list,
                                                          const unsigned* __restrict__ list_n) {
+  constexpr int kGemmBM = 16 * RPT;
   __shared__ double As[kGemmBK][kGemmBM + 1];
   __shared__ double Bs[kGemmBK][kGemmBN];
   __shared__ double red[kGemmBM][17];
   const int tid = threadIdx.x;
   const int ty = tid / 16, tx = tid % 16;
-  const int64_t row0 = (int64_t)blockIdx.x * kGemmBM;
-  if (list) {
-    n = (int64_t)*list_n;   // rows are list[0 .. *list_n)
-    if (row0 >= n) return;  // uniform over the block
-  }
-  double rmax[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int cb = 0; cb < m; cb += kGemmBN) {   // column blocks of A^-1 (one for m <= 128)
-    double acc[4][8];
+  if (list) n = (int64_t)*list_n;   // rows are list[0 .. *list_n)
+  for (int64_t row0 = (int64_t)blockIdx.x * kGemmBM; row0 < n; row0 += (int64_t)gridDim.x * kGemmBM) {
+    double rmax[RPT];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < RPT; ++r) rmax[r] = 0.0;
+    for (int cb = 0; cb < m; cb += kGemmBN) {   // column blocks of A^-1 (one for m <= 128)
+      double acc[RPT][8];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) acc[r][c] = 0.0;
-    for (int kb = 0; kb < m; kb += kGemmBK) {
+      for (int r = 0; r < RPT; ++r)
 #pragma unroll
-      for (int t = 0; t < (kGemmBM * kGemmBK) / 256; ++t) {
-        const int e = tid + 256 * t;
-        const int rr = e / kGemmBK, kk = e % kGemmBK;
-        const int64_t gr = row0 + rr;
-        const int64_t src = (gr < n && list) ? (int64_t)list[gr] : gr;
-        const int col = kb + kk;
-        As[kk][rr] = (gr < n && col < m) ? rows[src * ld + (cols ? cols[col] : col)] : 0.0;
+        for (int c = 0; c < 8; ++c) acc[r][c] = 0.0;
+      for (int kb = 0; kb < m; kb += kGemmBK) {
+#pragma unroll
+        for (int t = 0; t < (kGemmBM * kGemmBK) / 256; ++t) {
+          const int e = tid + 256 * t;
+          const int rr = e / kGemmBK, kk = e % kGemmBK;
+          const int64_t gr = row0 + rr;
+          const int64_t src = (gr < n && list) ? (int64_t)list[gr] : gr;
+          const int col = kb + kk;
+          As[kk][rr] = (gr < n && col < m) ? rows[src * ld + (cols ? cols[col] : col)] : 0.0;
+        }
+#pragma unroll
+        for (int t = 0; t < (kGemmBK * kGemmBN) / 256; ++t) {
+          const int e = tid + 256 * t;
+          const int kk = e / kGemmBN, cc = e % kGemmBN;
+          Bs[kk][cc] = (kb + kk < m && cb + cc < m) ? ainv[(int64_t)(kb + kk) * m + cb + cc] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kGemmBK; ++kk) {
+          if (kb + kk >= m) break;
+          double av[RPT], bv[8];
+#pragma unroll
+          for (int r = 0; r < RPT; ++r) av[r] = As[kk][ty * RPT + r];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) bv[c] = Bs[kk][tx + 16 * c];
+#pragma unroll
+          for (int r = 0; r < RPT; ++r)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
+        }
+        __syncthreads();
       }
 #pragma unroll
-      for (int t = 0; t < (kGemmBK * kGemmBN) / 256; ++t) {
-        const int e = tid + 256 * t;
-        const int kk = e / kGemmBN, cc = e % kGemmBN;
-        Bs[kk][cc] = (kb + kk < m && cb + cc < m) ? ainv[(int64_t)(kb + kk) * m + cb + cc] : 0.0;
-      }
-      __syncthreads();
+      for (int r = 0; r < RPT; ++r)
 #pragma unroll
-      for (int kk = 0; kk < kGemmBK; ++kk) {
-        double av[4], bv[8];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) av[r] = As[kk][ty * 4 + r];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) bv[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 8; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
-      }
-      __syncthreads();
+        for (int c = 0; c < 8; ++c) rmax[r] = fmax(rmax[r], fabs(acc[r][c]));
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 8; ++c) rmax[r] = fmax(rmax[r], fabs(acc[r][c]));
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) red[ty * 4 + r][tx] = rmax[r];
-  __syncthreads();
-  if (tid < kGemmBM) {
-    int64_t gr = row0 + tid;
-    if (gr < n) {
-      if (list) gr = list[gr];
-      double g = 0.0;
-      for (int t = 0; t < 16; ++t) g = fmax(g, red[tid][t]);
-      double bound = 0.0;
-      for (int j = 0; j < m; ++j) bound = fma(fabs(rows[gr * ld + (cols ? cols[j] : j)]), amax[j], bound);
-      bound *= kGradeRelErr;
-      gamma[gr] = g;
-      flags[gr] = (uint8_t)((g > tau_sel ? 1 : 0) | (g > tau_brk ? 2 : 0));
-      if (fabs(g - tau_sel) <= bound || fabs(g - tau_brk) <= bound) atomicAdd(n_ambiguous, 1ull);
-      atomicMax(gmax_bits, (unsigned long long)__double_as_longlong(g));
+    for (int r = 0; r < RPT; ++r) red[ty * RPT + r][tx] = rmax[r];
+    __syncthreads();
+    if (tid < kGemmBM) {
+      int64_t gr = row0 + tid;
+      if (gr < n) {
+        if (list) gr = list[gr];
+        double g = 0.0;
+        for (int t = 0; t < 16; ++t) g = fmax(g, red[tid][t]);
+        double bound = 0.0;
+        for (int j = 0; j < m; ++j) bound = fma(fabs(rows[gr * ld + (cols ? cols[j] : j)]), amax[j], bound);
+        bound *= kGradeRelErr;
+        gamma[gr] = g;
+        flags[gr] = (uint8_t)((g > tau_sel ? 1 : 0) | (g > tau_brk ? 2 : 0));
+        if (fabs(g - tau_sel) <= bound || fabs(g - tau_brk) <= bound) atomicAdd(n_ambiguous, 1ull);
+        atomicMax(gmax_bits, (unsigned long long)__double_as_longlong(g));
+      }
     }
+    __syncthreads();
   }
 }
 
@@ -245,6 +251,7 @@ extern "C" int mtp_compute_grade(mtp_handle* h, const mtp_nlist* nl, const doubl
     off += tc_x_bytes(chunk);
   }
   if ((rc = h->grade.ensure(off)) != MTP_OK) return rc;
+  if ((rc = h->order.ensure(sizeof(int32_t) * (size_t)chunk)) != MTP_OK) return rc;
   unsigned char* raw = h->grade.as<unsigned char>();
   double* base = h->grade.as<double>();
   unsigned long long* gmax_bits = reinterpret_cast<unsigned long long*>(base);
@@ -286,6 +293,8 @@ extern "C" int mtp_compute_grade(mtp_handle* h, const mtp_nlist* nl, const doubl
     const int64_t cnt = std::min<int64_t>(chunk, n - b);
     a.atom_begin = b;
     a.atom_end = b + cnt;
+    if ((rc = launch_row_order(a, h->order.as<int32_t>(), s)) != MTP_OK) return rc;
+    a.order = h->order.as<int32_t>();
     if ((rc = h->ops->rows(a, nullptr, cnt, rows, m, a_inv_cfg ? bsum : nullptr, s)) != MTP_OK) return rc;
     if (tensor) {
       auto* colmax = reinterpret_cast<unsigned long long*>(raw + o_colmax);
@@ -305,14 +314,14 @@ extern "C" int mtp_compute_grade(mtp_handle* h, const mtp_nlist* nl, const doubl
       if ((rc = tc_finalize(gbits, cnt, erow, fmax, tau_sel, tau_brk, gamma + b, flags + b, gmax_bits, list, list_n,
                             s)) != MTP_OK)
         return rc;
-      gemm_grade_kernel<<<(unsigned)((cnt + kGemmBM - 1) / kGemmBM), 256, 0, s>>>(
-          rows, m, nullptr, cnt, m, a_inv, amax, tau_sel, tau_brk, gamma + b, flags + b, gmax_bits, n_amb, list,
-          list_n);
+      const int64_t groups = std::min<int64_t>((cnt + 15) / 16, 8 * (int64_t)device_sms());
+      gemm_grade_kernel<1><<<(unsigned)groups, 256, 0, s>>>(rows, m, nullptr, cnt, m, a_inv, amax, tau_sel, tau_brk,
+                                                            gamma + b, flags + b, gmax_bits, n_amb, list, list_n);
       MTP_TRY_CUDA(cudaGetLastError());
       add_count_kernel<<<1, 1, 0, s>>>(n_rchk, list_n);
       MTP_TRY_CUDA(cudaGetLastError());
     } else if (a_inv) {
-      gemm_grade_kernel<<<(unsigned)((cnt + kGemmBM - 1) / kGemmBM), 256, 0, s>>>(
+      gemm_grade_kernel<4><<<(unsigned)((cnt + 63) / 64), 256, 0, s>>>(
           rows, m, nullptr, cnt, m, a_inv, amax, tau_sel, tau_brk, gamma + b, flags + b, gmax_bits, n_amb, nullptr,
           nullptr);
       MTP_TRY_CUDA(cudaGetLastError());
@@ -413,7 +422,7 @@ extern "C" int mtp_grade_rows(const double* rows, int64_t n_rows, int64_t ld, co
   if (e == cudaSuccess) {
     row_absmax_kernel<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(a_inv, m, amax);
     if (n_rows > 0)
-      gemm_grade_kernel<<<(unsigned)((n_rows + kGemmBM - 1) / kGemmBM), 256, 0, s>>>(
+      gemm_grade_kernel<4><<<(unsigned)((n_rows + 63) / 64), 256, 0, s>>>(
           rows, ld, cols, n_rows, m, a_inv, amax, tau_sel, tau_brk, gamma, flags, gmax_bits, n_amb, nullptr, nullptr);
     e = cudaGetLastError();
   }

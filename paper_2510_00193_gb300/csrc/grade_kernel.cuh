@@ -29,14 +29,15 @@ __global__ void __launch_bounds__(kRowsThreads) basis_rows_kernel(const EfvArgs 
   R* s_c = reinterpret_cast<R*>(smem_raw);
   R* s_xi = s_c + SS * cstride;
   fill_coefs<R, NMU>(s_c, a.radial_d, SS, nq);
-  for (int t = threadIdx.x; t < a.m; t += blockDim.x) s_xi[t] = a.xi_d[t];
+  for (int k = threadIdx.x; k < a.m; k += blockDim.x) s_xi[k] = a.xi_d[k];
   __syncthreads();
 
   const R rcut = R(a.r_cut);
   const R mid = R(0.5 * (a.r_min + a.r_cut));
   const R scale = R(2.0 / (a.r_cut - a.r_min));
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = r < n_rows;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool active = t < n_rows;
+  const int64_t r = active && a.order ? (int64_t)__ldg(a.order + t) : t;   // row (and without a list, atom) of this thread
   R B[LV::NBASIS];
 #pragma unroll
   for (int t = 0; t < LV::NBASIS; ++t) B[t] = R(0);

@@ -250,34 +250,51 @@ __global__ void __launch_bounds__(kTcK) tc_prep_y_kernel(const double* __restric
 }
 
 // Row exponents e_i and the BF16 slices of x = b D 2^-e, written as
-// [tile][s][128 x 128] in the X layout.  One thread per tile row; rows beyond
-// n (the ragged last tile) get zero slices.
-__global__ void __launch_bounds__(kTcM) tc_split_x_kernel(const double* __restrict__ rows, int64_t n, int m,
-                                                          const int* __restrict__ dexp, uint16_t* __restrict__ xs,
-                                                          int* __restrict__ erow) {
-  __shared__ int s_dexp[kTcK];
-  const int il = threadIdx.x;
-  s_dexp[il] = dexp[il];
+// [tile][s][128 x 128] in the X layout.  A block takes half a tile, 64 rows,
+// whose FP64 values it first brings into shared memory in one coalesced copy (a
+// thread that walked its own row read 32 sectors per instruction, twice); four
+// threads share a row.  Rows beyond n (the ragged last tile) get zero slices.
+// Bound: memory (920 bytes read and 1,792 written per row at m = 115).
+constexpr int kSplitRows = 64, kSplitParts = 4;
+__global__ void __launch_bounds__(kSplitRows * kSplitParts) tc_split_x_kernel(const double* __restrict__ rows,
+                                                                             int64_t n, int m,
+                                                                             const int* __restrict__ dexp,
+                                                                             uint16_t* __restrict__ xs,
+                                                                             int* __restrict__ erow) {
+  extern __shared__ __align__(16) double s_rows[];   // [kSplitRows][m]
+  __shared__ int s_dexp[kTcK], s_max[kSplitRows], s_bad[kSplitRows];
+  const int row_in = threadIdx.x % kSplitRows, part = threadIdx.x / kSplitRows;
+  const int64_t r0 = (int64_t)blockIdx.x * kSplitRows;
+  const int count = (int)max((int64_t)0, min((int64_t)kSplitRows, n - r0));
+  if (threadIdx.x < kTcK) s_dexp[threadIdx.x] = dexp[threadIdx.x];
+  if (threadIdx.x < kSplitRows) {
+    s_max[threadIdx.x] = INT_MIN;
+    s_bad[threadIdx.x] = 0;
+  }
+  for (int k = threadIdx.x; k < count * m; k += kSplitRows * kSplitParts) s_rows[k] = rows[r0 * m + k];
   __syncthreads();
-  const int64_t tile = blockIdx.x;
-  const int64_t r = tile * kTcM + il;
-  const bool valid = r < n;
-  const double* row = rows + r * m;
-  int e = 0;
-  bool bad = false;
+  const int64_t tile = r0 / kTcM, r = r0 + row_in;
+  const int il = (int)(r0 % kTcM) + row_in;
+  const bool valid = row_in < count;
+  const double* row = s_rows + row_in * m;
   if (valid) {
     // e_i = 1 + max_j floor(log2 |b_ij 2^d_j|), so that |x_ij| < 1
     int mx = INT_MIN;
-    for (int j = 0; j < m; ++j) {
+    bool bad = false;
+    for (int j = part; j < m; j += kSplitParts) {
       const long long bits = __double_as_longlong(row[j]);
       if (((bits >> 52) & 0x7FF) == 0x7FF) bad = true;
       if ((bits & 0x7FFFFFFFFFFFFFFFll) != 0) mx = max(mx, ilog2_bits(bits) + s_dexp[j]);
     }
-    e = (mx == INT_MIN || bad) ? 0 : mx + 1;
-    erow[r] = bad ? kBadRow : e;
+    atomicMax(s_max + row_in, mx);
+    if (bad) s_bad[row_in] = 1;
   }
+  __syncthreads();
+  const bool bad = s_bad[row_in] != 0;
+  const int e = (s_max[row_in] == INT_MIN || bad) ? 0 : s_max[row_in] + 1;
+  if (valid && part == 0) erow[r] = bad ? kBadRow : e;
   uint16_t* base = xs + tile * (int64_t)kTcS * (kTcM * kTcK);
-  for (int jc = 0; jc < kTcK / 8; ++jc) {
+  for (int jc = part; jc < kTcK / 8; jc += kSplitParts) {
     uint32_t q[8][kTcS];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -588,7 +605,10 @@ int tc_prepare(const double* rows, int64_t n, int m, const double* a_inv, const 
   tc_prep_y_kernel<<<kTcK, kTcK, 0, s>>>(a_inv, m, dexp, ys, fexp, fmax, status);
   MTP_TC_CHECK("tc_prep_y_kernel");
   const int64_t tiles = (n + kTcM - 1) / kTcM;
-  tc_split_x_kernel<<<(unsigned)tiles, kTcM, 0, s>>>(rows, n, m, dexp, xs, erow);
+  const size_t split_bytes = sizeof(double) * kSplitRows * (size_t)m;
+  MTP_TRY_CUDA(cudaFuncSetAttribute(tc_split_x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_bytes));
+  tc_split_x_kernel<<<(unsigned)(tiles * (kTcM / kSplitRows)), kSplitRows * kSplitParts, split_bytes, s>>>(
+      rows, n, m, dexp, xs, erow);
   MTP_TC_CHECK("tc_split_x_kernel");
   return MTP_OK;
 }

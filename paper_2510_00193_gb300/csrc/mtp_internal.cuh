@@ -82,8 +82,13 @@ struct EfvArgs {
   void* mbuf;               // levels with component groups: scratch of the split kernels in the working precision,
                             // n_parts buffers of partial moments, then the adjoints (nullptr: one fused kernel)
   int n_parts;              // shares into which the split kernels cut each atom's neighbours
+  const int32_t* order;     // kernels with one thread per atom: thread t of the range takes atom order[t] (nullptr: t)
 };
 
+// Atom of thread t of the range.
+__device__ __forceinline__ int64_t thread_atom(const EfvArgs& a, int64_t t) {
+  return a.atom_begin + (a.order ? (int64_t)__ldg(a.order + t) : t);
+}
 // List row of atom i.
 __device__ __forceinline__ void list_row(const EfvArgs& a, int64_t i, int64_t& beg, int64_t& end) {
   beg = __ldg(a.offsets + i);
@@ -112,6 +117,9 @@ struct PrepArgs {
   int* status;
 };
 int launch_prep(const PrepArgs& a, bool mixed, cudaStream_t s);
+// order[t], t < atom_end - atom_begin: the range's atoms (relative to
+// atom_begin), every 1,024 consecutive ones sorted by the length of their rows.
+int launch_row_order(const EfvArgs& a, int32_t* order, cudaStream_t s);
 // H^-1 of the cell rows, times `scale`.
 void inverse_rows(const double* cell, double scale, double* hi);
 
@@ -202,6 +210,7 @@ struct mtp_handle {
   mtp::DevBuf forces_f;  // FP32 force accumulator (mixed path)
   mtp::DevBuf grade;     // grade scratch: counters, row maxima, column sums, FP64 basis rows
   mtp::DevBuf mbuf;      // moment/adjoint scratch of levels whose contraction is interpreted
+  mtp::DevBuf order;     // atoms by row length (launch_row_order)
   int efv_variant = 0;   // 0: tuned or by size, 1: thread per atom, 2: warp per atom
   int8_t tuned[2][64] = {};   // [precision][floor(log2 N)]: 0 untuned, else the faster variant
 };
