@@ -1569,33 +1569,84 @@ class TileProgram:
         self.weights.insert(0, 1)
         assert len(self.weights) <= 64
 
+    def bank_order(self, records):
+        """Terms of the records that a quarter warp reads together, each in an order (and with its factors in one)
+        that puts the rows of one step in different bank groups of 16 bytes x 2 (slot mod 4) where that can be had.
+        Terms of weight 1 come first."""
+        pools = [sorted((t for t in r if t[2] == 1), key=str) for r in records]
+        late = [[t for t in r if t[2] != 1] for r in records]
+        out = [[] for _ in records]
+        while any(pools) or any(late):
+            options = []
+            for k, pool in enumerate(pools):
+                if not pool:
+                    pool[:], late[k] = late[k], []
+                kinds = {}
+                for t in pool:
+                    for x, y in ((t[0], t[1]), (t[1], t[0])):
+                        kinds.setdefault((x if x == self.one else x % 4, y if y == self.one else y % 4), []).append((x, y, t))
+                if pool:
+                    options.append((k, [v[0] for v in sorted(kinds.values(), key=lambda v: -len(v))]))
+            options.sort(key=lambda o: len(o[1]))
+            best, budget = [99, None], [400]
+
+            def search(depth, chosen):
+                cost = 0
+                for side in (0, 1):
+                    rows = {c[side] for c in chosen}
+                    cost += max([sum(r % 4 == g for r in rows) for g in range(4)])
+                if cost >= best[0] or budget[0] <= 0:
+                    return
+                if depth == len(options):
+                    best[:] = [cost, list(chosen)]
+                    return
+                for x, y, t in options[depth][1]:
+                    budget[0] -= best[1] is not None
+                    search(depth + 1, chosen + [(x, y, t)])
+                    if best[0] == 2:
+                        return
+
+            search(0, [])
+            for (k, _), (x, y, t) in zip(options, best[1]):
+                pools[k].remove(t)
+                out[k].append((x, y, t[2]))
+        return out
+
     def encode(self):
         """(words, slabs, phase_off): per phase its records, TILE_LANES at a time (a slab, all of the same number
         of 16-byte chunks), chunk-major so that the lanes of a warp read consecutive chunks.  A record's first chunk
         holds its destination (bit 13: accumulate) and 3 terms, the others 4 terms each; a term is
-        x | y << 13 | weight index << 26.  slabs: (first chunk, chunks << 1 | all weights are 1)."""
+        x | y << 13 | weight index << 26.  slabs: (first chunk, chunks << 1 | all weights are 1).  Records of the
+        same number of terms, and then of weights other than 1, share slabs: self.work holds per slab what the
+        warp runs, (terms of its longest record, leading chunks in which every weight is 1)."""
         widx = {w: k for k, w in enumerate(self.weights)}
-        words, slabs, phase_off = [], [], [0]
+        words, slabs, phase_off, self.work = [], [], [0], []
         pad = self.zero | self.zero << 13
         for ph in self.phases:
-            def chunks(r):
-                return 1 + max(0, -(-(len(r[2]) - 3) // 4))
-            recs = sorted(ph, key=lambda r: (all(w == 1 for _, _, w in r[2]), -chunks(r), r[0]))
+            def units(r):
+                return sum(w == 1 for _, _, w in r[2])
+            recs = sorted(ph, key=lambda r: (units(r) == len(r[2]), -len(r[2]), units(r), r[0]))
             mine = []
             for k in range(0, len(recs), TILE_LANES):
                 part = recs[k:k + TILE_LANES]
-                n = max(chunks(r) for r in part)
-                unit = all(w == 1 for r in part for _, _, w in r[2])
+                terms = max(len(r[2]) for r in part)
+                n = 1 + max(0, -(-(terms - 3) // 4))
                 cols = []
-                for r in part:
-                    cols.append([r[0] | int(r[1]) << 13] + [x | y << 13 | widx[w] << 26 for x, y, w in r[2]])
+                for q in range(0, len(part), 4):
+                    four = part[q:q + 4]
+                    for r, ts in zip(four, self.bank_order([r[2] for r in four])):
+                        cols.append([r[0] | int(r[1]) << 13] + [x | y << 13 | widx[w] << 26 for x, y, w in ts])
                 while len(cols) < TILE_LANES:
                     cols.append([TILE_NONE])
                 for c in cols:
                     c += [pad] * (4 * n - len(c))
-                mine.append((n, unit, [c[4 * q + i] for q in range(n) for c in cols for i in range(4)]))
-            for n, unit, w in sorted(mine, key=lambda t: -t[0]):
-                slabs.append((len(words) // 4, n << 1 | int(unit)))
+                unit = 0
+                while unit < n and all(c[4 * unit + i] >> 26 == 0 for c in cols for i in range(4)):
+                    unit += 1
+                mine.append((n, terms, unit, [c[4 * q + i] for q in range(n) for c in cols for i in range(4)]))
+            for n, terms, unit, w in sorted(mine, key=lambda t: -t[0]):
+                slabs.append((len(words) // 4, n << 1 | int(unit == n)))
+                self.work.append((terms, unit))
                 words += w
             phase_off.append(len(slabs))
         return words, slabs, phase_off
@@ -1608,15 +1659,15 @@ def emit_tile_program(lv):
     nm = "L%d" % lv.level
     tables = ["__device__ const uint4 kTileProg%s[] = {%s};" % (
                   nm, ",".join("{%uu,%uu,%uu,%uu}" % tuple(words[k:k + 4]) for k in range(0, len(words), 4))),
-              "__device__ const uint2 kTileSlab%s[] = {%s};" % (nm, ",".join("{%du,%du}" % s for s in slabs)),
+              "__device__ const uint2 kTileSlab%s[] = {%s};" % (nm, ",".join("{%du,%du}" % (s[0], t << 8 | u) for s, (t, u) in zip(slabs, tp.work))),
               "__device__ const int32_t kTilePhase%s[] = {%s};" % (nm, ",".join(str(v) for v in phase_off)),
               "__device__ const int32_t kTileWeight%s[] = {%s};" % (nm, ",".join(str(v) for v in tp.weights)),
               "__device__ const int32_t kTileBasis%s[] = {%s};" % (nm, ",".join(str(v) for v in tp.basis))]
     L = ["  // the contraction as phases of dot products over slots (tile_contract_kernel)",
          "  static constexpr int TILE_ONE = %d, TILE_ZERO = %d, TILE_AOFF = %d, TILE_SLOTS = %d;" % (
              tp.one, tp.zero, tp.aoff, tp.slots),
-         "  static constexpr int TILE_FORWARD = %d, TILE_PHASES = %d, TILE_WEIGHTS = %d;" % (
-             tp.n_forward, len(tp.phases), len(tp.weights))]
+         "  static constexpr int TILE_FORWARD = %d, TILE_PHASES = %d, TILE_SLABS = %d, TILE_WEIGHTS = %d;" % (
+             tp.n_forward, len(tp.phases), len(slabs), len(tp.weights))]
     for fn, ty, tab in (("tile_prog", "uint4", "kTileProg"), ("tile_slab", "uint2", "kTileSlab"),
                         ("tile_phase", "int32_t", "kTilePhase"), ("tile_weight", "int32_t", "kTileWeight"),
                         ("tile_basis", "int32_t", "kTileBasis")):

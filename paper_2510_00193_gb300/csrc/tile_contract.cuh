@@ -12,13 +12,16 @@
 //
 // Measured (whole evaluation, FCC level 20, against one thread per atom
 // interpreting the program on local-memory arrays, or one warp per atom with
-// shared-memory atomics for small systems): 2,016 atoms mixed 2.38 -> 0.140 ms,
+// shared-memory atomics for small systems): 2,016 atoms mixed 2.38 -> 0.134 ms,
 // 108,000 atoms mixed 10.4 -> 4.2 ms (there the graph kernels of efv_graphs.cuh
-// now take 1.41), one FP64 force-matching step of 4,000 atoms 41.3 -> 6.5 ms.
+// now take 1.41), one FP64 force-matching step of 4,000 atoms 41.3 -> 5.8 ms.
 //
-// Bound: shared-memory bandwidth on the FP32 path (two 16-byte reads per term
-// and thread; the four rows that a quarter warp reads lie in random bank
-// groups), the FP64 pipe on the FP64 path.
+// Bound: on the FP32 path latency, 23 phases of which 8 hold a single slab
+// (about 800 cycles each of a tile's 70,000), and the shared-memory reads
+// between them (two 16-byte reads per term and thread; the order of the terms
+// puts the four rows that a quarter warp reads in different bank groups where
+// it can: 24.8 instead of 31.0 thousand wavefronts per tile); on the FP64 path
+// its pipe, at 50 to 60% of its rate in the large phases.
 #pragma once
 #include <type_traits>
 
@@ -99,58 +102,130 @@ __device__ __forceinline__ void tile_term(const unsigned char* rows, const typen
   }
 }
 
-// One slab: each pair of threads runs one record of `chunks` 16-byte chunks.
+// `count` (1 to 4, the same for all lanes) terms of one chunk.
+template <class R, bool UNIT>
+__device__ __forceinline__ void tile_chunk(const unsigned char* rows, const typename ScalarOf<R>::T* wt, uint32_t t0,
+                                           uint32_t t1, uint32_t t2, uint32_t t3, int count, RowVec<R>& acc) {
+  if (count == 4) {
+    tile_term<R, UNIT>(rows, wt, t0, acc);
+    tile_term<R, UNIT>(rows, wt, t1, acc);
+    tile_term<R, UNIT>(rows, wt, t2, acc);
+    tile_term<R, UNIT>(rows, wt, t3, acc);
+  } else if (count == 3) {
+    tile_term<R, UNIT>(rows, wt, t0, acc);
+    tile_term<R, UNIT>(rows, wt, t1, acc);
+    tile_term<R, UNIT>(rows, wt, t2, acc);
+  } else if (count == 2) {
+    tile_term<R, UNIT>(rows, wt, t0, acc);
+    tile_term<R, UNIT>(rows, wt, t1, acc);
+  } else {
+    tile_term<R, UNIT>(rows, wt, t0, acc);
+  }
+}
+
+// One slab: each pair of threads runs one record, whose first chunk is in w0;
+// two more chunks are on their way while one runs (a chunk's work is shorter
+// than a read from L2).  `terms` is the number of terms of the longest record
+// (shorter ones are filled up with 0 * 0), and the first `unit` chunks hold
+// weights 1 only.  FP64 runs exactly these terms, the weights only where they
+// are (its pipe is the bound); FP32 runs whole chunks, of one kind per slab:
+// there each warp's latency counts, and the branches cost more than the filler
+// (2,016 atoms: 157 against 137 us per evaluation).
 template <class R, bool UNIT>
 __device__ __forceinline__ void tile_slab(unsigned char* rows, const typename ScalarOf<R>::T* wt,
-                                          const uint4* __restrict__ prog, int chunks) {
-  uint4 w = __ldg(prog);
-  const uint32_t head = w.x;
-  const uint32_t dst = head & 0x1FFFu;
+                                          const uint4* __restrict__ prog, uint4 w0, int terms, int unit) {
+  constexpr bool EXACT = sizeof(typename ScalarOf<R>::T) == 8;
+  const uint32_t dst = w0.x & 0x1FFFu;
+  uint4 w1 = w0, w2 = w0;
+  if (terms > 3) w1 = __ldg(prog + kTileLanes);
+  if (terms > 7) w2 = __ldg(prog + 2 * kTileLanes);
   RowVec<R> acc;
-  if (head & 0x2000u) {
+  if (w0.x & 0x2000u) {
     acc = row_load<R>(rows + (dst << 5));
   } else {
 #pragma unroll
     for (int k = 0; k < RowVec<R>::N; ++k) acc.e[k] = R(0);
   }
-  uint4 nxt = w;
-  if (chunks > 1) nxt = __ldg(prog + kTileLanes);
-  tile_term<R, UNIT>(rows, wt, w.y, acc);
-  tile_term<R, UNIT>(rows, wt, w.z, acc);
-  tile_term<R, UNIT>(rows, wt, w.w, acc);
-  for (int c = 1; c < chunks; ++c) {
-    w = nxt;
-    if (c + 1 < chunks) nxt = __ldg(prog + (c + 1) * kTileLanes);
-    tile_term<R, UNIT>(rows, wt, w.x, acc);
-    tile_term<R, UNIT>(rows, wt, w.y, acc);
-    tile_term<R, UNIT>(rows, wt, w.z, acc);
-    tile_term<R, UNIT>(rows, wt, w.w, acc);
+  if constexpr (EXACT) {
+    uint32_t t0 = w0.y, t1 = w0.z, t2 = w0.w, t3 = w0.w;
+    int count = min(terms, 3);
+    while (true) {
+      terms -= count;
+      if (unit > 0) tile_chunk<R, true>(rows, wt, t0, t1, t2, t3, count, acc);
+      else tile_chunk<R, false>(rows, wt, t0, t1, t2, t3, count, acc);
+      if (terms <= 0) break;
+      --unit;
+      t0 = w1.x; t1 = w1.y; t2 = w1.z; t3 = w1.w;
+      w1 = w2;
+      prog += kTileLanes;
+      if (terms > 8) w2 = __ldg(prog + 2 * kTileLanes);
+      count = min(terms, 4);
+    }
+  } else {
+    tile_term<R, UNIT>(rows, wt, w0.y, acc);
+    tile_term<R, UNIT>(rows, wt, w0.z, acc);
+    tile_term<R, UNIT>(rows, wt, w0.w, acc);
+    for (terms -= 3; terms > 0; terms -= 4) {
+      const uint4 w = w1;
+      w1 = w2;
+      prog += kTileLanes;
+      if (terms > 8) w2 = __ldg(prog + 2 * kTileLanes);
+      tile_term<R, UNIT>(rows, wt, w.x, acc);
+      tile_term<R, UNIT>(rows, wt, w.y, acc);
+      tile_term<R, UNIT>(rows, wt, w.z, acc);
+      tile_term<R, UNIT>(rows, wt, w.w, acc);
+    }
   }
   if (dst != 0x1FFFu) row_store<R>(rows + (dst << 5), acc);
 }
 
+// slab, phase: the program's slab descriptors and phase bounds, in shared
+// memory.  The first chunk of a warp's next slab is read while it runs the one
+// before, across the barrier between two phases too (a phase's slabs follow
+// the last one's, so its first slab of this warp is known by then).
 template <class LV, class R>
-__device__ __forceinline__ void tile_phases(unsigned char* rows, const typename ScalarOf<R>::T* wt, int from, int to) {
+__device__ __forceinline__ void tile_phases(unsigned char* rows, const typename ScalarOf<R>::T* wt,
+                                            const uint2* slab, const int* phase, int from, int to) {
+  constexpr int W = kTileThreads / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint4* __restrict__ base = LV::tile_prog() + (lane >> 1);
   rows += (lane & 1) * 16;
+  int start = phase[from], end = phase[from + 1];
+  int s = 0, ns = 0;
+  uint4 w;                                       // first chunk of slab s
+  bool ready = false;
   for (int p = from; p < to; ++p) {
-    const int end = __ldg(LV::tile_phase() + p + 1);
-    for (int s = __ldg(LV::tile_phase() + p) + warp; s < end; s += kTileThreads / 32) {
-      const uint2 sl = __ldg(LV::tile_slab() + s);
-      const uint4* prog = LV::tile_prog() + sl.x + (lane >> 1);
-      if (sl.y & 1u) tile_slab<R, true>(rows, wt, prog, (int)(sl.y >> 1));
-      else tile_slab<R, false>(rows, wt, prog, (int)(sl.y >> 1));
+    const int next_end = phase[min(p + 2, (int)LV::TILE_PHASES)];
+    if (!ready) {                                // the first phase, or the warp had no slab in the last one
+      s = start + warp;
+      ns = s + W < end ? s + W : end + warp;
+      w = __ldg(base + slab[min(s, LV::TILE_SLABS - 1)].x);
     }
+    ready = s < end;
+    while (s < end) {
+      const uint2 sl = slab[s];
+      const uint4 nw = __ldg(base + slab[min(ns, LV::TILE_SLABS - 1)].x);
+      const int stop = ns < end ? end : next_end;
+      const int n2 = ns + W < stop ? ns + W : stop + warp;
+      const int terms = (int)(sl.y >> 8), unit = (int)(sl.y & 0xFFu);
+      if constexpr (sizeof(typename ScalarOf<R>::T) == 8) tile_slab<R, false>(rows, wt, base + sl.x, w, terms, unit);
+      else if (unit == (terms + 4) >> 2) tile_slab<R, true>(rows, wt, base + sl.x, w, terms, unit);
+      else tile_slab<R, false>(rows, wt, base + sl.x, w, terms, unit);
+      s = ns; w = nw;
+      ns = n2;
+    }
+    start = end;
+    end = next_end;
     __syncthreads();
   }
 }
 
 // Shared memory: the slots, the weight table, one row of partial energies per
-// warp, the species counts.
+// warp, the slab descriptors and phase bounds, the species counts.
 template <class LV, class R>
 __host__ __device__ constexpr size_t tile_smem_bytes() {
   return (size_t)LV::TILE_SLOTS * kTileRowBytes + 64 * sizeof(double) + (kTileThreads / 32) * kTileRowBytes +
-         sizeof(int) * kMaxSpecies;
+         (size_t)LV::TILE_SLABS * sizeof(uint2) + sizeof(int) * (LV::TILE_PHASES + 1 + kMaxSpecies);
 }
 
 // a.mbuf: a.n_parts buffers of partial moments (the neighbour sweep's shares,
@@ -167,12 +242,16 @@ __global__ void __launch_bounds__(kTileThreads) tile_contract_kernel(const EfvAr
   unsigned char* rows = smem;
   S* wt = reinterpret_cast<S*>(smem + (size_t)LV::TILE_SLOTS * kTileRowBytes);
   R* esum = reinterpret_cast<R*>(smem + (size_t)LV::TILE_SLOTS * kTileRowBytes + 64 * sizeof(double));
-  int* cnt = reinterpret_cast<int*>(smem + tile_smem_bytes<LV, R>() - sizeof(int) * kMaxSpecies);
+  uint2* slab = reinterpret_cast<uint2*>(esum + (kTileThreads / 32) * AB);
+  int* phase = reinterpret_cast<int*>(slab + LV::TILE_SLABS);
+  int* cnt = phase + LV::TILE_PHASES + 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const S* __restrict__ xi;
   if constexpr (sizeof(S) == 4) xi = a.xi_f;
   else xi = a.xi_d;
   if (tid < LV::TILE_WEIGHTS) wt[tid] = (S)LV::tile_weight()[tid];
+  for (int k = tid; k < LV::TILE_SLABS; k += kTileThreads) slab[k] = LV::tile_slab()[k];
+  if (tid <= LV::TILE_PHASES) phase[tid] = LV::tile_phase()[tid];
   if (tid < kMaxSpecies) cnt[tid] = 0;
   if (tid < AB) {
     reinterpret_cast<R*>(rows + (size_t)LV::TILE_ONE * kTileRowBytes)[tid] = R(1);
@@ -183,12 +262,21 @@ __global__ void __launch_bounds__(kTileThreads) tile_contract_kernel(const EfvAr
   const int64_t tiles = (n + AB - 1) / AB;
   const R* __restrict__ mom = static_cast<const R*>(a.mbuf);
   R* __restrict__ dout = static_cast<R*>(a.mbuf) + part * a.n_parts;
-  double e_sum = 0.0;                            // threads < AB: site energies of their column
+  double e_sum = 0.0;                            // lane 0 of warps < AB: site energies of column `warp`
   constexpr int BPT = (LV::NBASIS + kTileThreads - 1) / kTileThreads;
   double b_sum[BPT];                             // dE/dxi of basis values tid, tid + kTileThreads, ...
 #pragma unroll
   for (int k = 0; k < BPT; ++k) b_sum[k] = 0.0;
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t mine = tile * AB + warp;         // the atom whose site energy lane 0 of warps < AB forms
+    int zi = 0;
+    double e0 = 0.0;
+    if constexpr (!DUAL) {
+      if (warp < AB && lane == 0 && mine < n) {
+        zi = species_at(a.z, a.atom_begin + mine, a.n_species);
+        e0 = a.species_energy[zi];
+      }
+    }
     // moments into the component rows, the shares of the sweep's parts added
     for (int u = tid; u < C * H; u += kTileThreads) {
       const unsigned char* src = reinterpret_cast<const unsigned char*>(mom + tile * (C * AB)) + u * 16;
@@ -201,7 +289,7 @@ __global__ void __launch_bounds__(kTileThreads) tile_contract_kernel(const EfvAr
       row_store<R>(rows + u * 16, v);
     }
     __syncthreads();
-    tile_phases<LV, R>(rows, wt, 0, LV::TILE_FORWARD);
+    tile_phases<LV, R>(rows, wt, slab, phase, 0, LV::TILE_FORWARD);
     // basis values: site energies, dE/dxi, and the seeds of the reverse pass
     RowVec<R> e;
 #pragma unroll
@@ -247,20 +335,17 @@ __global__ void __launch_bounds__(kTileThreads) tile_contract_kernel(const EfvAr
     }
     __syncthreads();
     if constexpr (!DUAL) {
-      const int64_t t = tile * AB + tid;
-      if (tid < AB && t < n) {
-        double ei = 0.0;
-        for (int w = 0; w < kTileThreads / 32; ++w) ei += (double)esum[w * AB + tid];
-        const int64_t i = a.atom_begin + t;
-        const int zi = species_at(a.z, i, a.n_species);
-        ei += a.species_energy[zi];
-        a.e_atom[i] = ei;
-        e_sum += ei;
-        if (!isfinite(ei)) flag_status(a.status, MTP_ERR_NONFINITE);
-        if (WANT_B) atomicAdd(cnt + zi, 1);
+      if (warp < AB) {                             // one warp per column (a serial sum: 5,000 cycles of a tile's 74,000)
+        const double ei = warp_sum((double)esum[lane * AB + warp]) + e0;
+        if (lane == 0 && mine < n) {
+          a.e_atom[a.atom_begin + mine] = ei;
+          e_sum += ei;
+          if (!isfinite(ei)) flag_status(a.status, MTP_ERR_NONFINITE);
+          if (WANT_B) atomicAdd(cnt + zi, 1);
+        }
       }
     }
-    tile_phases<LV, R>(rows, wt, LV::TILE_FORWARD, LV::TILE_PHASES);
+    tile_phases<LV, R>(rows, wt, slab, phase, LV::TILE_FORWARD, LV::TILE_PHASES);
     {
       unsigned char* dst = reinterpret_cast<unsigned char*>(dout + tile * (C * AB));
       const unsigned char* src = rows + (size_t)LV::TILE_AOFF * kTileRowBytes;
@@ -269,10 +354,7 @@ __global__ void __launch_bounds__(kTileThreads) tile_contract_kernel(const EfvAr
     __syncthreads();
   }
   if constexpr (!DUAL) {
-    if (warp == 0) {
-      const double s = warp_sum(tid < AB ? e_sum : 0.0);
-      if (tid == 0) atomicAdd(a.e_total, s);
-    }
+    if (warp < AB && lane == 0) atomicAdd(a.e_total, e_sum);
   }
   if constexpr (WANT_B) {
     const int64_t xoff = a.n_species + (int64_t)LV::NMU * a.n_q * a.n_species * a.n_species;
