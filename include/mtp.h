@@ -147,12 +147,15 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x_dev, con
 /* Kernel for mtp_compute_efv (same results within rounding):
  *   1: one thread per centre atom (the thread-parallel variant, for large
  *      systems; paper Sec. 2.1, Table 1);
- *   2: one warp per centre atom, the warp's lanes sharing the atom's pairs
- *      (the block-parallel variant for small systems and high levels, paper
- *      Sec. 2.1, Table 1, Sec. 4); at levels 18 and 20 the warp also shares
- *      the interpreted contraction, level by level of its records;
+ *   2: the warps of a block share up to 32 atoms, their pairs and the parts
+ *      of their contraction (the block-parallel variant for small systems,
+ *      paper Sec. 2.1, Table 1, Sec. 4);
  *   0 (default): the variant mtp_efv_tune measured faster for the atom count's
- *      power-of-two size class, else warp per atom up to 2048 atoms. */
+ *      power-of-two size class, else 2 while its blocks fit in one wave (up to
+ *      64 atoms per SM: 9,728 atoms on 152 SMs) and 1 above.
+ * Levels 18 and 20 run the same split kernels under every variant.
+ * In a stream capture before which no call has sized the handle's scratch, the
+ * FP64 path needs none (levels 18 and 20 then run as one slower kernel). */
 int mtp_set_efv_variant(mtp_handle* h, int32_t variant);
 /* Times both variants on this configuration (one warm-up and three timed
  * evaluations each, CUDA events on `stream`) and records the faster for its
@@ -306,8 +309,8 @@ void mtp_batch_free(mtp_batch* b);
  * make that first call before any stream capture starts.  All calls on a
  * device share the scratch array, so calls that overlap on the GPU race:
  * issue them one after another.  Levels 18 and 20 run here as one fused
- * kernel (mtp_compute_efv splits them into three kernels through a scratch
- * buffer it allocates): same results, about 3.4x slower at level 20.
+ * kernel (mtp_compute_efv splits them into several kernels through a scratch
+ * buffer it allocates): same results, about 14x slower at level 20.
  * Arguments and outputs as mtp_compute_efv. */
 int mtp_compute_efv_noalloc(mtp_handle* h, const mtp_nlist* nl, const double* x_dev, const int32_t* z_dev,
                             int64_t n_atoms, const double* cell, int64_t chunk_atoms, double* e_atom_dev,

@@ -269,7 +269,8 @@ EFV_AUTO, EFV_THREAD_PER_ATOM, EFV_WARP_PER_ATOM = 0, 1, 2
 
 
 def mtp_set_efv_variant(potential: Potential, variant: int) -> None:
-    """Energy/force kernel: 0 tuned/auto, 1 one thread per atom, 2 one warp per atom."""
+    """Energy/force kernel: 0 tuned/auto, 1 one thread per atom, 2 the warps of a block share
+    up to 32 atoms (levels 18 and 20: the same kernels under each)."""
     check(_lib.load().mtp_set_efv_variant(potential.handle, int(variant)))
 
 

@@ -12,8 +12,10 @@
 //
 // Measured, level 20, 108,000 atoms, mixed: contraction 3.60 ms (tile program)
 // -> 0.59 ms (values 104, products 48, adjoints 435 us); the whole evaluation
-// 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays: at 2,016 atoms it
-// takes 0.11 ms, and these kernels would run on less than half a wave each.
+// 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays (whole evaluation:
+// 2,016 atoms 0.131 ms, 4,000 atoms 0.205; these kernels 0.231 at 4,400 and 0.260
+// at 5,324, where the tile program would take about 0.225 and 0.27): they would
+// run on less than half a wave each.
 // Bound: instruction issue at 8 warps per SM (255 registers); the groups that
 // touch many components (281 of 295 in one) also wait for their D columns.
 #pragma once

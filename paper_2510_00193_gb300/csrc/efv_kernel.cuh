@@ -21,7 +21,7 @@
 
 namespace mtp {
 
-constexpr int kEfvThreads = 128;       // split and warp-per-atom kernels
+constexpr int kEfvThreads = 128;       // split and tangent kernels
 constexpr int kEfvFusedThreads = 128;  // the fused one-thread-per-atom kernel
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -837,10 +837,11 @@ __device__ __forceinline__ void adjoint_sweep(const EfvArgs& a, const EfvShared<
 // second sweep): a lane without an atom passes active = false and a valid
 // atom index i, runs no pairs, writes nothing and contributes zeros (every
 // basis function vanishes at zero moments).
-// Levels with component groups (the interpreted contractions of levels 18
-// and 20: 201 and 295 components) sweep the neighbours once per group, so
-// that a group's moments, then its adjoints, stay in registers; the full
-// vectors meet the interpreter once per atom.
+// Levels with component groups (18 and 20: 201 and 295 components) come here
+// only where no scratch may be allocated (mtp_compute_efv_noalloc, batches, a
+// stream capture); they sweep the neighbours once per group, so that a group's
+// moments, then its adjoints, stay in registers; the full vectors meet the
+// interpreter once per atom.
 // The contraction of a single-group level: the generated whole-DAG form
 // (DAG) or the default for R (per graph in FP32).
 template <class LV, bool DAG, class R, bool WANT_B, class MV, class BV>

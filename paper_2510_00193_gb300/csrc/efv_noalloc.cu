@@ -23,7 +23,7 @@
 // (moment sweep, contraction, adjoint sweep) through a moment scratch buffer
 // that it allocates; with no buffer to hand, this entry point runs them as the
 // one fused kernel (per-group neighbour sweeps, interpreted contraction in
-// local memory), which gives the same results but is about 3.4x slower at
+// local memory), which gives the same results but is about 14x slower at
 // level 20.
 //
 // Sharing.  All calls on a device share the one array and it keeps whatever

@@ -251,7 +251,7 @@ extern "C" int mtp_compute_grade(mtp_handle* h, const mtp_nlist* nl, const doubl
     off += tc_x_bytes(chunk);
   }
   if ((rc = h->grade.ensure(off)) != MTP_OK) return rc;
-  if ((rc = h->order.ensure(sizeof(int32_t) * (size_t)chunk)) != MTP_OK) return rc;
+  const bool ordered = h->order.try_ensure(sizeof(int32_t) * (size_t)chunk);
   unsigned char* raw = h->grade.as<unsigned char>();
   double* base = h->grade.as<double>();
   unsigned long long* gmax_bits = reinterpret_cast<unsigned long long*>(base);
@@ -293,8 +293,10 @@ extern "C" int mtp_compute_grade(mtp_handle* h, const mtp_nlist* nl, const doubl
     const int64_t cnt = std::min<int64_t>(chunk, n - b);
     a.atom_begin = b;
     a.atom_end = b + cnt;
-    if ((rc = launch_row_order(a, h->order.as<int32_t>(), s)) != MTP_OK) return rc;
-    a.order = h->order.as<int32_t>();
+    if (ordered) {
+      if ((rc = launch_row_order(a, h->order.as<int32_t>(), s)) != MTP_OK) return rc;
+      a.order = h->order.as<int32_t>();
+    }
     if ((rc = h->ops->rows(a, nullptr, cnt, rows, m, a_inv_cfg ? bsum : nullptr, s)) != MTP_OK) return rc;
     if (tensor) {
       auto* colmax = reinterpret_cast<unsigned long long*>(raw + o_colmax);

@@ -36,6 +36,21 @@ int DevBuf::ensure(size_t want) {
   return MTP_OK;
 }
 
+bool DevBuf::try_ensure(size_t want) {
+  if (ensure(want) == MTP_OK) return true;
+  (void)cudaGetLastError();
+  return false;
+}
+
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 void DevBuf::release() {
   if (ptr) cudaFree(ptr);
   ptr = nullptr;
@@ -564,8 +579,8 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
     if (rc != MTP_OK) return rc;
   }
   const int64_t chunk = chunk_atoms > 0 ? chunk_atoms : n;
-  // energy/force kernel: one thread per atom, or one warp per atom (small
-  // systems); forced by mtp_set_efv_variant, else the tuned choice for this
+  // energy/force kernel: one thread per atom, or the warps of a block sharing
+  // 32 (small systems); forced by mtp_set_efv_variant, else the tuned choice for this
   // size (mtp_efv_tune), else by size
   int variant = h->efv_variant;
   if (variant == 0) {
@@ -573,25 +588,29 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
     variant = h->tuned[precision == MTP_MIXED ? 1 : 0][bucket];
     if (variant == 0) variant = n <= team_atoms() ? 2 : 1;
   }
+  const bool capturing = is_capturing(s);
   if (h->ops->split_comps > 0 && n > 0) {
     // moment/adjoint scratch of the split kernels (levels with component
-    // groups), bounded by the chunk as the paper's chunk size bounds memory
+    // groups), bounded by the chunk as the paper's chunk size bounds memory;
+    // a capture that no call before has sized it for takes the one fused kernel
     const int64_t range = std::min<int64_t>(chunk, n);
     a.n_parts = split_parts(range, device_sms());
-    int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, range, a.n_parts,
-                                                precision == MTP_MIXED ? sizeof(float) : sizeof(double),
-                                                precision == MTP_MIXED && range >= kGraphAtoms ? h->ops->split_graphs : 0));
-    if (rc != MTP_OK) return rc;
-    a.mbuf = h->mbuf.ptr;
+    const size_t want = split_scratch_bytes(h->ops->split_comps, range, a.n_parts,
+                                            precision == MTP_MIXED ? sizeof(float) : sizeof(double),
+                                            precision == MTP_MIXED && range >= kGraphAtoms ? h->ops->split_graphs : 0);
+    if (!capturing || want <= h->mbuf.bytes) {
+      const int rc = h->mbuf.ensure(want);
+      if (rc != MTP_OK) return rc;
+      a.mbuf = h->mbuf.ptr;
+    }
   }
   // FP64 only: there the pipe's time is what a warp's longest row costs (48,546
   // atoms with dE/dtheta 2.90 -> 2.77 ms); the mixed kernel loses more to
-  // scattered loads than it gains (1,024,000 atoms: 1.41 -> 1.44 ms)
-  const bool ordered = variant == 1 && h->ops->split_comps == 0 && precision == MTP_FP64;
-  if (ordered) {
-    const int rc = h->order.ensure(sizeof(int32_t) * (size_t)std::min<int64_t>(chunk, n));
-    if (rc != MTP_OK) return rc;
-  }
+  // scattered loads than it gains (1,024,000 atoms: 1.41 -> 1.44 ms).  The
+  // order changes no result, so a capture (which must not allocate, and whose
+  // replays may outlive the buffer) and a call without room for it do without.
+  const bool ordered = variant == 1 && h->ops->split_comps == 0 && precision == MTP_FP64 && !capturing &&
+                       h->order.try_ensure(sizeof(int32_t) * (size_t)std::min<int64_t>(chunk, n));
   for (int64_t b = 0; b < n; b += chunk) {
     a.atom_begin = b;
     a.atom_end = b + chunk < n ? b + chunk : n;
@@ -613,7 +632,7 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
 
 int mtp_set_efv_variant(mtp_handle* h, int32_t variant) {
   if (!h || variant < 0 || variant > 2) {
-    set_error("mtp_set_efv_variant: variant must be 0 (auto), 1 (thread per atom) or 2 (warp per atom)");
+    set_error("mtp_set_efv_variant: variant must be 0 (auto), 1 (thread per atom) or 2 (warps share atoms)");
     return MTP_ERR_ARG;
   }
   h->efv_variant = variant;

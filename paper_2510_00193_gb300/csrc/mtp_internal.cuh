@@ -26,6 +26,7 @@ struct DevBuf {
   void* ptr = nullptr;
   size_t bytes = 0;
   int ensure(size_t want);
+  bool try_ensure(size_t want);   // for scratch that a call can do without
   void release();
   template <class T> T* as() const { return static_cast<T*>(ptr); }
 };
@@ -120,6 +121,8 @@ int launch_prep(const PrepArgs& a, bool mixed, cudaStream_t s);
 // order[t], t < atom_end - atom_begin: the range's atoms (relative to
 // atom_begin), every 1,024 consecutive ones sorted by the length of their rows.
 int launch_row_order(const EfvArgs& a, int32_t* order, cudaStream_t s);
+// Whether work queued on s goes into a graph (or cannot be queued at all).
+bool is_capturing(cudaStream_t s);
 // H^-1 of the cell rows, times `scale`.
 void inverse_rows(const double* cell, double scale, double* hi);
 
@@ -177,7 +180,7 @@ struct LevelEntry {
   TangentLaunch tangent;
   int split_comps;   // components per atom of the EfvArgs::mbuf scratch (0: the level needs none)
   int split_graphs;  // graphs per atom of that scratch (0: the level needs none)
-  EfvLaunch team;    // warp-per-atom energy/force kernel (levels with component groups: the split kernels)
+  EfvLaunch team;    // kernel whose warps share atoms (levels with component groups: the split kernels)
 };
 
 const LevelEntry* find_level(int level);
@@ -209,9 +212,9 @@ struct mtp_handle {
   mtp::DevBuf xq;        // fixed-point positions scratch
   mtp::DevBuf forces_f;  // FP32 force accumulator (mixed path)
   mtp::DevBuf grade;     // grade scratch: counters, row maxima, column sums, FP64 basis rows
-  mtp::DevBuf mbuf;      // moment/adjoint scratch of levels whose contraction is interpreted
+  mtp::DevBuf mbuf;      // moment/adjoint scratch of the split kernels (levels with component groups)
   mtp::DevBuf order;     // atoms by row length (launch_row_order)
-  int efv_variant = 0;   // 0: tuned or by size, 1: thread per atom, 2: warp per atom
+  int efv_variant = 0;   // 0: tuned or by size, 1: thread per atom, 2: warps share atoms
   int8_t tuned[2][64] = {};   // [precision][floor(log2 N)]: 0 untuned, else the faster variant
 };
 

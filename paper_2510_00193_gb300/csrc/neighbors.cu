@@ -723,8 +723,8 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
     if (g.pbc[k] && g.reach[k] > g.nb[k]) columns = false;   // a bin wrap beyond +-1
   uint32_t* found = nullptr;
   int* column_count = nullptr;
-  if (n > 0 && columns) {
-    if ((rc = nl->columns.ensure(sizeof(int) * (size_t)n * lanes * (depth + 1))) != MTP_OK) return rc;
+  // without room for them the rows are searched twice
+  if (n > 0 && columns && nl->columns.try_ensure(sizeof(int) * (size_t)n * lanes * (depth + 1))) {
     column_count = nl->columns.as<int>();
     found = reinterpret_cast<uint32_t*>(column_count + n * lanes);
   }
