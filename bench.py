@@ -308,8 +308,10 @@ def time_tc_kernel(P, torch, rows=262144, reps=5):
 def run_small(P, torch, args):
     """Small systems (the paper's block-parallel regime, ~2,000 atoms per GPU):
     level-16 BCC boxes of 2,000 and 16,000 atoms (3 species, sigma 0.08 A) and
-    a level-20 FCC box of 2,048 atoms (4 species), mixed precision, one thread
-    per atom against one warp per atom, and the tuner's choice."""
+    a level-20 FCC box of 2,048 atoms (4 species), mixed precision, both kernel
+    variants (the keys keep their names: variant 2 shares atoms between the
+    warps of a block; level 20 runs the same kernels under both), and the
+    tuner's choice."""
     import synth
     pot = P.Potential.from_file(os.path.join(ROOT, "potentials", POTENTIAL + ".json"))
     out = {}
@@ -336,7 +338,7 @@ def run_small(P, torch, args):
         P.mtp_set_efv_variant(pot, 0)
         res["tuner"] = P.mtp_efv_tune(pot, nl, x, z, st.cell, precision=P.MTP_MIXED)
         out["%d_atoms" % st.n] = res
-    # level 20 (interpreted contraction): 2,048-atom FCC, 4 species, the
+    # level 20 (split kernels): 2,048-atom FCC, 4 species, the
     # differentiation recipe at small size
     pot20 = P.Potential.from_file(os.path.join(ROOT, "potentials", "fcc-l20-s4.json"))
     st = synth.crystal("fcc", (8, 8, 8), 3.6, 0.1, 4, 3)
