@@ -451,6 +451,12 @@ template <class R> struct AccView {
     return vec ? p[(t >> 2) * 4 * stride + (t & 3)] : p[t * stride];
   }
 };
+// Sweeps of one component group: entries per neighbour species, and the entry
+// that the first one kept has among all groups'.
+template <class R> struct GroupAccView : AccView<R> {
+  int per, first;
+  __device__ __forceinline__ GroupAccView(AccView<R> v, int per_, int first_) : AccView<R>(v), per(per_), first(first_) {}
+};
 // This thread's accumulators: a column of the shared array (mixed path), or `local`.
 template <class R, int NQ>
 __device__ __forceinline__ AccView<R> own_accumulators(R* shared, R* local) {
@@ -565,6 +571,31 @@ __device__ __forceinline__ void add_warp_gradients(const EfvShared<R, NMU, DTHET
       }
     }
     __syncwarp();
+  }
+}
+
+// The same for accumulators that already lie in shared memory as [entry][thread]
+// with a stride of one more than the block's threads (entries [lo, hi) of each
+// neighbour species only): lane e reads entry e of all lanes where they are.
+template <class R, int NMU, bool DTHETA>
+__device__ __forceinline__ void add_warp_columns(const EfvShared<R, NMU, DTHETA>& sm, const R* cols, int lo, int hi,
+                                                 int zi, bool active) {
+  const int per = NMU * sm.nq, width = hi - lo, stride = (int)blockDim.x + 1;
+  const int lane = threadIdx.x & 31;
+  cols += threadIdx.x & ~31u;
+  unsigned of[kAccSpecies];
+#pragma unroll
+  for (int s = 0; s < kAccSpecies; ++s) of[s] = __ballot_sync(0xffffffffu, active && zi == s);
+  __syncwarp();
+  for (int e = lane; e < sm.S * width; e += 32) {
+    R* dst = sm.dc + (e / width) * per + lo + e % width;
+#pragma unroll
+    for (int s = 0; s < kAccSpecies; ++s) {
+      if (!of[s]) continue;
+      R sum = R(0);
+      for (unsigned l = of[s]; l; l &= l - 1) sum += cols[e * stride + __ffs(l) - 1];
+      atomicAdd(dst + s * sm.S * per, sum);
+    }
   }
 }
 
@@ -689,10 +720,10 @@ __device__ __forceinline__ void moment_sweep(const EfvArgs& a, const EfvShared<R
 
 // One pair of the second sweep: g = dE_i/dr_ij from D, the force and virial
 // terms and, with DTHETA, the dE/dc terms Q_k(r) S_mu.
-template <class LV, class R, bool DTHETA, int G, int NQ>
+template <class LV, class R, bool DTHETA, int G, int NQ, class Acc>
 __device__ __forceinline__ void adjoint_pair(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm, int zi,
                                              int32_t j, int zj, R dx, R dy, R dz, R rinv, const R* f, const R* df,
-                                             const R* q, const R* D, R& fx, R& fy, R& fz, R* w, AccView<R> acc,
+                                             const R* q, const R* D, R& fx, R& fy, R& fz, R* w, Acc acc,
                                              bool own_acc) {
   constexpr int NMU = LV::NMU;
   R gx, gy, gz, Smu[NMU];
@@ -716,7 +747,8 @@ __device__ __forceinline__ void adjoint_pair(const EfvArgs& a, const EfvShared<R
     }
     const int nq = NQ > 0 ? NQ : sm.nq;
     if (own_acc) {
-      const int base = zj * NMU * nq;
+      int base = zj * NMU * nq;
+      if constexpr (G >= 0) base = zj * acc.per - acc.first;
       if constexpr (sizeof(R) == 4 && NQ > 0 && NQ % 4 == 0) {   // the view's vec layout
         float4* v = reinterpret_cast<float4*>(acc.p) + (base >> 2) * acc.stride;
 #pragma unroll
@@ -766,12 +798,11 @@ __device__ __forceinline__ void adjoint_pair(const EfvArgs& a, const EfvShared<R
 // CLOSE64 as in moment_sweep; without it and without DTHETA the sweep is
 // software-pipelined like moment_sweep (with DTHETA the next pair's Q_k
 // values would stay live as well, which measured slower).
-template <class LV, class R, bool DTHETA, int G, bool CLOSE64 = false, int NQ = 0>
+template <class LV, class R, bool DTHETA, int G, bool CLOSE64 = false, int NQ = 0, class Acc>
 __device__ __forceinline__ void adjoint_sweep(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm,
                                               const PairGeom<R>& geom, const double* cell64, int zi, int64_t beg,
                                               int64_t end,
-                                              const R* D, R& fx, R& fy, R& fz, R* w, AccView<R> acc,
-                                              bool own_acc) {
+                                              const R* D, R& fx, R& fy, R& fz, R* w, Acc acc, bool own_acc) {
   constexpr int NMU = LV::NMU;
   PairStream<R> ps;
   int32_t j, img;
@@ -931,12 +962,14 @@ __device__ __forceinline__ void efv_atom(const EfvArgs& a, const EfvShared<R, LV
     {
       R Dg[LV::NCOMP];
       LV::template load_group<0, R>(D, 1, Dg);
-      adjoint_sweep<LV, R, DTHETA, 0>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w, acc, own_acc);
+      adjoint_sweep<LV, R, DTHETA, 0>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
+                                          GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
     }
     {
       R Dg[LV::NCOMP];
       LV::template load_group<1, R>(D, 1, Dg);
-      adjoint_sweep<LV, R, DTHETA, 1>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w, acc, own_acc);
+      adjoint_sweep<LV, R, DTHETA, 1>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
+                                          GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
     }
   }
   if (own_acc) add_warp_gradients(sm, 0, NMU * sm.nq, zi, active, [&](int t) { return acc[t]; });

@@ -62,6 +62,24 @@ __global__ void __launch_bounds__(kEfvThreads) split_moments_kernel(const EfvArg
   else split_moments<LV, R, 1>(a, sm, s, n);
 }
 
+// The mixed path's dE/dc accumulators: [entry of one group][thread], one more
+// column than threads.  One group's entries without a staging area, instead of
+// all groups' with one, let two blocks share an SM at level 20 with n_q = 10
+// (132 KB a block before: 108,000 atoms 1.64 ms for this kernel, 1.07 now).
+template <class LV> constexpr int largest_group_mus() {
+  int mus = 0;
+  for (int g = 0; g < LV::NGROUPS; ++g) {
+    const int n = LV::GROUP_MU_HI[g] - LV::GROUP_MU_LO[g];
+    mus = n > mus ? n : mus;
+  }
+  return mus;
+}
+template <class LV>
+__host__ __device__ inline size_t split_columns_bytes(int S, int nq, int threads) {
+  constexpr int mus = largest_group_mus<LV>();
+  return sizeof(float) * (size_t)S * mus * nq * (threads + 1);
+}
+
 template <class LV, class R, bool DTHETA, int G>
 __device__ __forceinline__ void split_adjoint(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm,
                                               const SplitShare& s, int64_t n, R* w) {
@@ -70,19 +88,25 @@ __device__ __forceinline__ void split_adjoint(const EfvArgs& a, const EfvShared<
   geom.load_centre(a, s.i, cell_of<R>(a));
   const int zi = species_at(a.z, s.i, a.n_species);
   R fx = R(0), fy = R(0), fz = R(0);
-  R acc_local[(DTHETA && sizeof(R) == 8) ? kAccSpecies * NMU * kMaxQ : 1];
-  const AccView<R> acc = own_accumulators<R, 0>(sm.acc, acc_local);
+  constexpr int mu_lo = LV::GROUP_MU_LO[G], mu_hi = LV::GROUP_MU_HI[G];
+  constexpr bool kColumns = sizeof(R) == 4;   // FP32: in shared memory, FP64: thread-private
+  R acc_local[(DTHETA && !kColumns) ? kAccSpecies * NMU * kMaxQ : 1];
+  GroupAccView<R> acc({acc_local, 1}, NMU * sm.nq, 0);
+  if (kColumns)
+    acc = GroupAccView<R>({sm.acc ? sm.acc + threadIdx.x : nullptr, (int)blockDim.x + 1}, (mu_hi - mu_lo) * sm.nq,
+                          mu_lo * sm.nq);
   const bool own_acc = DTHETA && sm.S <= kAccSpecies && acc.p != nullptr;
   if (own_acc) {
-    for (int u = 0; u < sm.S * NMU * sm.nq; ++u) acc[u] = R(0);
+    for (int u = 0; u < sm.S * acc.per; ++u) acc[u] = R(0);
   }
   R Dg[LV::NCOMP];
   const R* buf = static_cast<const R*>(a.mbuf) + (int64_t)a.n_parts * (tile_padded(n) * LV::NCOMP);
   LV::template load_group<G, R>(buf + tile_offset<R>(s.active ? s.t : 0, LV::NCOMP), tile_atoms<R>(), Dg);
   adjoint_sweep<LV, R, DTHETA, G, true>(a, sm, geom, a.cell, zi, s.beg, s.end, Dg, fx, fy, fz, w, acc, own_acc);
-  if (own_acc)
-    add_warp_gradients(sm, LV::GROUP_MU_LO[G] * sm.nq, LV::GROUP_MU_HI[G] * sm.nq, zi, s.active,
-                       [&](int t) { return acc[t]; });
+  if (own_acc) {
+    if constexpr (kColumns) add_warp_columns(sm, sm.acc, mu_lo * sm.nq, mu_hi * sm.nq, zi, s.active);
+    else add_warp_gradients(sm, mu_lo * sm.nq, mu_hi * sm.nq, zi, s.active, [&](int t) { return acc[t]; });
+  }
   if (!s.active) return;
   scatter_force(a, s.i, fx, fy, fz);
   if (!isfinite((double)fx) || !isfinite((double)fy) || !isfinite((double)fz))
@@ -93,7 +117,12 @@ template <class LV, class R, bool DTHETA>
 __global__ void __launch_bounds__(kEfvThreads) split_adjoint_kernel(const EfvArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EfvShared<R, LV::NMU, DTHETA> sm;
-  sm.setup(a, smem_raw);
+  sm.template setup<false>(a, smem_raw);
+  if (DTHETA && sizeof(R) == 4 && sm.S <= kAccSpecies) {
+    const size_t off = (efv_smem_bytes<R, LV::NMU, DTHETA>(sm.SS, sm.nq, sm.m) + 15) & ~size_t(15);
+    if (dynamic_smem_size() >= off + split_columns_bytes<LV>(sm.S, sm.nq, blockDim.x))
+      sm.acc = reinterpret_cast<R*>(smem_raw + off);
+  }
   sm.zero_gradients();
   __syncthreads();
   const int64_t n = a.atom_end - a.atom_begin;
@@ -133,7 +162,12 @@ int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
   const dim3 grid((unsigned)((n + threads - 1) / threads), 2 * a.n_parts);
   const size_t b0 = efv_smem_bytes<R, LV::NMU, false>(SS, a.n_q, a.m);
   const size_t base = (efv_smem_bytes<R, LV::NMU, DTHETA>(SS, a.n_q, a.m) + 15) & ~size_t(15);
-  const size_t b1 = base + efv_acc_bytes<R, LV::NMU, DTHETA>(base, a.n_species, a.n_q, threads);
+  size_t b1 = base;
+  if (DTHETA && a.n_species <= kAccSpecies) {
+    const size_t more = sizeof(R) == 4 ? split_columns_bytes<LV>(a.n_species, a.n_q, threads)
+                                       : efv_stage_bytes<R, DTHETA>(a.n_species, threads);
+    if (base + more <= kMaxBlockSmem) b1 += more;
+  }
   int rc;
   if ((rc = set_smem(split_moments_kernel<LV, R>, b0)) != MTP_OK) return rc;
   if ((rc = set_smem(split_adjoint_kernel<LV, R, DTHETA>, b1)) != MTP_OK) return rc;
