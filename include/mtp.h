@@ -115,7 +115,9 @@ int mtp_set_theta(mtp_handle* h, const double* theta_dev, void* stream);
  * (j, n1, n2, n3).  R_cut comes from the handle.
  * *inout: NULL to create a list, or an existing list to rebuild in place
  * (its storage grows when needed).  Synchronises `stream` (the pair count
- * sizes the list).  MTP_ERR_NEIGHBOR_OVERFLOW if an image exceeds +-511. */
+ * sizes the list).  MTP_ERR_NEIGHBOR_OVERFLOW if an image exceeds +-511.
+ * After a failure an existing list is what it was before the call (after
+ * MTP_ERR_OOM it may be empty: 0 atoms). */
 int mtp_build_neighbors(mtp_handle* h, const double* x_dev, int64_t n_atoms, const double* cell,
                         const int32_t* pbc, mtp_nlist** inout, void* stream);
 int mtp_nlist_info(const mtp_nlist* nl, int64_t* n_atoms, int64_t* n_pairs);

@@ -403,9 +403,10 @@ __global__ void __launch_bounds__(kSearchThreads) count_kernel(const SearchArgs 
 
 // List rows from what count_kernel found: a block gathers the columns of its
 // atoms and forms (j, image) of every entry, then one warp per atom orders the
-// row and writes it.  May run
-// before the host knows the pair count: does nothing if the pairs do not fit
-// in `capacity` or a column ran over.
+// row and writes it, and its offset.  May run before the host knows the pair
+// count or whether the build failed: does nothing if the pairs do not fit in
+// `capacity`, a column ran over or an error is recorded, so that a list built
+// in place keeps its offsets and rows until they are replaced together.
 constexpr int kOrderWarps = 8;
 constexpr int kOrderBuffer = 512;   // entries of one row
 template <int LANES>
@@ -413,12 +414,15 @@ __global__ void __launch_bounds__(32 * kOrderWarps) order_kernel(const SearchArg
                                                                  const uint32_t* __restrict__ found,
                                                                  const int* __restrict__ column_count,
                                                                  const int64_t* __restrict__ offsets, int64_t capacity,
+                                                                 int64_t* __restrict__ out_offsets,
                                                                  int32_t* __restrict__ out_j,
                                                                  int32_t* __restrict__ out_img) {
   __shared__ __align__(16) uint32_t buf[kOrderWarps][2][kOrderBuffer];
   __shared__ int start[kOrderWarps * LANES];   // by column of the block: its place in the row
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (__ldg(offsets + s.n) > capacity || __ldg(s.status + 1) != 0) return;
+  const int64_t total = __ldg(offsets + s.n);
+  if (total > capacity || __ldg(s.status) != 0 || __ldg(s.status + 1) != 0) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) out_offsets[s.n] = total;
   const int64_t slot0 = (int64_t)blockIdx.x * kOrderWarps, cols = s.n * LANES;
   const int atoms = (int)min((int64_t)kOrderWarps, s.n - slot0);
   constexpr int width = kOrderWarps * LANES;
@@ -452,7 +456,9 @@ __global__ void __launch_bounds__(32 * kOrderWarps) order_kernel(const SearchArg
   if (lane < ((4 - (cnt & 3)) & 3)) buf[warp][0][cnt + lane] = 0xFFFFFFFFu;
   __syncthreads();
   if (warp >= atoms) return;
-  const int64_t base = __ldg(offsets + __ldg(s.bin_meta + slot0 + warp).w);
+  const int atom = __ldg(s.bin_meta + slot0 + warp).w;
+  const int64_t base = __ldg(offsets + atom);
+  if (lane == 0) out_offsets[atom] = base;
   if (g.unique) place_row_any<true>(buf[warp][0], buf[warp][1], cnt, lane, out_j + base, out_img + base);
   else place_row_any<false>(buf[warp][0], buf[warp][1], cnt, lane, out_j + base, out_img + base);
 }
@@ -462,12 +468,15 @@ __global__ void __launch_bounds__(32 * kOrderWarps) order_kernel(const SearchArg
 // the warp orders one row after the other and writes it.
 __global__ void __launch_bounds__(kSearchThreads) fill_kernel(const SearchArgs s, const NbrGeom g,
                                                               const int64_t* __restrict__ offsets, int64_t capacity,
+                                                              int64_t* __restrict__ out_offsets,
                                                               int32_t* __restrict__ out_j,
                                                               int32_t* __restrict__ out_img) {
   __shared__ __align__(16) uint32_t buf[kSearchThreads / 32][2][kRowBuffer];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t slot = (int64_t)blockIdx.x * kSearchThreads + threadIdx.x;
-  if (__ldg(offsets + s.n) > capacity) return;
+  const int64_t total = __ldg(offsets + s.n);
+  if (total > capacity) return;
+  if (slot == 0) out_offsets[s.n] = total;
   uint32_t* bj = buf[warp][0];
   uint32_t* bi = buf[warp][1];
   bool todo = slot < s.n;
@@ -479,6 +488,7 @@ __global__ void __launch_bounds__(kSearchThreads) fill_kernel(const SearchArgs s
     pw = __ldg(s.bin_xw + slot);
     mi = __ldg(s.bin_meta + slot);
     base = __ldg(offsets + mi.w);
+    out_offsets[mi.w] = base;
     const int64_t c64 = __ldg(offsets + mi.w + 1) - base;
     cnt = (int)c64;
     if (cnt > kRowBuffer) {
@@ -578,11 +588,6 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   }
   g.rc2 = r_cut * r_cut;
   for (int k = 0; k < 9; ++k) g.cellf[k] = (float)cell[k];
-
-  for (int k = 0; k < 9; ++k) nl->cell[k] = cell[k];
-  for (int k = 0; k < 3; ++k) nl->pbc[k] = g.pbc[k];
-  nl->r_cut = r_cut;
-  nl->n_atoms = n;
 
   const int T = 256;
   const unsigned blocks = (unsigned)((n + T - 1) / T);
@@ -703,12 +708,14 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   MTP_TRY_CUDA(cub::DeviceScan::ExclusiveScan(nullptr, tmp2, (int*)nullptr, (int64_t*)nullptr, ::cuda::std::plus<>{},
                                               (int64_t)0, (int)(n + 1), stream));
   tmp_bytes = std::max(tmp_bytes, tmp2);
-  if ((rc = nl->counts.ensure(sizeof(int) * (size_t)((n + 4) & ~int64_t(3)) + tmp_bytes + 64)) != MTP_OK) return rc;
+  // counts, the new offsets, the scans' temporary storage
+  const size_t counts_bytes = sizeof(int) * (size_t)((n + 4) & ~int64_t(3)), offsets_bytes = sizeof(int64_t) * (n + 1);
+  if ((rc = nl->counts.ensure(counts_bytes + ((offsets_bytes + 15) & ~size_t(15)) + tmp_bytes + 64)) != MTP_OK)
+    return rc;
   int* counts = nl->counts.as<int>();
-  void* tmp = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(counts + n + 1) + 15) & ~uintptr_t(15));
+  int64_t* offsets = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(counts) + counts_bytes);
+  void* tmp = reinterpret_cast<char*>(offsets) + ((offsets_bytes + 15) & ~size_t(15));
   MTP_TRY_CUDA(cub::DeviceScan::ExclusiveSum(tmp, tmp_bytes, bin_count, bin_start, (int)(nbins + 1), stream));
-  if ((rc = nl->offsets.ensure(sizeof(int64_t) * (n + 1))) != MTP_OK) return rc;
-  int64_t* offsets = nl->offsets.as<int64_t>();
   MTP_TRY_CUDA(cudaMemsetAsync(counts + n, 0, sizeof(int), stream));
   const unsigned search_blocks = (unsigned)((n + kSearchThreads - 1) / kSearchThreads);
   // Columns of found neighbours.  Threads per atom: more for small systems,
@@ -743,13 +750,14 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   auto order = [&]() {
     auto kern = lanes == 1 ? order_kernel<1> : lanes == 2 ? order_kernel<2> : order_kernel<4>;
     kern<<<(unsigned)((n + kOrderWarps - 1) / kOrderWarps), 32 * kOrderWarps, 0, stream>>>(
-        sa, g, found, column_count, offsets, list_room(), nl->nbr_j.as<int32_t>(), nl->nbr_img.as<int32_t>());
+        sa, g, found, column_count, offsets, list_room(), nl->offsets.as<int64_t>(), nl->nbr_j.as<int32_t>(),
+        nl->nbr_img.as<int32_t>());
   };
   int64_t total = 0;
   int st[2] = {0, 0};
   MTP_TRY_CUDA(cudaMemcpyAsync(&total, offsets + n, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
   MTP_TRY_CUDA(cudaMemcpyAsync(st, status, sizeof(st), cudaMemcpyDeviceToHost, stream));
-  const int64_t room = found ? list_room() : 0;
+  const int64_t room = found && nl->offsets.bytes >= offsets_bytes ? list_room() : 0;
   if (room > 0) order();
   MTP_TRY_CUDA(cudaGetLastError());
   MTP_TRY_CUDA(cudaStreamSynchronize(stream));
@@ -761,16 +769,27 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
     set_error("mtp_build_neighbors: a neighbour image exceeds +-511 cells (cell too thin for the cutoff)");
     return MTP_ERR_NEIGHBOR_OVERFLOW;
   }
-  nl->n_pairs = total;
+  // the build succeeded: from here on the list is the new one.  An allocation
+  // that fails leaves an empty list (its arrays are gone)
+  nl->n_atoms = 0;
+  nl->n_pairs = 0;
+  if ((rc = nl->offsets.ensure(offsets_bytes)) != MTP_OK) return rc;
   if ((rc = nl->nbr_j.ensure(sizeof(int32_t) * std::max<int64_t>(total, 1))) != MTP_OK) return rc;
   if ((rc = nl->nbr_img.ensure(sizeof(int32_t) * std::max<int64_t>(total, 1))) != MTP_OK) return rc;
-  if (total > 0 && (!found || st[1])) {
-    fill_kernel<<<search_blocks, kSearchThreads, 0, stream>>>(sa, g, offsets, list_room(), nl->nbr_j.as<int32_t>(),
-                                                              nl->nbr_img.as<int32_t>());
+  if (total == 0) {
+    MTP_TRY_CUDA(cudaMemcpyAsync(nl->offsets.ptr, offsets, offsets_bytes, cudaMemcpyDeviceToDevice, stream));
+  } else if (!found || st[1]) {
+    fill_kernel<<<search_blocks, kSearchThreads, 0, stream>>>(sa, g, offsets, list_room(), nl->offsets.as<int64_t>(),
+                                                              nl->nbr_j.as<int32_t>(), nl->nbr_img.as<int32_t>());
   } else if (total > room) {
     order();
   }
   MTP_TRY_CUDA(cudaGetLastError());
+  for (int k = 0; k < 9; ++k) nl->cell[k] = cell[k];
+  for (int k = 0; k < 3; ++k) nl->pbc[k] = g.pbc[k];
+  nl->r_cut = r_cut;
+  nl->n_atoms = n;
+  nl->n_pairs = total;
   return MTP_OK;
 }
 
