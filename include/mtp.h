@@ -390,6 +390,11 @@ int mtp_md_status(mtp_md* md, int64_t* steps_since_build, int64_t* rebuilds, voi
  * synchronisation per step) and the skin list is rebuilt at once when an atom
  * has moved more than skin/2, so no step uses an incomplete list (the LAMMPS
  * default of checking every step).
+ * A list build that fails inside the run stops it: the exact list is then that
+ * of the last completed step, while x has moved and forces and e_pot of the
+ * stopped step are undefined.  After MTP_ERR_OOM there may be no list:
+ * mtp_md_run and mtp_md_nlist then return MTP_ERR_STALE_LIST until
+ * mtp_md_rebuild has succeeded.
  * rebuild_every > 0: the skin list is rebuilt after every rebuild_every steps
  * (the displacement check is read before each rebuild and at the end, which
  * synchronises; MTP_ERR_STALE_LIST stops the run).  rebuild_every = 0: no

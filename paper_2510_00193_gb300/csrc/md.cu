@@ -130,13 +130,14 @@ __device__ __forceinline__ bool md_keep_pair(const double* __restrict__ x, const
 // (coalesced list reads) and a ballot keeps the kept ones in list order,
 // packed at the start of the atom's skin-list segment of tmp_j / tmp_img;
 // counts[i] = their number (the warp of i = n writes counts[n] = 0 for the
-// scan).
-__global__ void md_filter_kernel(const double* __restrict__ x, const float4* __restrict__ xf, int64_t n, MdFilterGeom g,
+// scan).  skip: where it is set the rows of the pass before stay (nullptr: never).
+__global__ void md_filter_kernel(const int* __restrict__ skip, const double* __restrict__ x, const float4* __restrict__ xf, int64_t n, MdFilterGeom g,
                                  const int64_t* __restrict__ off, const int32_t* __restrict__ nj,
                                  const int32_t* __restrict__ nimg, int64_t* __restrict__ counts,
                                  int32_t* __restrict__ tmp_j, int32_t* __restrict__ tmp_img) {
   const int lane = threadIdx.x & 31;
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (skip && __ldg(skip) != 0) return;
   if (i == n && lane == 0) counts[n] = 0;
   if (i >= n) return;   // warp-uniform
   const float4 pi = xf[i];
@@ -177,9 +178,16 @@ __global__ void md_compact_kernel(int64_t n, const int64_t* __restrict__ off, co
   }
 }
 
+// spec: status word of an evaluation queued before its list was known to be
+// complete; it is now, so its error goes into the handle's word (nullptr: none).
 __global__ void md_kick_kernel(double* __restrict__ v, const double* __restrict__ f, const int32_t* __restrict__ z,
-                               MdMass mm, double dt, int64_t n, double* __restrict__ e_kin) {
+                               MdMass mm, double dt, int64_t n, double* __restrict__ e_kin, int* __restrict__ spec,
+                               int* __restrict__ status) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && spec && *spec != 0) {
+    atomicCAS(status, 0, *spec);
+    *spec = 0;
+  }
   double ke = 0.0;
   if (i < n) {
     const int zi = min(max(z[i], 0), kMaxSpecies - 1);   // species checked by the force pass
@@ -246,10 +254,11 @@ struct mtp_md {
   mtp::DevBuf counts;               // int64 [N + 1] and the scan's temporary storage
   mtp::DevBuf tmp;                  // kept pairs at their skin-list positions: j, then image [2][P_skin]
   bool compact = true;              // `exact` holds the kept pairs of the last filter pass
+  bool rows_valid = false;          // tmp and counts hold rows of the skin list (not after a build that ran out of memory)
   int* host_flag = nullptr;         // pinned copy of the displacement flag, and the event after the copy
   cudaEvent_t flag_read = nullptr;
   size_t scan_bytes = 0;
-  mtp::DevBuf e_atom, small;        // site energies [N]; virial [6], E_pot [1], flags [1]
+  mtp::DevBuf e_atom, small;        // site energies [N]; virial [6], E_pot, displacement flag, E_kin, md_spec word
   mtp::MdFilterGeom geom;
   int64_t steps_total = 0;          // steps run since creation
   double scale_since_build = 1.0;   // product of barostat scale factors since the last skin-list build
@@ -293,17 +302,24 @@ void md_set_cell(mtp_md* md, const double* cell) {
     for (int k = 0; k < 9; ++k) md->exact->cell[k] = cell[k];
 }
 
-// Exact rows of x at the start of the skin-list segments (md->tmp, counts).
-int md_filter(mtp_md* md, const double* x, cudaStream_t s) {
+// Device words of md->small: the displacement flag, and the status word of the
+// evaluations that mtp_md_run queues before it has read that flag.
+int* md_flag(const mtp_md* md) { return reinterpret_cast<int*>(md->small.as<double>() + 7); }
+int* md_spec(const mtp_md* md) { return reinterpret_cast<int*>(md->small.as<double>() + 9); }
+
+// Exact rows of x at the start of the skin-list segments (md->tmp, counts);
+// skip as in the kernel.
+int md_filter(mtp_md* md, const double* x, const int* skip, cudaStream_t s) {
   using namespace mtp;
   const int64_t n = md->n_atoms;
+  md->rows_valid = true;
   if (n == 0) return MTP_OK;
   const int T = 256;   // 8 atoms (warps) per block; n + 1 warps
   const unsigned blocks = (unsigned)((32 * (n + 1) + T - 1) / T);
   mtp_nlist* sl = md->skin_list;
   int32_t* tmp_j = md->tmp.as<int32_t>();
   int32_t* tmp_img = tmp_j + std::max<int64_t>(sl->n_pairs, 1);
-  md_filter_kernel<<<blocks, T, 0, s>>>(x, md->xf.as<float4>(), n, md->geom, sl->offsets.as<int64_t>(),
+  md_filter_kernel<<<blocks, T, 0, s>>>(skip, x, md->xf.as<float4>(), n, md->geom, sl->offsets.as<int64_t>(),
                                         sl->nbr_j.as<int32_t>(), sl->nbr_img.as<int32_t>(),
                                         md->counts.as<int64_t>(), tmp_j, tmp_img);
   MTP_TRY_CUDA(cudaGetLastError());
@@ -315,7 +331,7 @@ int md_filter(mtp_md* md, const double* x, cudaStream_t s) {
 int md_compact(mtp_md* md, cudaStream_t s) {
   using namespace mtp;
   const int64_t n = md->n_atoms;
-  if (n == 0 || md->compact) return MTP_OK;
+  if (n == 0 || md->compact || !md->rows_valid) return MTP_OK;
   const int T = 256;
   const unsigned blocks = (unsigned)((32 * (n + 1) + T - 1) / T);
   int64_t* counts = md->counts.as<int64_t>();
@@ -348,19 +364,30 @@ mtp_nlist md_rows(const mtp_md* md) {
   return v;
 }
 
+// An md whose last list build ran out of memory has no list.
+int md_check_rows(const mtp_md* md, const char* what) {
+  if (md->rows_valid) return MTP_OK;
+  set_error("%s: the last skin-list build ran out of memory; call mtp_md_rebuild first", what);
+  return MTP_ERR_STALE_LIST;
+}
+
 int md_read_flags(mtp_md* md, cudaStream_t s, int* flags) {
-  int* dflags = reinterpret_cast<int*>(md->small.as<double>() + 7);
-  MTP_TRY_CUDA(cudaMemcpyAsync(flags, dflags, sizeof(int), cudaMemcpyDeviceToHost, s));
+  MTP_TRY_CUDA(cudaMemcpyAsync(flags, md_flag(md), sizeof(int), cudaMemcpyDeviceToHost, s));
   MTP_TRY_CUDA(cudaStreamSynchronize(s));
   return MTP_OK;
 }
 
+// A build that fails leaves the skin list, and with it the rows of the last
+// filter pass and the exact list, as they were, unless it ran out of memory.
 int md_rebuild(mtp_handle* h, mtp_md* md, const double* x, cudaStream_t s) {
   using namespace mtp;
   const int64_t n = md->n_atoms;
   int rc = build_neighbors(md->skin_list, x, n, md->cell, md->pbc, md->r_cut + md->skin, s);
-  if (rc != MTP_OK) return rc;
-  md->skin_list->n_atoms = n;
+  if (rc != MTP_OK) {
+    if (rc == MTP_ERR_OOM && md->skin_list->n_atoms != n) md->rows_valid = false;
+    return rc;
+  }
+  md->rows_valid = false;   // until the filter pass below
   mtp_nlist* ex = md->exact;
   ex->n_atoms = n;
   ex->r_cut = md->r_cut;
@@ -377,13 +404,12 @@ int md_rebuild(mtp_handle* h, mtp_md* md, const double* x, cudaStream_t s) {
     md_float_positions_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(x, n, md->xf.as<float4>());
     MTP_TRY_CUDA(cudaGetLastError());
   }
-  int* dflags = reinterpret_cast<int*>(md->small.as<double>() + 7);
-  MTP_TRY_CUDA(cudaMemsetAsync(dflags, 0, sizeof(int), s));
+  MTP_TRY_CUDA(cudaMemsetAsync(md_flag(md), 0, sizeof(int), s));
   md->since_build = 0;
   md->rebuilds += 1;
   md->scale_since_build = 1.0;
   (void)h;
-  return md_filter(md, x, s);
+  return md_filter(md, x, nullptr, s);
 }
 
 // The displacement flag of the last drift, read while the GPU goes on with
@@ -392,8 +418,7 @@ int md_rebuild(mtp_handle* h, mtp_md* md, const double* x, cudaStream_t s) {
 int md_flag_queue(mtp_md* md, cudaStream_t s) {
   if (!md->host_flag) MTP_TRY_CUDA(cudaHostAlloc((void**)&md->host_flag, sizeof(int), cudaHostAllocDefault));
   if (!md->flag_read) MTP_TRY_CUDA(cudaEventCreateWithFlags(&md->flag_read, cudaEventDisableTiming));
-  int* dflags = reinterpret_cast<int*>(md->small.as<double>() + 7);
-  MTP_TRY_CUDA(cudaMemcpyAsync(md->host_flag, dflags, sizeof(int), cudaMemcpyDeviceToHost, s));
+  MTP_TRY_CUDA(cudaMemcpyAsync(md->host_flag, md_flag(md), sizeof(int), cudaMemcpyDeviceToHost, s));
   MTP_TRY_CUDA(cudaEventRecord(md->flag_read, s));
   return MTP_OK;
 }
@@ -469,6 +494,7 @@ int mtp_md_create(mtp_handle* h, const double* x, int64_t n, const double* cell,
     mtp_md_free(md);
     return rc;
   }
+  cudaMemsetAsync(md_spec(md), 0, sizeof(int), s);
   if ((rc = md_rebuild(h, md, x, s)) != MTP_OK || (rc = md_compact(md, s)) != MTP_OK) {
     mtp_md_free(md);
     return rc;
@@ -493,6 +519,8 @@ int mtp_md_nlist(mtp_md* md, const mtp_nlist** nl, void* stream) {
   }
   cudaStream_t s = (cudaStream_t)stream;
   int64_t total = 0;
+  const int rc = md_check_rows(md, "mtp_md_nlist");
+  if (rc != MTP_OK) return rc;
   if (md->n_atoms > 0) {
     MTP_TRY_CUDA(cudaMemcpyAsync(&total, md->exact->offsets.as<int64_t>() + md->n_atoms, sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, s));
@@ -530,7 +558,7 @@ int mtp_md_run(mtp_handle* h, mtp_md* md, double* x, double* v, const int32_t* z
                double* e_kin, void* stream) {
   const int rc = md_run_steps(h, md, x, v, z, mass, dt, n_steps, rebuild_every, precision, forces, e_pot, e_kin, stream);
   if (!md) return rc;
-  const int rc2 = md_compact(md, (cudaStream_t)stream);   // also after a run that stopped early
+  const int rc2 = md_compact(md, (cudaStream_t)stream);   // also after a run that stopped early: its last rows
   return rc != MTP_OK ? rc : rc2;
 }
 
@@ -551,6 +579,8 @@ static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const i
     set_error("mtp_md_run: dt is not finite");
     return MTP_ERR_ARG;
   }
+  int rc = md_check_rows(md, "mtp_md_run");
+  if (rc != MTP_OK) return rc;
   MdMass mm;
   for (int k = 0; k < kMaxSpecies; ++k) mm.inv_m[k] = mm.half_m[k] = 0.0;
   for (int k = 0; k < h->n_species; ++k) {
@@ -565,10 +595,12 @@ static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const i
   const int64_t n = md->n_atoms;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   double* small = md->small.as<double>();
-  int* dflags = reinterpret_cast<int*>(small + 7);
+  int* dflags = md_flag(md);
   const bool npt = md->tau_p > 0.0;
   const bool graded = md->a_inv && md->grade_every > 0;
-  int rc;
+  const bool checked = rebuild_every < 0;
+  int* status = h->status.as<int>();
+  int* spec = checked ? md_spec(md) : nullptr;
   for (int32_t step = 0; step < n_steps; ++step) {
     // half the skin, less what the barostat has compressed the cell by since
     // the last build: a pair beyond R_cut + skin then was at least
@@ -586,8 +618,8 @@ static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const i
     double* ek = e_kin ? e_kin + step : (npt ? small + 8 : nullptr);
     auto evaluate = [&]() {
       const mtp_nlist rows = md_rows(md);
-      return mtp_compute_efv(h, &rows, x, z, n, md->cell, precision, 0, md->e_atom.as<double>(), forces, small, ep,
-                             nullptr, stream);
+      return compute_efv(h, &rows, x, z, n, md->cell, precision, 0, md->e_atom.as<double>(), forces, small, ep,
+                         nullptr, checked ? spec : status, s);
     };
     if (n > 0) {
       md_kick_drift_kernel<<<blocks, 256, 0, s>>>(x, v, forces, z, mm, dt, n, md->xref.as<double>(), half_skin2,
@@ -596,19 +628,24 @@ static int md_run_steps(mtp_handle* h, mtp_md* md, double* x, double* v, const i
     } else if (ek) {
       MTP_TRY_CUDA(cudaMemsetAsync(ek, 0, sizeof(double), s));
     }
-    if (rebuild_every < 0 && (rc = md_flag_queue(md, s)) != MTP_OK) return rc;
-    if ((rc = md_filter(md, x, s)) != MTP_OK || (rc = evaluate()) != MTP_OK) return rc;
-    if (rebuild_every < 0) {
+    if (checked && (rc = md_flag_queue(md, s)) != MTP_OK) return rc;
+    if ((rc = md_filter(md, x, checked ? dflags : nullptr, s)) != MTP_OK || (rc = evaluate()) != MTP_OK) return rc;
+    if (checked) {
       // displacement check of this step's positions.  The evaluation is queued
       // before the flag is known, so that the GPU does not wait for the host; in
-      // the rare step whose list may be incomplete it is done again (every
-      // output is overwritten) on a fresh list before anything uses it
+      // the rare step whose list may be incomplete the filter leaves the rows of
+      // the step before (they stay the exact list should the build fail), and
+      // the evaluation on them is done again (every output is overwritten, its
+      // status word dropped) on a fresh list before anything uses it
       int flags = 0;
       if ((rc = md_flag_wait(md, &flags)) != MTP_OK) return rc;
-      if (flags && ((rc = md_rebuild(h, md, x, s)) != MTP_OK || (rc = evaluate()) != MTP_OK)) return rc;
+      if (flags) {
+        MTP_TRY_CUDA(cudaMemsetAsync(spec, 0, sizeof(int), s));
+        if ((rc = md_rebuild(h, md, x, s)) != MTP_OK || (rc = evaluate()) != MTP_OK) return rc;
+      }
     }
     if (n > 0) {
-      md_kick_kernel<<<blocks, 256, 0, s>>>(v, forces, z, mm, dt, n, ek);
+      md_kick_kernel<<<blocks, 256, 0, s>>>(v, forces, z, mm, dt, n, ek, spec, status);
       MTP_TRY_CUDA(cudaGetLastError());
     }
     md->since_build += 1;

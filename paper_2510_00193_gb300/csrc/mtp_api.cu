@@ -490,6 +490,15 @@ void mtp_free_nlist(mtp_nlist* nl) {
 int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const int32_t* z, int64_t n,
                     const double* cell, int32_t precision, int64_t chunk_atoms, double* e_atom, double* forces,
                     double* virial, double* e_total, double* dtheta, void* stream) {
+  return compute_efv(h, nl, x, z, n, cell, precision, chunk_atoms, e_atom, forces, virial, e_total, dtheta,
+                     h ? h->status.as<int>() : nullptr, (cudaStream_t)stream);
+}
+
+}  // extern "C"
+
+int mtp::compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const int32_t* z, int64_t n,
+                     const double* cell, int32_t precision, int64_t chunk_atoms, double* e_atom, double* forces,
+                     double* virial, double* e_total, double* dtheta, int* status, cudaStream_t s) {
   if (!h || !nl || !cell || !e_atom || !forces || !virial || !e_total || (n > 0 && (!x || !z))) {
     set_error("mtp_compute_efv: NULL argument");
     return MTP_ERR_ARG;
@@ -515,7 +524,6 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
       return MTP_ERR_ARG;
     }
   }
-  cudaStream_t s = (cudaStream_t)stream;
   if (n == 0) {
     MTP_TRY_CUDA(cudaMemsetAsync(virial, 0, sizeof(double) * 6, s));
     MTP_TRY_CUDA(cudaMemsetAsync(e_total, 0, sizeof(double), s));
@@ -552,7 +560,7 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   a.virial = virial;
   a.e_total = e_total;
   a.dtheta = dtheta;
-  a.status = h->status.as<int>();
+  a.status = status;
   PrepArgs pa;
   std::memset(&pa, 0, sizeof(pa));
   pa.x = x;
@@ -629,6 +637,8 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const i
   }
   return MTP_OK;
 }
+
+extern "C" {
 
 int mtp_set_efv_variant(mtp_handle* h, int32_t variant) {
   if (!h || variant < 0 || variant > 2) {

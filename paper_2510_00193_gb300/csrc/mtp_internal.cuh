@@ -228,3 +228,10 @@ struct mtp_nlist {
   const int64_t* row_counts = nullptr;   // entries of row i from offsets[i] on (nullptr: up to offsets[i + 1])
   mtp::DevBuf counts, bins, bin_start, bin_atoms, wrapped, columns, status;
 };
+
+namespace mtp {
+// mtp_compute_efv with the device word that takes its error status.
+int compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const int32_t* z, int64_t n, const double* cell,
+                int32_t precision, int64_t chunk_atoms, double* e_atom, double* forces, double* virial,
+                double* e_total, double* dtheta, int* status, cudaStream_t s);
+}  // namespace mtp
