@@ -70,13 +70,18 @@ template <int M> struct StagedBasisSink {
   }
 };
 
+// Shared memory of the products kernel: no pair coefficients, so it does not
+// grow with the species or n_q, and the staging area always fits beside the sums.
+template <class LV, bool DTHETA> constexpr size_t graph_products_bytes() {
+  return efv_sums_bytes<float, LV::NBASIS>() + (DTHETA ? sizeof(float) * 33 * kEfvThreads : 0);
+}
+
 template <class GR, class LV, bool DTHETA>
 __global__ void __launch_bounds__(kEfvThreads) graph_products_kernel(const EfvArgs a, const float* __restrict__ G,
                                                                      float* __restrict__ GB, int64_t gld) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EfvShared<float, LV::NMU, DTHETA> sm;
-  sm.setup(a, smem_raw);
-  sm.zero_gradients();
+  sm.template setup_sums<LV::NBASIS>(a, smem_raw);
   __syncthreads();
   const int64_t n = a.atom_end - a.atom_begin;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -87,9 +92,9 @@ __global__ void __launch_bounds__(kEfvThreads) graph_products_kernel(const EfvAr
   const int64_t u = active ? t : 0;
   if (__any_sync(0xffffffffu, active)) {
     // the scratch has room for the padding atoms of the last block's warps: see split_scratch_bytes
-    __shared__ float stage[DTHETA ? kEfvThreads * 33 : 1];
-    const StagedBasisSink<LV::NBASIS> sink{stage + (DTHETA ? (threadIdx.x >> 5) * 32 * 33 : 0), sm.dxi,
-                                           (int)(threadIdx.x & 31), active};
+    float* stage = reinterpret_cast<float*>(smem_raw + efv_sums_bytes<float, LV::NBASIS>());
+    const StagedBasisSink<LV::NBASIS> sink{stage + (threadIdx.x >> 5) * 32 * 33, sm.dxi, (int)(threadIdx.x & 31),
+                                           active};
     const float e = GR::template products<DTHETA>(G + u, gld, sm.xi, GB + t, sink);
     if (active) {
       const int64_t i = a.atom_begin + t;
@@ -124,9 +129,8 @@ int graphs_launch_seq(const EfvArgs& a, cudaStream_t stream, std::integer_sequen
   float* G = D + part;
   float* GB = G + gld * LV::NGRAPH;
   const unsigned grid = (unsigned)((n + kEfvThreads - 1) / kEfvThreads);
-  const size_t bytes = efv_smem_bytes<float, LV::NMU, DTHETA>(a.n_species * a.n_species, a.n_q, a.m);
-  int rc = set_smem(graph_products_kernel<GR, LV, DTHETA>, bytes);
-  if (rc != MTP_OK) return rc;
+  constexpr size_t bytes = graph_products_bytes<LV, DTHETA>();
+  static_assert(bytes <= 48 * 1024, "within the default limit of a launch");
   if (a.n_parts > 1)
     sum_shares_kernel<GR><<<(unsigned)((part + 255) / 256), 256, 0, stream>>>(mom, part, a.n_parts);
   (graph_values_kernel<GR, LV::NCOMP, V><<<grid, kEfvThreads, 0, stream>>>(mom, n, G, gld), ...);

@@ -383,6 +383,13 @@ __host__ __device__ __forceinline__ size_t efv_smem_bytes(int SS, int nq, int m)
          ((sizeof(int) * kMaxSpecies + 7) & ~size_t(7)) + sizeof(double) * kMaxWarps;
 }
 
+// EfvShared::setup_sums: xi and dE/dxi of M basis functions, the reduction area, the counts.
+template <class R, int M>
+__host__ __device__ constexpr size_t efv_sums_bytes() {
+  return ((2 * sizeof(R) * M + 15) & ~size_t(15)) + sizeof(double) * 8 * kMaxWarps +
+         ((sizeof(int) * kMaxSpecies + 15) & ~size_t(15));
+}
+
 // With DTHETA, after the areas above: on the mixed path each thread's dE/dc
 // accumulators [zj][mu][k], strided by the block size (conflict-free; as a
 // thread-private array indexed with the run-time n_q they lived in local
@@ -518,6 +525,26 @@ struct EfvShared {
     rmin = R(a.r_min);
     mid = R(0.5 * (a.r_min + a.r_cut));
     scale = R(2.0 / (a.r_cut - a.r_min));
+  }
+
+  // For a kernel without pairs: xi, and dE/dxi and the counts as zeros (FP32
+  // coefficients; M = m basis functions).  efv_block_flush without kFlushDc works on it.
+  template <int M>
+  __device__ __forceinline__ void setup_sums(const EfvArgs& a, unsigned char* raw) {
+    S = a.n_species;
+    SS = S * S;
+    nq = a.n_q;
+    m = M;
+    c = dc = acc = stage = discard = nullptr;
+    xi = reinterpret_cast<R*>(raw);
+    dxi = xi + M;
+    red = reinterpret_cast<double*>(raw + ((2 * sizeof(R) * M + 15) & ~size_t(15)));
+    cnt = reinterpret_cast<int*>(red + 8 * kMaxWarps);
+    for (int t = threadIdx.x; t < M; t += blockDim.x) {
+      xi[t] = a.xi_f[t];
+      dxi[t] = R(0);
+    }
+    for (int t = threadIdx.x; t < S; t += blockDim.x) cnt[t] = 0;
   }
 
   __device__ __forceinline__ void zero_gradients() {
