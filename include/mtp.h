@@ -157,7 +157,11 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x_dev, con
  *      64 atoms per SM: 9,728 atoms on 152 SMs) and 1 above.
  * Levels 18 and 20 run the same split kernels under every variant.
  * In a stream capture before which no call has sized the handle's scratch, the
- * FP64 path needs none (levels 18 and 20 then run as one slower kernel). */
+ * FP64 path needs none (levels 18 and 20 then run as one slower kernel).
+ * Scratch that a capture has recorded (the mixed path's, and at levels 18 and
+ * 20 the moments of both) stays allocated until mtp_free, also when a later,
+ * larger call outgrows it, so a graph can be replayed as long as the handle
+ * lives; a replay counts as use of the handle. */
 int mtp_set_efv_variant(mtp_handle* h, int32_t variant);
 /* Times both variants on this configuration (one warm-up and three timed
  * evaluations each, CUDA events on `stream`) and records the faster for its

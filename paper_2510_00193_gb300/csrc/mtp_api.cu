@@ -24,7 +24,11 @@ void set_error(const char* fmt, ...) {
 
 int DevBuf::ensure(size_t want) {
   if (want <= bytes && ptr) return MTP_OK;
-  release();
+  if (in_graph) kept.push_back(ptr);
+  else if (ptr) cudaFree(ptr);
+  ptr = nullptr;
+  bytes = 0;
+  in_graph = false;
   cudaError_t e = cudaMalloc(&ptr, want);
   if (e != cudaSuccess) {
     ptr = nullptr;
@@ -53,8 +57,11 @@ bool is_capturing(cudaStream_t s) {
 
 void DevBuf::release() {
   if (ptr) cudaFree(ptr);
+  for (void* p : kept) cudaFree(p);
+  kept.clear();
   ptr = nullptr;
   bytes = 0;
+  in_graph = false;
 }
 
 static const tables::LevelTable* find_table(int level) {
@@ -572,12 +579,14 @@ int mtp::compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const 
   pa.e_total = e_total;
   pa.dtheta = dtheta;
   pa.status = a.status;
+  const bool capturing = is_capturing(s);
   if (precision == MTP_MIXED) {
     int rc = h->xq.ensure(sizeof(long long) * 4 * (size_t)n);
     if (rc != MTP_OK) return rc;
     if ((rc = h->forces_f.ensure(sizeof(float) * 3 * (size_t)n)) != MTP_OK) return rc;
     a.xq = pa.xq = h->xq.as<long long>();
     a.forces_f = pa.forces_f = h->forces_f.as<float>();
+    if (capturing) h->xq.in_graph = h->forces_f.in_graph = true;
     inverse_rows(cell, 4294967296.0, pa.h);
   } else {
     pa.forces = forces;
@@ -596,7 +605,6 @@ int mtp::compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const 
     variant = h->tuned[precision == MTP_MIXED ? 1 : 0][bucket];
     if (variant == 0) variant = n <= team_atoms() ? 2 : 1;
   }
-  const bool capturing = is_capturing(s);
   if (h->ops->split_comps > 0 && n > 0) {
     // moment/adjoint scratch of the split kernels (levels with component
     // groups), bounded by the chunk as the paper's chunk size bounds memory;
@@ -610,6 +618,7 @@ int mtp::compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const 
       const int rc = h->mbuf.ensure(want);
       if (rc != MTP_OK) return rc;
       a.mbuf = h->mbuf.ptr;
+      if (capturing) h->mbuf.in_graph = true;
     }
   }
   // FP64 only: there the pipe's time is what a warp's longest row costs (48,546
@@ -788,6 +797,7 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
   pa.n_species = h->n_species;
   pa.dtheta = dtheta_tan;
   pa.status = t.base.status;
+  const bool capturing = is_capturing(s);
   if (precision == MTP_MIXED) {
     int rc = h->xq.ensure(sizeof(long long) * 4 * (size_t)n);
     if (rc != MTP_OK) return rc;
@@ -796,6 +806,7 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
       return MTP_ERR_ARG;
     }
     t.base.xq = pa.xq = h->xq.as<long long>();
+    if (capturing) h->xq.in_graph = true;
     inverse_rows(cell, 4294967296.0, pa.h);
     if (force_tan) MTP_TRY_CUDA(cudaMemsetAsync(force_tan, 0, sizeof(double) * 3 * (size_t)n, s));
   } else {
@@ -815,6 +826,7 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
                                                 2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double)), 0));
     if (rc != MTP_OK) return rc;
     t.base.mbuf = h->mbuf.ptr;
+    if (capturing) h->mbuf.in_graph = true;
   }
   return h->ops->tangent(t, precision, s);
 }

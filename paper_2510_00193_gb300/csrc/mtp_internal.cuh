@@ -21,10 +21,14 @@ void set_error(const char* fmt, ...);
     }                                                                                           \
   } while (0)
 
-// Device buffer that only grows.
+// Device buffer that only grows.  Memory that a stream capture has recorded is
+// not freed when the buffer grows (the graph may be replayed at any later
+// time), only by release().
 struct DevBuf {
   void* ptr = nullptr;
   size_t bytes = 0;
+  bool in_graph = false;       // a capture has recorded ptr
+  std::vector<void*> kept;     // outgrown memory that captures have recorded
   int ensure(size_t want);
   bool try_ensure(size_t want);   // for scratch that a call can do without
   void release();

@@ -1,0 +1,51 @@
+"""A captured evaluation replayed after a larger call has outgrown the handle's
+scratch: the graph's own scratch is still there and the results are the same."""
+import pytest
+
+import synth
+from tests.helpers import pot_dict
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("precision", [0, 1])   # FP64, mixed
+@pytest.mark.parametrize("name,lattice,a,kinds", [("fcc-l20-s4", "fcc", 3.6, 4), ("bcc-l16-s3", "bcc", 3.16, 3)])
+def test_replay_after_growth(precision, name, lattice, a, kinds):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_00193_gb300 import build as B
+    B.build()
+    import paper_2510_00193_gb300 as P
+    pot = P.Potential.from_dict(pot_dict(name))
+
+    def made(cells):
+        st = synth.crystal(lattice, cells, a, 0.08, kinds, 11)
+        x = torch.tensor(st.x, device="cuda")
+        return st, x, torch.tensor(st.z, dtype=torch.int32, device="cuda"), P.mtp_build_neighbors(pot, x, st.cell, st.pbc)
+
+    st, x, z, nl = made((5, 5, 5))
+    ref = P.mtp_compute_efv(pot, nl, x, z, st.cell, precision=precision)
+    ref = {k: v.clone() for k, v in ref.items() if torch.is_tensor(v)}
+    graphs = []
+    for cells in ((9, 9, 9), (12, 12, 12)):
+        out = {k: torch.zeros_like(v) for k, v in ref.items()}
+        out["dtheta"] = None
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            P.mtp_compute_efv(pot, nl, x, z, st.cell, precision=precision, out=out)
+        graphs.append((graph, out))
+        big, xb, zb, nb = made(cells)
+        other = P.Potential.from_dict(pot_dict(name))
+        for p in (pot, other):   # outgrows the scratch; the second handle takes what the first would have freed
+            P.mtp_compute_efv(p, nb, xb, zb, big.cell, precision=precision)
+    for graph, out in graphs:
+        graph.replay()
+        torch.cuda.synchronize()
+        for k, r in ref.items():
+            # the same sums in another order: FP64 1e-11; FP32 forces, about 100 additions of 6e-8 on partial
+            # sums a few times the largest force
+            tol = 1e-11 if precision == 0 or k == "e_atom" else 2e-5
+            assert (out[k] - r).abs().max() <= tol * r.abs().max(), k
+    assert P.mtp_device_status(pot) == 0
