@@ -32,6 +32,7 @@
 #include <cstring>
 
 #include "mtp_internal.cuh"
+#include "scratch_plan.h"
 
 namespace mtp {
 
@@ -179,6 +180,11 @@ __device__ __forceinline__ unsigned long long row_key(int32_t j, int32_t img) {
 }
 
 constexpr int kSearchThreads = 128;
+// Columns of found neighbours above this size (some 10 million atoms at 60
+// neighbours) are given back after the build.  Below it the list keeps them and
+// a build in place allocates nothing: giving them back costs a build of 9.8
+// million atoms 1.3 of 8.0 ms (4.2 GB).
+constexpr size_t kColumnsKept = size_t(4) << 30;
 constexpr int kRowBuffer = 1536;   // entries per warp kept in shared memory while their rows are put in order
 
 // Places the buffered entries lane, lane + 32, ... (R of them from entry
@@ -594,16 +600,31 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   int rc;
   const int64_t n1 = std::max<int64_t>(n, 1);
   const bool periodic = g.pbc[0] && g.pbc[1] && g.pbc[2];
-  if ((rc = nl->wrapped.ensure((sizeof(float4) + sizeof(int4) + sizeof(double) * 3) * n1 + 64)) != MTP_OK) return rc;
+  // Memory the build needs; where it does not fit beside the columns of found
+  // neighbours (this build's or an earlier one's), those go, and the rows are searched twice.
+  uint32_t* found = nullptr;
+  auto need = [&](DevBuf& buf, size_t bytes) {
+    int e = MTP_OK;
+    allocate_dropping([&]() { return (e = buf.ensure(bytes)) == MTP_OK; },
+                      [&]() {
+                        if (!nl->columns.ptr) return false;
+                        nl->columns.release();
+                        found = nullptr;
+                        (void)cudaGetLastError();
+                        return true;
+                      });
+    return e;
+  };
+  if ((rc = need(nl->wrapped, (sizeof(float4) + sizeof(int4) + sizeof(double) * 3) * n1 + 64)) != MTP_OK) return rc;
   float4* xw = nl->wrapped.as<float4>();
   int4* meta = reinterpret_cast<int4*>(xw + n1);
   double* sw = reinterpret_cast<double*>(meta + n1);
   unsigned long long* extent = reinterpret_cast<unsigned long long*>(sw + 3 * n1);
-  if ((rc = nl->bin_atoms.ensure((sizeof(float4) + sizeof(int4) + sizeof(int)) * n1)) != MTP_OK) return rc;
+  if ((rc = need(nl->bin_atoms, (sizeof(float4) + sizeof(int4) + sizeof(int)) * n1)) != MTP_OK) return rc;
   float4* bin_xw = nl->bin_atoms.as<float4>();
   int4* bin_meta = reinterpret_cast<int4*>(bin_xw + n1);
   int* rank = reinterpret_cast<int*>(bin_meta + n1);
-  if ((rc = nl->status.ensure(sizeof(int) * 4)) != MTP_OK) return rc;
+  if ((rc = need(nl->status, sizeof(int) * 4)) != MTP_OK) return rc;
   int* status = nl->status.as<int>();
   MTP_TRY_CUDA(cudaMemsetAsync(status, 0, 2 * sizeof(int), stream));
   unsigned long long ext_bits[6];
@@ -689,9 +710,9 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
     g.rc2_lo = lo > 0.0 ? (float)(lo * lo * (1.0 - 1e-6)) : 0.0f;
     g.rz2 = (float)(4.0 * err * err * (1.0 + 1e-6)) + 1e-30f;
   }
-  if ((rc = nl->bins.ensure(sizeof(int) * (nbins + 1))) != MTP_OK) return rc;
+  if ((rc = need(nl->bins, sizeof(int) * (nbins + 1))) != MTP_OK) return rc;
   int* bin_count = nl->bins.as<int>();
-  if ((rc = nl->bin_start.ensure(sizeof(int) * (nbins + 1))) != MTP_OK) return rc;
+  if ((rc = need(nl->bin_start, sizeof(int) * (nbins + 1))) != MTP_OK) return rc;
   int* bin_start = nl->bin_start.as<int>();
   MTP_TRY_CUDA(cudaMemsetAsync(bin_count, 0, sizeof(int) * (nbins + 1), stream));
   if (n > 0) {
@@ -710,7 +731,7 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   tmp_bytes = std::max(tmp_bytes, tmp2);
   // counts, the new offsets, the scans' temporary storage
   const size_t counts_bytes = sizeof(int) * (size_t)((n + 4) & ~int64_t(3)), offsets_bytes = sizeof(int64_t) * (n + 1);
-  if ((rc = nl->counts.ensure(counts_bytes + ((offsets_bytes + 15) & ~size_t(15)) + tmp_bytes + 64)) != MTP_OK)
+  if ((rc = need(nl->counts, counts_bytes + ((offsets_bytes + 15) & ~size_t(15)) + tmp_bytes + 64)) != MTP_OK)
     return rc;
   int* counts = nl->counts.as<int>();
   int64_t* offsets = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(counts) + counts_bytes);
@@ -728,7 +749,6 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   bool columns = n < (int64_t(1) << kSlotBits) && depth * lanes <= kOrderBuffer;
   for (int k = 0; k < 3; ++k)
     if (g.pbc[k] && g.reach[k] > g.nb[k]) columns = false;   // a bin wrap beyond +-1
-  uint32_t* found = nullptr;
   int* column_count = nullptr;
   // without room for them the rows are searched twice
   if (n > 0 && columns && nl->columns.try_ensure(sizeof(int) * (size_t)n * lanes * (depth + 1))) {
@@ -773,9 +793,10 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   // that fails leaves an empty list (its arrays are gone)
   nl->n_atoms = 0;
   nl->n_pairs = 0;
-  if ((rc = nl->offsets.ensure(offsets_bytes)) != MTP_OK) return rc;
-  if ((rc = nl->nbr_j.ensure(sizeof(int32_t) * std::max<int64_t>(total, 1))) != MTP_OK) return rc;
-  if ((rc = nl->nbr_img.ensure(sizeof(int32_t) * std::max<int64_t>(total, 1))) != MTP_OK) return rc;
+  const size_t row_bytes = sizeof(int32_t) * std::max<int64_t>(total, 1);
+  if ((rc = need(nl->offsets, offsets_bytes)) != MTP_OK || (rc = need(nl->nbr_j, row_bytes)) != MTP_OK ||
+      (rc = need(nl->nbr_img, row_bytes)) != MTP_OK)
+    return rc;
   if (total == 0) {
     MTP_TRY_CUDA(cudaMemcpyAsync(nl->offsets.ptr, offsets, offsets_bytes, cudaMemcpyDeviceToDevice, stream));
   } else if (!found || st[1]) {
@@ -785,6 +806,7 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
     order();
   }
   MTP_TRY_CUDA(cudaGetLastError());
+  if (nl->columns.bytes > kColumnsKept) nl->columns.release();   // waits for order_kernel
   for (int k = 0; k < 9; ++k) nl->cell[k] = cell[k];
   for (int k = 0; k < 3; ++k) nl->pbc[k] = g.pbc[k];
   nl->r_cut = r_cut;
