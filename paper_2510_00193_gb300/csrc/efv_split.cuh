@@ -174,7 +174,7 @@ int efv_split_launch(const EfvArgs& a, cudaStream_t stream) {
   split_moments_kernel<LV, R><<<grid, threads, b0, stream>>>(a);
   if constexpr (std::is_same<R, float>::value) {
     // the scratch of a chunked call is sized for its first, largest range
-    if (n >= kGraphAtoms) rc = graphs_launch<LV::LEVEL>(a, DTHETA, stream);
+    if (a.graphs && n >= kGraphAtoms) rc = graphs_launch<LV::LEVEL>(a, DTHETA, stream);
     else rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream);
   } else {
     rc = tile_contract_launch<LV, R, DTHETA>(a, a.dtheta, stream);

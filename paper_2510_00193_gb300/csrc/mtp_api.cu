@@ -9,6 +9,7 @@
 
 #include "mtp_internal.cuh"
 #include "mtp_tables.h"
+#include "scratch_plan.h"
 #include "tangent_kernel.cuh"
 
 namespace mtp {
@@ -607,16 +608,18 @@ int mtp::compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x, const 
   }
   if (h->ops->split_comps > 0 && n > 0) {
     // moment/adjoint scratch of the split kernels (levels with component
-    // groups), bounded by the chunk as the paper's chunk size bounds memory;
-    // a capture that no call before has sized it for takes the one fused kernel
+    // groups), bounded by the chunk as the paper's chunk size bounds memory.  A
+    // capture takes what earlier calls have sized, or the one fused kernel
     const int64_t range = std::min<int64_t>(chunk, n);
-    a.n_parts = split_parts(range, device_sms());
-    const size_t want = split_scratch_bytes(h->ops->split_comps, range, a.n_parts,
-                                            precision == MTP_MIXED ? sizeof(float) : sizeof(double),
-                                            precision == MTP_MIXED && range >= kGraphAtoms ? h->ops->split_graphs : 0);
-    if (!capturing || want <= h->mbuf.bytes) {
-      const int rc = h->mbuf.ensure(want);
-      if (rc != MTP_OK) return rc;
+    const SplitPlan plan = plan_split_scratch(
+        h->ops->split_comps, range, split_parts(range, device_sms()),
+        precision == MTP_MIXED ? sizeof(float) : sizeof(double),
+        precision == MTP_MIXED && range >= kGraphAtoms ? h->ops->split_graphs : 0,
+        [&](size_t bytes) { return capturing ? bytes <= h->mbuf.bytes : h->mbuf.try_ensure(bytes); });
+    if (!plan.ok && !capturing) return MTP_ERR_OOM;   // message from the last allocation
+    if (plan.ok) {
+      a.n_parts = plan.parts;
+      a.graphs = plan.graphs;
       a.mbuf = h->mbuf.ptr;
       if (capturing) h->mbuf.in_graph = true;
     }
@@ -821,10 +824,12 @@ extern "C" int mtp_compute_efv_tangent(mtp_handle* h, const mtp_nlist* nl, const
   t.base.atom_end = n;
   if (h->ops->split_comps > 0 && n > 0) {
     // dual moments and adjoints of the split tangent kernels: (value, tangent) pairs
-    t.base.n_parts = split_parts(n, device_sms());
-    int rc = h->mbuf.ensure(split_scratch_bytes(h->ops->split_comps, n, t.base.n_parts,
-                                                2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double)), 0));
-    if (rc != MTP_OK) return rc;
+    const SplitPlan plan = plan_split_scratch(
+        h->ops->split_comps, n, split_parts(n, device_sms()),
+        2 * (precision == MTP_MIXED ? sizeof(float) : sizeof(double)), 0,
+        [&](size_t bytes) { return h->mbuf.try_ensure(bytes); });
+    if (!plan.ok) return MTP_ERR_OOM;   // message from the last allocation
+    t.base.n_parts = plan.parts;
     t.base.mbuf = h->mbuf.ptr;
     if (capturing) h->mbuf.in_graph = true;
   }

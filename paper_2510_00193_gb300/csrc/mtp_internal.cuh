@@ -87,6 +87,7 @@ struct EfvArgs {
   void* mbuf;               // levels with component groups: scratch of the split kernels in the working precision,
                             // n_parts buffers of partial moments, then the adjoints (nullptr: one fused kernel)
   int n_parts;              // shares into which the split kernels cut each atom's neighbours
+  int graphs;               // mbuf has room for the graph values (straight-line contraction)
   const int32_t* order;     // kernels with one thread per atom: thread t of the range takes atom order[t] (nullptr: t)
 };
 
@@ -153,13 +154,6 @@ inline int split_parts(int64_t n, int sms) {
 }
 // Row length of the graph values G[graph][atom]: whole blocks of 128 threads.
 __host__ __device__ inline int64_t graph_padded(int64_t n) { return (n + 127) / 128 * 128; }
-// Bytes of EfvArgs::mbuf for n atoms: the shares' moments and the adjoints, with
-// the atoms rounded up to whole tiles of 8, then the values and adjoints of the
-// graphs (the straight-line contraction; graphs = 0 without it).
-inline size_t split_scratch_bytes(int comps, int64_t n, int parts, size_t entry, int graphs) {
-  return entry * ((size_t)comps * (size_t)((n + 7) / 8 * 8) * (size_t)(parts + 1) +
-                  2 * (size_t)graphs * (size_t)graph_padded(n));
-}
 // From this many atoms of a range on, the mixed path of the levels with
 // component groups contracts with the straight-line graph kernels.
 constexpr int64_t kGraphAtoms = 4096;

@@ -49,3 +49,34 @@ def test_replay_after_growth(precision, name, lattice, a, kinds):
             tol = 1e-11 if precision == 0 or k == "e_atom" else 2e-5
             assert (out[k] - r).abs().max() <= tol * r.abs().max(), k
     assert P.mtp_device_status(pot) == 0
+
+
+def test_capture_with_room_for_the_tile_program_only():
+    """4,200 atoms at level 20, mixed, captured when earlier calls have sized the scratch for the moments but
+    not for the graph values: the tile program runs on them, against the graph kernels of an ordinary call."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_00193_gb300 import build as B
+    B.build()
+    import paper_2510_00193_gb300 as P
+    st = synth.crystal("fcc", (7, 10, 15), 3.6, 0.1, 4, 11)
+    assert st.n == 4200
+    x, z = torch.tensor(st.x, device="cuda"), torch.tensor(st.z, dtype=torch.int32, device="cuda")
+    pot, other = (P.Potential.from_dict(pot_dict("fcc-l20-s4")) for _ in range(2))
+    nl = P.mtp_build_neighbors(pot, x, st.cell, st.pbc)
+    ref = P.mtp_compute_efv(other, nl, x, z, st.cell, dtheta=True)
+    exact = P.mtp_compute_efv(other, nl, x, z, st.cell, precision=P.MTP_FP64, dtheta=True)
+    out = {k: torch.zeros_like(v) for k, v in ref.items()}
+    P.mtp_compute_efv(pot, nl, x, z, st.cell, chunk_atoms=1000)                           # the mixed path's own scratch
+    P.mtp_compute_efv(pot, nl, x, z, st.cell, precision=P.MTP_FP64, chunk_atoms=2520)     # between the two sizes
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        P.mtp_compute_efv(pot, nl, x, z, st.cell, dtheta=True, out=out)
+    graph.replay()
+    torch.cuda.synchronize()
+    for k in ("e_atom", "forces", "virial", "dtheta"):
+        r = exact[k]
+        off = [float((o[k] - r).norm() / r.norm()) for o in (out, ref)]
+        assert off[0] <= 2e-5 and off[1] <= 2e-5, (k, off)   # FP32 sums of terms good to ~1e-6
+    assert P.mtp_device_status(pot) == 0

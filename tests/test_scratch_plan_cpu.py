@@ -34,3 +34,23 @@ def test_allocate_dropping(tmp_path, room, held, expect):
                                    [&] { if (!held) return false; held = 0; return true; });
   std::printf("%%d %%ld", (int)ok, held);""" % (room, held))
     assert out == expect
+
+
+@pytest.mark.parametrize("room,n,parts,graphs,expect", [
+    # 295 components and 159 graphs in FP32: 1,180 B per atom and buffer, 1,272 B of graph values
+    (10 ** 9, 4200, 4, 159, "1 4 1"),                       # everything fits
+    (5 * 1180 * 4200 + 2 * 4 * 159 * 4224, 4200, 4, 159, "1 4 1"),       # to the byte
+    (5 * 1180 * 4200 + 2 * 4 * 159 * 4224 - 1, 4200, 4, 159, "1 4 0"),   # not the graph values
+    (5 * 1180 * 4200, 4200, 4, 159, "1 4 0"),
+    (5 * 1180 * 4200 - 1, 4200, 4, 159, "1 1 0"),           # one share of the neighbours
+    (2 * 1180 * 4200, 4200, 4, 159, "1 1 0"),
+    (2 * 1180 * 4200 - 1, 4200, 4, 159, "0 0 0"),
+    (2 * 1180 * 4200 - 1, 4200, 1, 0, "0 0 0"),
+    (2 * 1180 * 8, 1, 1, 0, "1 1 0"),                       # one atom: a whole tile of 8
+    (2 * 1180 * 8 - 1, 1, 1, 0, "0 0 0"),
+])
+def test_split_plan(tmp_path, room, n, parts, graphs, expect):
+    out = compiled_run(tmp_path, """
+  const auto p = mtp::plan_split_scratch(295, %d, %d, sizeof(float), %d, [](size_t b) { return b <= (size_t)%dll; });
+  std::printf("%%d %%d %%d", (int)p.ok, p.parts, (int)p.graphs);""" % (n, parts, graphs, room))
+    assert out == expect
