@@ -304,12 +304,14 @@ __device__ __forceinline__ void fill_coefs(C* dst, const SRC* __restrict__ src, 
 // pair vector comes from the FP64 positions and the distance, the radial
 // functions, their derivatives and (with WANT_Q) the basis values Q_k are
 // evaluated in FP64 with the FP64 coefficients, then rounded to FP32 once.
-// `cell` holds the FP64 rows of the configuration's cell.  Used by the
-// level-18/20 split kernels; the fused kernels keep FP32 for every pair
-// (an inlined FP64 branch cost them 20% at level 16, where no pair of the
-// 1,024,000-atom workload comes closer than R_min, and 3x on the random
-// gases, where a third of the warp iterations hold a pair between the 1.9 A
-// minimum separation and R_min = 2 A and GB300's FP64 pipe serialises them).
+// `cell` holds the FP64 rows of the configuration's cell.  Used by both sweeps
+// of the level-18/20 split kernels, and with dE/dtheta by the second sweep of
+// the one-configuration kernels.  Those keep FP32 for every pair otherwise (an
+// inlined FP64 branch cost them 20% at level 16, where no pair of the
+// 1,024,000-atom workload comes closer than R_min), and so does the batch
+// kernel (3x on the random gases, where a third of the warp iterations hold a
+// pair between the 1.9 A minimum separation and R_min = 2 A and GB300's FP64
+// pipe serialises them).
 template <int NMU, bool DERIV, bool WANT_Q>
 __device__ __forceinline__ void close_pair_fp64(const EfvArgs& a, const double* cell, int32_t ci, int32_t j,
                                                 int32_t img, int zi, int zj, float& dx, float& dy, float& dz,
@@ -824,8 +826,10 @@ __device__ __forceinline__ void adjoint_pair(const EfvArgs& a, const EfvShared<R
 // dE/dc terms Q_k(r) S_mu into acc (own_acc) or the shared accumulators.
 // CLOSE64 as in moment_sweep; without it and without DTHETA the sweep is
 // software-pipelined like moment_sweep (with DTHETA the next pair's Q_k
-// values would stay live as well, which measured slower).
-template <class LV, class R, bool DTHETA, int G, bool CLOSE64 = false, int NQ = 0, class Acc>
+// values would stay live as well, which measured slower).  CELL64: cell64 is
+// there, and the FP32 sweep that is not pipelined evaluates pairs closer than
+// R_min in FP64; without it cell64 is not read.
+template <class LV, class R, bool DTHETA, int G, bool CLOSE64 = false, int NQ = 0, bool CELL64 = true, class Acc>
 __device__ __forceinline__ void adjoint_sweep(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm,
                                               const PairGeom<R>& geom, const double* cell64, int zi, int64_t beg,
                                               int64_t end,
@@ -869,7 +873,7 @@ __device__ __forceinline__ void adjoint_sweep(const EfvArgs& a, const EfvShared<
         if (close != second) continue;
       }
       R f[NMU], df[NMU], q[DTHETA ? kMaxQ : 1];
-      if constexpr (std::is_same<R, float>::value) {
+      if constexpr (CELL64 && std::is_same<R, float>::value) {
         if (r < sm.rmin)
           close_pair_fp64<NMU, true, DTHETA>(a, cell64, geom.ci, j, img, zi, zj, dx, dy, dz, rinv, f, df, q);
         else
@@ -910,7 +914,7 @@ __device__ __forceinline__ R contract_atom(MV M, const typename ScalarOf<R>::T* 
     return LV::template contract<R, WANT_B, MV, BV>(M, xi, D, B);
 }
 
-template <class LV, class R, bool DTHETA, bool PHASE_SYNC = false, int NQ = 0, bool DAG = false>
+template <class LV, class R, bool DTHETA, bool PHASE_SYNC = false, int NQ = 0, bool DAG = false, bool CELL64 = true>
 __device__ __forceinline__ void efv_atom(const EfvArgs& a, const EfvShared<R, LV::NMU, DTHETA>& sm, int64_t i,
                                          bool active, const R* cell, const double* cell64, double& e_i, R* w) {
   constexpr int NMU = LV::NMU;
@@ -984,19 +988,20 @@ __device__ __forceinline__ void efv_atom(const EfvArgs& a, const EfvShared<R, LV
     for (int t = 0; t < sm.S * NMU * sm.nq; ++t) acc[t] = R(0);
   }
   if constexpr (LV::NGROUPS == 1) {
-    adjoint_sweep<LV, R, DTHETA, -1, false, NQ>(a, sm, geom, cell64, zi, beg, end, D, fx, fy, fz, w, acc, own_acc);
+    adjoint_sweep<LV, R, DTHETA, -1, false, NQ, CELL64>(a, sm, geom, cell64, zi, beg, end, D, fx, fy, fz, w, acc,
+                                                        own_acc);
   } else {
     {
       R Dg[LV::NCOMP];
       LV::template load_group<0, R>(D, 1, Dg);
-      adjoint_sweep<LV, R, DTHETA, 0>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
-                                          GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
+      adjoint_sweep<LV, R, DTHETA, 0, false, 0, CELL64>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
+                                                        GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
     }
     {
       R Dg[LV::NCOMP];
       LV::template load_group<1, R>(D, 1, Dg);
-      adjoint_sweep<LV, R, DTHETA, 1>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
-                                          GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
+      adjoint_sweep<LV, R, DTHETA, 1, false, 0, CELL64>(a, sm, geom, cell64, zi, beg, end, Dg, fx, fy, fz, w,
+                                                        GroupAccView<R>(acc, NMU * sm.nq, 0), own_acc);
     }
   }
   if (own_acc) add_warp_gradients(sm, 0, NMU * sm.nq, zi, active, [&](int t) { return acc[t]; });
