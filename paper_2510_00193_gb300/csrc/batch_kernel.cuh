@@ -72,13 +72,8 @@ int batch_launch_typed(const BatchArgs& b, int threads, cudaStream_t stream) {
   if constexpr (LV::NGROUPS == 1) {
     if (b.base.n_q == kFixedQ) kern = batch_kernel<LV, R, DTHETA, kFixedQ>;
   }
-  if (bytes > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-      set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-  }
+  const int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
   int per_sm = 0, sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

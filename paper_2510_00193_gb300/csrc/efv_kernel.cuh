@@ -1101,6 +1101,7 @@ int set_smem(K kern, size_t bytes) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) {
       set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+      (void)cudaGetLastError();   // reported; the next call's check of its launches must not see it
       return MTP_ERR_CUDA;
     }
   }

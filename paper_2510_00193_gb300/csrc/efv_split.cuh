@@ -208,13 +208,8 @@ int efv_launch_typed(const EfvArgs& a, cudaStream_t stream) {
   if constexpr (LV::NGROUPS == 1) {
     if (a.n_q == kFixedQ) kern = efv_kernel<LV, R, DTHETA, kFixedQ>;
   }
-  if (bytes > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-      set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-  }
+  const int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
   kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -90,13 +90,8 @@ int basis_rows_launch(const EfvArgs& a, const int32_t* list, int64_t n_rows, dou
   if constexpr (LV::NGROUPS == 1) {
     if (a.n_q == kFixedQ) kern = basis_rows_kernel<LV, kFixedQ>;
   }
-  if (bytes > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-      set_error("cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-  }
+  const int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
   const int threads = fp64_threads(n_rows, 1);
   kern<<<(unsigned)((n_rows + threads - 1) / threads), threads, bytes, stream>>>(a, list, n_rows, rows, ld, bsum);
   cudaError_t e = cudaGetLastError();

@@ -35,17 +35,14 @@ int DevBuf::ensure(size_t want) {
     ptr = nullptr;
     bytes = 0;
     set_error("cudaMalloc(%zu bytes): %s", want, cudaGetErrorString(e));
+    (void)cudaGetLastError();   // reported; the next call's check of its launches must not see it
     return MTP_ERR_OOM;
   }
   bytes = want;
   return MTP_OK;
 }
 
-bool DevBuf::try_ensure(size_t want) {
-  if (ensure(want) == MTP_OK) return true;
-  (void)cudaGetLastError();
-  return false;
-}
+bool DevBuf::try_ensure(size_t want) { return ensure(want) == MTP_OK; }
 
 bool is_capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;

@@ -610,7 +610,6 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
                         if (!nl->columns.ptr) return false;
                         nl->columns.release();
                         found = nullptr;
-                        (void)cudaGetLastError();
                         return true;
                       });
     return e;
