@@ -137,11 +137,12 @@ __global__ void md_filter_kernel(const int* __restrict__ skip, const double* __r
                                  int32_t* __restrict__ tmp_j, int32_t* __restrict__ tmp_img) {
   const int lane = threadIdx.x & 31;
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (skip && __ldg(skip) != 0) return;
-  if (i == n && lane == 0) counts[n] = 0;
+  const bool stay = skip && __ldg(skip) != 0;
+  if (i == n && lane == 0 && !stay) counts[n] = 0;
   if (i >= n) return;   // warp-uniform
   const float4 pi = xf[i];
   const int64_t beg = off[i], end = off[i + 1];
+  if (stay) return;     // read together with the row's bounds: one latency, not two
   int64_t w = beg;
   for (int64_t k0 = beg; k0 < end; k0 += 32) {
     const int64_t k = k0 + lane;
@@ -184,10 +185,7 @@ __global__ void md_kick_kernel(double* __restrict__ v, const double* __restrict_
                                MdMass mm, double dt, int64_t n, double* __restrict__ e_kin, int* __restrict__ spec,
                                int* __restrict__ status) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && spec && *spec != 0) {
-    atomicCAS(status, 0, *spec);
-    *spec = 0;
-  }
+  const int err = i == 0 && spec ? *spec : 0;
   double ke = 0.0;
   if (i < n) {
     const int zi = min(max(z[i], 0), kMaxSpecies - 1);   // species checked by the force pass
@@ -200,6 +198,10 @@ __global__ void md_kick_kernel(double* __restrict__ v, const double* __restrict_
       vv += vc * vc;
     }
     ke = mm.half_m[zi] * vv;
+  }
+  if (err != 0) {
+    atomicCAS(status, 0, err);
+    *spec = 0;
   }
   if (!e_kin) return;
 #pragma unroll

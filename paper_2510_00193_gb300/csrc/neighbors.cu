@@ -409,10 +409,11 @@ __global__ void __launch_bounds__(kSearchThreads) count_kernel(const SearchArgs 
 
 // List rows from what count_kernel found: a block gathers the columns of its
 // atoms and forms (j, image) of every entry, then one warp per atom orders the
-// row and writes it, and its offset.  May run before the host knows the pair
-// count or whether the build failed: does nothing if the pairs do not fit in
-// `capacity`, a column ran over or an error is recorded, so that a list built
-// in place keeps its offsets and rows until they are replaced together.
+// row and writes it; the blocks also write the offsets.  May run before the
+// host knows the pair count or whether the build failed: does nothing if the
+// pairs do not fit in `capacity`, a column ran over or an error is recorded, so
+// that a list built in place keeps its offsets and rows until they are replaced
+// together.
 constexpr int kOrderWarps = 8;
 constexpr int kOrderBuffer = 512;   // entries of one row
 template <int LANES>
@@ -428,9 +429,11 @@ __global__ void __launch_bounds__(32 * kOrderWarps) order_kernel(const SearchArg
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t total = __ldg(offsets + s.n);
   if (total > capacity || __ldg(s.status) != 0 || __ldg(s.status + 1) != 0) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) out_offsets[s.n] = total;
   const int64_t slot0 = (int64_t)blockIdx.x * kOrderWarps, cols = s.n * LANES;
   const int atoms = (int)min((int64_t)kOrderWarps, s.n - slot0);
+  // the block's share of the offsets, by atom index (one sector; by the atoms of its slots: eight)
+  if ((int)threadIdx.x < atoms) out_offsets[slot0 + threadIdx.x] = __ldg(offsets + slot0 + threadIdx.x);
+  if (blockIdx.x == 0 && threadIdx.x == 0) out_offsets[s.n] = total;
   constexpr int width = kOrderWarps * LANES;
   // the block's columns side by side: a sector of `found` holds the same entry of 8 columns
   const int c = threadIdx.x % width;
@@ -462,9 +465,7 @@ __global__ void __launch_bounds__(32 * kOrderWarps) order_kernel(const SearchArg
   if (lane < ((4 - (cnt & 3)) & 3)) buf[warp][0][cnt + lane] = 0xFFFFFFFFu;
   __syncthreads();
   if (warp >= atoms) return;
-  const int atom = __ldg(s.bin_meta + slot0 + warp).w;
-  const int64_t base = __ldg(offsets + atom);
-  if (lane == 0) out_offsets[atom] = base;
+  const int64_t base = __ldg(offsets + __ldg(s.bin_meta + slot0 + warp).w);
   if (g.unique) place_row_any<true>(buf[warp][0], buf[warp][1], cnt, lane, out_j + base, out_img + base);
   else place_row_any<false>(buf[warp][0], buf[warp][1], cnt, lane, out_j + base, out_img + base);
 }
@@ -482,6 +483,7 @@ __global__ void __launch_bounds__(kSearchThreads) fill_kernel(const SearchArgs s
   const int64_t slot = (int64_t)blockIdx.x * kSearchThreads + threadIdx.x;
   const int64_t total = __ldg(offsets + s.n);
   if (total > capacity) return;
+  if (slot < s.n) out_offsets[slot] = __ldg(offsets + slot);
   if (slot == 0) out_offsets[s.n] = total;
   uint32_t* bj = buf[warp][0];
   uint32_t* bi = buf[warp][1];
@@ -494,7 +496,6 @@ __global__ void __launch_bounds__(kSearchThreads) fill_kernel(const SearchArgs s
     pw = __ldg(s.bin_xw + slot);
     mi = __ldg(s.bin_meta + slot);
     base = __ldg(offsets + mi.w);
-    out_offsets[mi.w] = base;
     const int64_t c64 = __ldg(offsets + mi.w + 1) - base;
     cnt = (int)c64;
     if (cnt > kRowBuffer) {
