@@ -170,7 +170,8 @@ int mtp_compute_efv(mtp_handle* h, const mtp_nlist* nl, const double* x_dev, con
 int mtp_set_efv_variant(mtp_handle* h, int32_t variant);
 /* Times both variants on this configuration (one warm-up and three timed
  * evaluations each, CUDA events on `stream`) and records the faster for its
- * precision and power-of-two size class in the handle.  chosen (HOST,
+ * precision and power-of-two size class in the handle (levels 18 and 20: the
+ * same kernels twice).  chosen (HOST,
  * nullable): 1 or 2; ms (HOST [2], nullable): mean ms per evaluation of
  * each.  Allocates scratch outputs for
  * the call; synchronises `stream`. */

@@ -265,7 +265,7 @@ def mtp_compute_efv(potential: Potential, nlist: NeighborList, x, z, cell, preci
     return out
 
 
-EFV_AUTO, EFV_THREAD_PER_ATOM, EFV_WARP_PER_ATOM = 0, 1, 2
+EFV_AUTO, EFV_THREAD_PER_ATOM, EFV_WARP_PER_ATOM = 0, 1, 2   # 2: warps that share atoms
 
 
 def mtp_set_efv_variant(potential: Potential, variant: int) -> None:

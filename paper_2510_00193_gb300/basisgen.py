@@ -1051,7 +1051,7 @@ class GraphCode:
         key, rank = self.lv.dag.nodes[n]
         return n_sym(rank) * n_sym(self.lv.dag.rank(key[2])) if key[0] == "C" else 0
 
-    def comps(self, nodes, with_sources=True):
+    def comps(self, nodes):
         """Moment components that the nodes read (and the swept ones they are formed from)."""
         lv, used = self.lv, set()
         for n in nodes:

@@ -12,10 +12,13 @@
 //
 // Measured, level 20, 108,000 atoms, mixed: contraction 3.60 ms (tile program)
 // -> 0.59 ms (values 104, products 48, adjoints 435 us); the whole evaluation
-// 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays (whole evaluation:
-// 2,016 atoms 0.131 ms, 4,000 atoms 0.205; these kernels 0.231 at 4,400 and 0.260
-// at 5,324, where the tile program would take about 0.225 and 0.27): they would
-// run on less than half a wave each.
+// 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays: these kernels would
+// run on less than half a wave each.  Tile program / these, whole call (us):
+//   level 18:  2,048 atoms 87/109, 2,916 111/119, 4,000 129/119, 5,808 170/143, 8,788 217/141
+//   level 20:  2,048 127/213, 4,000 202/222, 4,840 208/227, 5,808 271/255, 8,788 374/266
+// with dE/dtheta at level 20: 4,000 239/271, 4,840 241/271, 5,808 328/327.  One
+// line for both levels: each loses up to a tenth close to it, level 18 below,
+// level 20 above.
 // Bound: instruction issue at 8 warps per SM (255 registers); the groups that
 // touch many components (281 of 295 in one) also wait for their D columns.
 #pragma once
@@ -27,8 +30,7 @@
 namespace mtp {
 
 // Partial moments of the neighbour sweep's shares added into the first.
-template <class GR>
-__global__ void __launch_bounds__(256) sum_shares_kernel(float* __restrict__ mom, int64_t part, int n_parts) {
+static __global__ void __launch_bounds__(256) sum_shares_kernel(float* __restrict__ mom, int64_t part, int n_parts) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= part) return;
   float s = mom[k];
@@ -132,7 +134,7 @@ int graphs_launch_seq(const EfvArgs& a, cudaStream_t stream, std::integer_sequen
   constexpr size_t bytes = graph_products_bytes<LV, DTHETA>();
   static_assert(bytes <= 48 * 1024, "within the default limit of a launch");
   if (a.n_parts > 1)
-    sum_shares_kernel<GR><<<(unsigned)((part + 255) / 256), 256, 0, stream>>>(mom, part, a.n_parts);
+    sum_shares_kernel<<<(unsigned)((part + 255) / 256), 256, 0, stream>>>(mom, part, a.n_parts);
   (graph_values_kernel<GR, LV::NCOMP, V><<<grid, kEfvThreads, 0, stream>>>(mom, n, G, gld), ...);
   graph_products_kernel<GR, LV, DTHETA><<<grid, kEfvThreads, bytes, stream>>>(a, G, GB, gld);
   (graph_adjoint_kernel<GR, LV::NCOMP, A><<<grid, kEfvThreads, 0, stream>>>(mom, n, GB, gld, D), ...);

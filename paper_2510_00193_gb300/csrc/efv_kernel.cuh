@@ -423,8 +423,6 @@ __device__ __forceinline__ uint32_t dynamic_smem_size() {
   return r;
 }
 
-// Accumulator array with a stride: thread-private (stride 1) or a thread's
-// column of the shared [entry][thread] array.
 // Basis-value sink of the contraction: the warp's sum of basis value a
 // (lanes without an atom add zero) is added to the block's dE/dxi slot.
 template <class R> struct WarpBasisSink {
@@ -451,7 +449,9 @@ template <class R> struct DiscardBasisSink {
   }
 };
 
-// vec: four consecutive entries side by side ([entry / 4][thread][4]).
+// Accumulator array with a stride: thread-private (stride 1) or a thread's
+// column of the shared [entry][thread] array; vec: four consecutive entries side
+// by side ([entry / 4][thread][4]).
 template <class R> struct AccView {
   R* p;
   int stride;

@@ -23,8 +23,8 @@
 // 137 / 464, 3,432 272 / 959, 8,704 558 / 941, 16,000 1,081 / 953.  With 32 atoms
 // per block always, FP64 at 128 atoms took 269 us: four SMs' FP64 pipes.
 // The form before (one warp per atom, every lane running the whole contraction)
-// took 59 us at 2,000 atoms.  Bound: instruction fetch (ncu: 3.1 of 6.5 stalled
-// warps per issue wait for instructions at 2,000 atoms).
+// took 59 us at 2,000 atoms.  Bound: instruction fetch (ncu: 4.4 of 8.3 warps per
+// issue wait for instructions at 2,000 atoms).
 // Levels with component groups (18 and 20) run the split kernels at every size.
 #pragma once
 #include "efv_kernel.cuh"

@@ -199,7 +199,11 @@ using namespace mtp;
 
 namespace mtp {
 // Up to this many atoms an untuned handle takes the team kernel: one wave of
-// its blocks (32 atoms, two blocks per SM); times on both sides stand at the kernel.
+// its blocks (32 atoms, two blocks per SM).  One thread per atom / team kernel
+// below that line, whole calls (us), at levels 2, 8, 12, 14 and 16: 9,248 atoms mixed
+// 31/25, 33/27, 35/28, 39/32, 50/40, mixed with dE/dtheta 49/29 to 105/60, FP64
+// 182/96 to 888/580.  Just above it (9,792) the mixed call without dE/dtheta
+// turns at the higher levels: 31/25, 33/27, 35/30, 39/42, 50/58.
 static int64_t team_atoms() { return 64 * (int64_t)device_sms(); }
 }  // namespace mtp
 

@@ -155,7 +155,8 @@ inline int split_parts(int64_t n, int sms) {
 // Row length of the graph values G[graph][atom]: whole blocks of 128 threads.
 __host__ __device__ inline int64_t graph_padded(int64_t n) { return (n + 127) / 128 * 128; }
 // From this many atoms of a range on, the mixed path of the levels with
-// component groups contracts with the straight-line graph kernels.
+// component groups contracts with the straight-line graph kernels (times on both
+// sides stand there).
 constexpr int64_t kGraphAtoms = 4096;
 // The straight-line contraction of level LEVEL (generated).
 template <int LEVEL> int graphs_launch(const EfvArgs& a, bool want_dtheta, cudaStream_t s);

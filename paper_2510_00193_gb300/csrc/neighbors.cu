@@ -12,8 +12,8 @@
 // each operation separately rounded (explicit _rn intrinsics, no contraction),
 // wherever an FP32 estimate with a proven error bound cannot decide it.
 //
-// Measured (build of 500,000 BCC atoms at R_cut 5 A: 1.31 -> 0.58 ms; list and
-// level-16 evaluation of 14,858 atoms 0.434 -> 0.245 ms) against two searches
+// Measured (build of 500,000 BCC atoms at R_cut 5 A: 1.31 -> 0.54 ms; list and
+// level-16 evaluation of 14,858 atoms 0.434 -> 0.214 ms) against two searches
 // by one thread per atom that handled each found neighbour inside the candidate
 // loop, and a sorting network over 64-bit keys.  What it rests on:
 //   - one search: count_kernel leaves what it finds, order_kernel makes rows;
@@ -742,6 +742,10 @@ int build_neighbors(mtp_nlist* nl, const double* x, int64_t n, const double* cel
   // Columns of found neighbours.  Threads per atom: more for small systems,
   // whose search is a chain of dependent loads on too few threads.  Entries per
   // column: half more than the mean density gives, and some.
+  // BCC at R_cut 5 A, build in place with 1 / 2 / 4 threads (us): 2,000 atoms
+  // 129 / 115 / 111, 16,000 145 / 133 / 121, 31,250 153 / 141 / 139, 50,460
+  // 171 / 158 / 162, 98,568 200 / 200 / 215, 203,136 282 / 292 / 337; hence 4 up to
+  // 50,000 atoms and 2 up to 100,000 (some 1,300 threads per SM).
   int lanes = 1;
   while (lanes < 4 && 2 * n * lanes <= 200000) lanes *= 2;
   const double mean = (double)n / std::fabs(det) * 4.1887902047863905 * r_cut * r_cut * r_cut;

@@ -17,11 +17,12 @@
 // now take 1.41), one FP64 force-matching step of 4,000 atoms 41.3 -> 5.8 ms.
 //
 // Bound: on the FP32 path latency, 23 phases of which 8 hold a single slab
-// (about 800 cycles each of a tile's 70,000), and the shared-memory reads
+// (about 800 cycles each of a tile's 70,000; 14 of 23 warps per issue wait at
+// barriers), and the shared-memory reads
 // between them (two 16-byte reads per term and thread; the order of the terms
 // puts the four rows that a quarter warp reads in different bank groups where
 // it can: 24.8 instead of 31.0 thousand wavefronts per tile); on the FP64 path
-// its pipe, at 50 to 60% of its rate in the large phases.
+// its pipe, 57% busy over the whole dual kernel.
 #pragma once
 #include <type_traits>
 
