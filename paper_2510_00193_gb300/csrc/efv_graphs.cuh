@@ -15,7 +15,7 @@
 // 4.22 -> 1.41 ms.  Below 4,096 atoms the tile program stays: these kernels would
 // run on less than half a wave each.  Tile program / these, whole call (us):
 //   level 18:  2,048 atoms 87/109, 2,916 111/119, 4,000 129/119, 5,808 170/143, 8,788 217/141
-//   level 20:  2,048 127/213, 4,000 202/222, 4,840 208/227, 5,808 271/255, 8,788 374/266
+//   level 20:  2,048 117 to 127/213, 4,000 202/222, 4,840 208/227, 5,808 271/255, 8,788 374/266
 // with dE/dtheta at level 20: 4,000 239/271, 4,840 241/271, 5,808 328/327.  One
 // line for both levels: each loses up to a tenth close to it, level 18 below,
 // level 20 above.

@@ -25,8 +25,14 @@ void set_error(const char* fmt, ...) {
 
 int DevBuf::ensure(size_t want) {
   if (want <= bytes && ptr) return MTP_OK;
-  if (in_graph) kept.push_back(ptr);
-  else if (ptr) cudaFree(ptr);
+  if (in_graph) {
+    try {
+      kept.push_back(ptr);
+    } catch (...) {   // no host memory for the note: the graph's memory is never freed
+    }
+  } else if (ptr) {
+    cudaFree(ptr);
+  }
   ptr = nullptr;
   bytes = 0;
   in_graph = false;

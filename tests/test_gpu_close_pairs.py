@@ -11,13 +11,18 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("level", [8, 16, 20])
-def test_close_pairs(level):
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("level", [8, 16, 20])
+def test_close_pairs(P, level):
     if level == 16:
         pot = P.Potential.from_dict(pot_dict("gas-l16-s2"))
     else:

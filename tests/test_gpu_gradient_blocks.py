@@ -10,14 +10,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("level,kinds,n_q", [(8, 1, 8), (12, 3, 8), (12, 4, 5), (8, 5, 8), (16, 2, 8), (16, 4, 16)])
-@pytest.mark.parametrize("cells", [(2, 3, 2), (5, 4, 7)])
-def test_blocks(level, kinds, n_q, cells):
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("level,kinds,n_q", [(8, 1, 8), (12, 3, 8), (12, 4, 5), (8, 5, 8), (16, 2, 8), (16, 4, 16)])
+@pytest.mark.parametrize("cells", [(2, 3, 2), (5, 4, 7)])
+def test_blocks(P, level, kinds, n_q, cells):
     info = P.mtp_basis_info(level)
     raw = synth.raw_potential(level, kinds, n_q, 2.0, 5.0, info["n_mu"], info["m"], 31)
     pot = P.Potential(level, kinds, n_q, 2.0, 5.0, raw.species_energy, 0.05 * raw.radial, raw.xi_raw)

@@ -9,14 +9,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("precision", [0, 1])   # FP64, mixed
-@pytest.mark.parametrize("name,lattice,a,kinds", [("fcc-l20-s4", "fcc", 3.6, 4), ("bcc-l16-s3", "bcc", 3.16, 3)])
-def test_replay_after_growth(precision, name, lattice, a, kinds):
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("precision", [0, 1])   # FP64, mixed
+@pytest.mark.parametrize("name,lattice,a,kinds", [("fcc-l20-s4", "fcc", 3.6, 4), ("bcc-l16-s3", "bcc", 3.16, 3)])
+def test_replay_after_growth(P, precision, name, lattice, a, kinds):
     pot = P.Potential.from_dict(pot_dict(name))
 
     def made(cells):
@@ -51,14 +56,9 @@ def test_replay_after_growth(precision, name, lattice, a, kinds):
     assert P.mtp_device_status(pot) == 0
 
 
-def test_capture_with_room_for_the_tile_program_only():
+def test_capture_with_room_for_the_tile_program_only(P):
     """4,200 atoms at level 20, mixed, captured when earlier calls have sized the scratch for the moments but
     not for the graph values: the tile program runs on them, against the graph kernels of an ordinary call."""
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2510_00193_gb300 import build as B
-    B.build()
-    import paper_2510_00193_gb300 as P
     st = synth.crystal("fcc", (7, 10, 15), 3.6, 0.1, 4, 11)
     assert st.n == 4200
     x, z = torch.tensor(st.x, device="cuda"), torch.tensor(st.z, dtype=torch.int32, device="cuda")

@@ -10,14 +10,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("steps_before", [0, 3])
-def test_list_after_a_failed_rebuild(precision, steps_before):
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("steps_before", [0, 3])
+def test_list_after_a_failed_rebuild(P, precision, steps_before):
     pot = P.Potential.from_dict(pot_dict("bcc-l16-s3"))
     st = synth.crystal("bcc", (6, 5, 7), 3.16, 0.08, 3, 2)
     masses, dt = [183.84, 95.95, 50.94], 1e-3
@@ -47,11 +52,8 @@ def test_list_after_a_failed_rebuild(precision, steps_before):
     assert md.rebuilds() == builds + 1
 
 
-def test_errors_of_checked_steps_are_reported():
+def test_errors_of_checked_steps_are_reported(P):
     """The status of an evaluation queued before the displacement flag is read reaches the handle."""
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    import paper_2510_00193_gb300 as P
     pot = P.Potential.from_dict(pot_dict("bcc-l16-s3"))
     st = synth.crystal("bcc", (4, 4, 4), 3.16, 0.08, 3, 2)
     x = torch.tensor(st.x, device="cuda")

@@ -11,14 +11,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("level", [18, 20])
-@pytest.mark.parametrize("kinds,n_q", [(8, 10), (9, 8), (6, 16), (16, 16)])
-def test_many_species(level, kinds, n_q):
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("level", [18, 20])
+@pytest.mark.parametrize("kinds,n_q", [(8, 10), (9, 8), (6, 16), (16, 16)])
+def test_many_species(P, level, kinds, n_q):
     info = P.mtp_basis_info(level)
     raw = synth.raw_potential(level, kinds, n_q, 2.0, 5.0, info["n_mu"], info["m"], 18)
     pot = P.Potential(level, kinds, n_q, 2.0, 5.0, raw.species_energy, 0.02 * raw.radial, raw.xi_raw)

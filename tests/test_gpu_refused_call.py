@@ -7,14 +7,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("call", ["efv", "batch"])
-def test_valid_call_after_a_refused_one(call):
-    """16 species with n_q = 16: the FP64 coefficients and dE/dc sums exceed a block's shared memory."""
+@pytest.fixture(scope="module")
+def P():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2510_00193_gb300 import build as B
     B.build()
     import paper_2510_00193_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("call", ["efv", "batch"])
+def test_valid_call_after_a_refused_one(P, call):
+    """16 species with n_q = 16: the FP64 coefficients and dE/dc sums exceed a block's shared memory."""
     info = P.mtp_basis_info(20)
     raw = synth.raw_potential(20, 16, 16, 2.0, 5.0, info["n_mu"], info["m"], 18)
     pot = P.Potential(20, 16, 16, 2.0, 5.0, raw.species_energy, 0.02 * raw.radial, raw.xi_raw)
