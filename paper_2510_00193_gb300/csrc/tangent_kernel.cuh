@@ -47,8 +47,16 @@ struct TangentGeom {
   }
 };
 
+// Blocks per SM stated to ptxas (0: none).  The FP64 form of level 16, left to
+// itself, it compiles for 32 registers (53 KB of stack, 245 KB of spills a thread);
+// with two blocks stated it takes 255 (18 KB, 61 KB): 10,404 atoms 6.1 -> 3.1 ms.
+// The other forms need no such hint, and level 8 in FP32 would lose resident blocks.
+template <class LV, class S> constexpr int tangent_min_blocks() {
+  return LV::LEVEL >= 16 && sizeof(S) == 8 ? 2 : 0;
+}
+
 template <class LV, class S>
-__global__ void __launch_bounds__(kEfvThreads) tangent_kernel(const TangentArgs t) {
+__global__ void __launch_bounds__(kEfvThreads, (tangent_min_blocks<LV, S>())) tangent_kernel(const TangentArgs t) {
   using R = Dual<S>;
   constexpr int NMU = LV::NMU;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -325,6 +333,53 @@ int tangent_split_launch(const TangentArgs& t, cudaStream_t stream) {
   return MTP_OK;
 }
 
+// One kernel (levels with one component group).  Two rules, with whole calls in us:
+//   staging area: everywhere (level 8, 10,404 atoms mixed 141 -> 93) but at level 16
+//   in FP32 with more than one block per SM, where the spills want the cache that
+//   the area takes (two species: 21,296 atoms 600 -> 487, 182,250 atoms 4,051 ->
+//   3,166; three: 704 -> 632, 4,237 -> 4,160).  With one species all lanes' sums meet
+//   on the same addresses, and the line is at four blocks (21,296 atoms 433 against
+//   483, 182,250 atoms 3,245 -> 2,587); with four the area stays (69,696 atoms 1,566
+//   against 1,674);
+//   the blocks that a last, partial wave leaves, from half a block of 128 to one for
+//   every SM, go in a launch of their own: in one launch the SMs that finish first
+//   take several of them each (54,000 atoms FP64: level 8 2,385 -> 1,946, level 12
+//   4,795 -> 4,052, level 16 10,310 -> 8,675).  With 4 blocks left over, or 103 of 64
+//   threads, the launch would cost 3 to 5%.
+template <class LV, class S>
+int tangent_fused_launch(const TangentArgs& t, cudaStream_t stream) {
+  const EfvArgs& a = t.base;
+  const int64_t n = a.atom_end - a.atom_begin, sms = device_sms();
+  const int threads = sizeof(S) == 8 ? fp64_threads(n, 1) : kEfvThreads;
+  const int64_t blocks = (n + threads - 1) / threads;
+  auto kern = tangent_kernel<LV, S>;
+  const bool staged = LV::LEVEL < 16 || sizeof(S) == 8 || a.n_species >= kAccSpecies ||
+                      blocks <= (a.n_species == 1 ? 4 : 1) * sms;
+  const size_t bytes =
+      staged ? tangent_smem<S, LV::NMU>(a, threads) : efv_smem_bytes<S, LV::NMU, true>(a.n_species * a.n_species, a.n_q, a.m);
+  const int rc = set_smem(kern, bytes);
+  if (rc != MTP_OK) return rc;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, bytes) != cudaSuccess || per_sm < 1)
+    per_sm = 1;
+  int64_t rest = blocks % (per_sm * sms);
+  if (rest == blocks || rest > sms || 2 * rest * threads < sms * kEfvThreads) rest = 0;
+  TangentArgs part = t;
+  if (rest) part.base.atom_end = a.atom_begin + (blocks - rest) * threads;
+  kern<<<(unsigned)(blocks - rest), threads, bytes, stream>>>(part);
+  if (rest) {
+    part.base.atom_begin = part.base.atom_end;
+    part.base.atom_end = a.atom_end;
+    kern<<<(unsigned)rest, threads, bytes, stream>>>(part);
+  }
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("tangent kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
+    return MTP_ERR_CUDA;
+  }
+  return MTP_OK;
+}
+
 template <class LV>
 int tangent_launch(const TangentArgs& t, int precision, cudaStream_t stream) {
   const EfvArgs& a = t.base;
@@ -334,28 +389,8 @@ int tangent_launch(const TangentArgs& t, int precision, cudaStream_t stream) {
     return precision == MTP_MIXED ? tangent_split_launch<LV, float>(t, stream)
                                   : tangent_split_launch<LV, double>(t, stream);
   } else {
-    cudaError_t e;
-    if (precision == MTP_MIXED) {
-      const int threads = kEfvThreads;
-      const size_t bytes = tangent_smem<float, LV::NMU>(a, threads);
-      auto kern = tangent_kernel<LV, float>;
-      const int rc = set_smem(kern, bytes);
-      if (rc != MTP_OK) return rc;
-      kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(t);
-    } else {
-      const int threads = fp64_threads(n, 1);
-      const size_t bytes = tangent_smem<double, LV::NMU>(a, threads);
-      auto kern = tangent_kernel<LV, double>;
-      const int rc = set_smem(kern, bytes);
-      if (rc != MTP_OK) return rc;
-      kern<<<(unsigned)((n + threads - 1) / threads), threads, bytes, stream>>>(t);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      set_error("tangent kernel launch (level %d): %s", LV::LEVEL, cudaGetErrorString(e));
-      return MTP_ERR_CUDA;
-    }
-    return MTP_OK;
+    return precision == MTP_MIXED ? tangent_fused_launch<LV, float>(t, stream)
+                                  : tangent_fused_launch<LV, double>(t, stream);
   }
 }
 
